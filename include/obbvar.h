@@ -292,7 +292,8 @@ obb_status obb_tune_counting(obb_ctx* ctx, const obb_lattice* lat, const obb_qbo
  * dOmega / 3 (r_e^3 - sum s_i r_i^3 - chi_e r_e^3) (cone volumes; Eq. 10 read
  * as a volume integral).  out[k] float64 is the estimate in world units^3 for
  * box k; the mesh must be closed with outward-oriented triangles.  FP32 ray
- * tests against every triangle: a cross-check, not the exact count.
+ * tests against the triangles each texel can meet: a cross-check, not the
+ * exact count.
  * 1 <= m <= 256. */
 obb_status obb_directional_outer_volume(obb_ctx* ctx, const obb_mesh* mesh, const obb_box* boxes, int64_t K,
                                         int32_t m, double* out, int32_t on_device);
