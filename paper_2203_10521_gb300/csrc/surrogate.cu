@@ -4,8 +4,8 @@
 // only the most promising candidate moves per cluster; the exact lattice count
 // still decides every accepted move.
 //
-// Features (524 per box), from the quantised box alone, FP64 with a fixed
-// operation order (so the patch bits are reproducible):
+// Features (524 per box), from the quantised box alone, exact integers and
+// then FP32 with a fixed operation order (so the patch bits are reproducible):
 //   Lq, Hq = ceil(lo / 256), floor(hi / 256); M = n (3x3), M^-1 by cofactors;
 //   sample s in {0..7}^3: v_a = Lq_a + (Hq_a - Lq_a) (2 s_a + 1) / 16,
 //   p = M^-1 v, index = floor(p + 1/2), bit = occupancy (0 outside [0, N)^3);
@@ -15,9 +15,8 @@
 // fraction); predicted outer volume = fraction x box volume in lattice cells
 // (prod (Hq_a - Lq_a + 1) / |det M|).  Training: mean squared error on the
 // fraction, Adam, FP32 master weights; inference reads an FP16 copy of the
-// weights and accumulates in FP32.  The contraction is 100k multiply-adds per
-// box on a few thousand boxes, so it runs on CUDA cores (tiled GEMM in shared
-// memory), not tensor cores.
+// weights and accumulates in FP32 on the tensor cores; training and FP32
+// inference keep FP32 products on CUDA cores.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -242,24 +241,6 @@ __device__ __forceinline__ void tc_bulk_load(void* dst, const void* src, uint32_
 constexpr int64_t kTcW1Chunk = (int64_t)kH * kTcChunk;               // halves per W1 chunk
 constexpr int64_t kTcPacked = (kTcK1 / kTcChunk) * kTcW1Chunk + 2 * (int64_t)kH * kH;
 
-__global__ void k_pack_tc(const __half* __restrict__ wh, __half* __restrict__ wtc)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t n1 = (int64_t)kH * kTcK1;
-    if (i < n1) {
-        const int n = (int)(i % kH), k = (int)(i / kH);
-        const int q = k / kTcChunk, c = k % kTcChunk;
-        wtc[q * kTcW1Chunk + tc_off(n, c, kTcChunk) / 2] = k < kIn ? wh[oW1 + (int64_t)k * kH + n] : __float2half_rn(0.f);
-    } else if (i < n1 + 2 * (int64_t)kH * kH) {
-        const int64_t j = i - n1;
-        const int layer = (int)(j / ((int64_t)kH * kH));
-        const int e = (int)(j % ((int64_t)kH * kH));
-        const int n = e % kH, c = e / kH;
-        const int64_t base = (kTcK1 / kTcChunk) * kTcW1Chunk + layer * (int64_t)kH * kH;
-        wtc[base + tc_off(n, c, kH) / 2] = wh[(layer == 0 ? oW2 : oW3) + (int64_t)c * kH + n];
-    }
-}
-
 constexpr int kTcSmem = 65536 + (4 * kH + 4) * 4;   // A and B tiles, biases, w4, b4
 
 // y = sigmoid(W4 relu(W3 relu(W2 relu(W1 x + b1) + b2) + b3) + b4) for rows
@@ -419,116 +400,434 @@ __device__ __forceinline__ float box_cells(const obb_qbox& q)
     return det != 0.0 ? (float)(v / fabs(det)) : 0.f;
 }
 
-// ---------------------------------------------------------------- GEMM
+// ------------------------------------------------------- FP32 network
+//
+// Training and FP32 inference run on CUDA cores in FP32 (no reduced-precision
+// products).  An Adam step is three kernels:
+//   k_mlp_rows   forward and backward of R rows a block: activations stay in
+//                shared memory, the weights stream through a ring;
+//   k_mlp_wgrad  all weight and bias gradients;
+//   k_adam       the update, and every copy of the weights that a kernel
+//                reads.
+// Every sum is one chain of fused multiply-adds in ascending order (inputs of
+// a neuron, rows of a batch): training amplifies any rounding (a sign of a
+// pre-activation near zero), and a fixed order keeps a run reproducible
+// whatever the tiles are.  A layer at a time as 64 x 64 tiles the step was 18
+// launches, most of 2 to 32 blocks (0.83 ms at a batch of 1,024); the three
+// kernels take 0.043 ms (23.9 + 15.7 + 2.9 us).
 
-// C[m][n] = act(sum_k A(m, k) B(k, n) + bias[n]) (* (mask[m][n] > 0)), with
-// A(m, k) = A[m sAm + k sAk], B(k, n) = B[k sBk + n sBn]; rows m >= *d_M
-// (when given) are skipped.  act: 0 none, 1 ReLU, 2 sigmoid.  Tiles 64 x 64,
-// 256 threads, 4 x 4 outputs per thread, K in steps of 16 through shared memory.
-template <typename TB>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* __restrict__ A, int64_t sAm,
-                                              int64_t sAk, const TB* __restrict__ B, int64_t sBk, int64_t sBn,
-                                              float* __restrict__ C, int64_t ldc, const float* __restrict__ bias,
-                                              int act, const float* __restrict__ mask, int64_t ldm,
-                                              const int32_t* __restrict__ d_M)
+constexpr int kRowsThreads = kH;   // a thread per column
+constexpr int kRowsBatch = 32;     // weight rows a thread loads ahead
+constexpr int kIn4 = kIn / 4;
+static_assert(kIn % 4 == 0, "features are read four at a time");
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int n>
+__device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(n) : "memory");
+}
+
+// bytes of k_mlp_rows' dynamic shared memory: features and activations
+// [k][R], and the rows past the last that its read-ahead touches
+constexpr int rows_smem(int R, bool train)
+{
+    return (int)sizeof(float) * (kIn * R + (train ? 4 : 2) * kH * R + 32);
+}
+
+struct RowsOut {   // training only: [B][128] activations and gradients, [B] output gradients, loss per block
+    float *h1, *h2, *h3, *d1, *d2, *d3, *dy, *loss;
+};
+
+// Rows [R blockIdx.x, + R) of X through the network; y = the predicted
+// fractions.  kTrain: also the gradients of the mean squared error against
+// target down to the first layer's pre-activations.  A thread owns a column
+// and R rows, so it alone needs its column's weights: it loads them (the
+// transposed copies in wt on the way back) straight into registers, 32 rows
+// ahead and across the layers, and each serves R products; the inputs are
+// broadcast reads of shared memory, read four products' groups ahead.
+// Staging the weights in shared memory by cp.async instead costs its writes
+// and a barrier per chunk: 25.7 against 23.9 us at a batch of 1,024 (64 rows
+// ahead: 26.3 us).
+// R = 8 puts that batch on 128 SMs, a warp per scheduler, so the loop lives
+// on instruction-level parallelism; R = 16 halves the passes over the weights
+// (0.4 MB a block, from L2) once there are blocks enough.
+template <int R, bool kTrain>
+__global__ void __launch_bounds__(kRowsThreads) k_mlp_rows(const float* __restrict__ X, int M,
+                                                           const int32_t* __restrict__ d_M,
+                                                           const float* __restrict__ w, const float* __restrict__ wt,
+                                                           const float* __restrict__ target, float* __restrict__ y,
+                                                           RowsOut out)
 {
     if (d_M) M = min(M, *d_M);
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    if (m0 >= M) return;
-    __shared__ float As[16][64 + 1];
-    __shared__ float Bs[16][64 + 1];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
-        // A is read along its contiguous index (k when sAk = 1, else m) and B
-        // along n, so the loads coalesce; the padded rows of the shared tiles
-        // keep the transposed stores free of bank conflicts
-        if (sAk == 1) {
-            for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-                const int mm = i >> 4, kk = i & 15;
-                const int m = m0 + mm, k = k0 + kk;
-                As[kk][mm] = (m < M && k < K) ? A[m * sAm + k] : 0.f;
-            }
-        } else {
-            for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-                const int kk = i >> 6, mm = i & 63;
-                const int m = m0 + mm, k = k0 + kk;
-                As[kk][mm] = (m < M && k < K) ? A[m * sAm + k * sAk] : 0.f;
-            }
+    const int m0 = blockIdx.x * R;
+    if (m0 >= M) return;   // uniform
+    extern __shared__ __align__(16) float rows_smem_base[];
+    float* xs = rows_smem_base;
+    float* act = xs + kIn * R;                              // [2 or 4][kH][R]
+    __shared__ float s_dy[R], s_l[R], s_w4[kH];
+    const int tid = threadIdx.x;
+
+    // what the ends of the layers need, loaded up front
+    const float bias1 = __ldg(w + oB1 + tid), bias2 = __ldg(w + oB2 + tid), bias3 = __ldg(w + oB3 + tid),
+                w4 = __ldg(w + oW4 + tid), b4 = __ldg(w + oB4);
+    const float want = kTrain && tid < R && m0 + tid < M ? __ldg(target + m0 + tid) : 0.f;
+    float cur[kRowsBatch], nxt[kRowsBatch];   // this column's weights: the batch in use, the one after it
+    auto load = [&](float (&v)[kRowsBatch], const float* src, int rows) {
+#pragma unroll
+        for (int i = 0; i < kRowsBatch; ++i) v[i] = i < rows ? __ldg(src + i * kH) : 0.f;
+    };
+    load(cur, w + oW1 + tid, kRowsBatch);
+    s_w4[tid] = w4;
+
+    // the features, transposed to [k][R]; rows past M are zero
+    if ((reinterpret_cast<uintptr_t>(X) & 15) == 0) {
+        for (int i = tid; i < R * kIn4; i += kRowsThreads) {
+            const int r = i / kIn4, k = 4 * (i % kIn4);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (m0 + r < M) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)(m0 + r) * kIn + k));
+            xs[k * R + r] = v.x;
+            xs[(k + 1) * R + r] = v.y;
+            xs[(k + 2) * R + r] = v.z;
+            xs[(k + 3) * R + r] = v.w;
         }
-        for (int i = threadIdx.x; i < 16 * 64; i += 256) {
-            const int kk = i >> 6, nn = i & 63;
-            const int n = n0 + nn, k = k0 + kk;
-            Bs[kk][nn] = (n < N && k < K) ? (float)B[k * sBk + n * sBn] : 0.f;
+    } else {
+        for (int i = tid; i < R * kIn; i += kRowsThreads) {
+            const int r = i / kIn, k = i % kIn;
+            xs[k * R + r] = m0 + r < M ? __ldg(X + (int64_t)(m0 + r) * kIn + k) : 0.f;
         }
+    }
+
+    float acc[R];
+    // acc[r] = sum over k of in[k][r] times weight row k of this column (wp); next: the weights after these.
+    // The barrier orders what was written to `in` before, and the readers of the buffer written after.
+    auto layer = [&](const float* in, int K, const float* wp, const float* next) {
+        constexpr int G = 32 / R;   // inputs read together: 32 floats
         __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            float a[4], bb[4];
+        for (int r = 0; r < R; ++r) acc[r] = 0.f;
+        for (int k0 = 0; k0 < K; k0 += kRowsBatch) {
+            const int rows = min(kRowsBatch, K - k0), after = K - k0 - kRowsBatch;
+            if (after > 0) load(nxt, wp + (k0 + kRowsBatch) * kH, after);
+            else if (next) load(nxt, next, kRowsBatch);
+            float4 x[2][8];
+            auto read = [&](float4 (&v)[8], int k) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = As[kk][ty * 4 + i];
-                bb[i] = Bs[kk][tx * 4 + i];
+                for (int i = 0; i < 8; ++i) v[i] = *reinterpret_cast<const float4*>(in + k * R + 4 * i);
+            };
+            read(x[0], k0);
+#pragma unroll
+            for (int g = 0; g < kRowsBatch / G; ++g) {
+                if (g * G >= rows) break;   // K is a multiple of 4
+                if (g + 1 < kRowsBatch / G) read(x[(g + 1) & 1], k0 + (g + 1) * G);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 v = x[g & 1][i];
+                    const float wv = cur[g * G + 4 * i / R];
+                    const int r = 4 * i % R;
+                    acc[r] = fmaf(v.x, wv, acc[r]);
+                    acc[r + 1] = fmaf(v.y, wv, acc[r + 1]);
+                    acc[r + 2] = fmaf(v.z, wv, acc[r + 2]);
+                    acc[r + 3] = fmaf(v.w, wv, acc[r + 3]);
+                }
             }
+#pragma unroll
+            for (int i = 0; i < kRowsBatch; ++i) cur[i] = nxt[i];
+        }
+    };
+    // acc to an activation buffer [column][R] and, in training, to [B][128]
+    auto store = [&](float* a, float* h) {
+        if (a)
+#pragma unroll
+            for (int r = 0; r < R; r += 4)
+                *reinterpret_cast<float4*>(a + tid * R + r) = make_float4(acc[r], acc[r + 1], acc[r + 2], acc[r + 3]);
+        if (kTrain)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (m0 + r < M) h[(int64_t)(m0 + r) * kH + tid] = acc[r];
+    };
+    float* a1 = act;
+    float* a2 = act + kH * R;
+    float* a3 = kTrain ? act + 2 * kH * R : a1;
+    float* da = act + 3 * kH * R;
+    // a gradient passes where its activation is positive
+    auto masked = [&](const float* a) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (!(a[tid * R + r] > 0.f)) acc[r] = 0.f;
+    };
+    // one copy of the loop's code for the three layers and the two steps back (five copies do not fit the
+    // instruction caches)
+#pragma unroll 1
+    for (int l = 0; l < (kTrain ? 5 : 3); ++l) {
+        const float *w2 = w + oW2 + tid, *w3 = w + oW3 + tid, *w3t = wt + kH * kH + tid, *w2t = wt + tid;
+        layer(l == 0 ? xs : l == 1 ? a1 : l == 2 ? a2 : l == 3 ? da : a3, l == 0 ? kIn : kH,
+              l == 0 ? w + oW1 + tid : l == 1 ? w2 : l == 2 ? w3 : l == 3 ? w3t : w2t,
+              l == 0 ? w2 : l == 1 ? w3 : l == 2 ? (kTrain ? w3t : nullptr) : l == 3 ? w2t : nullptr);
+        if (l < 3) {
+            const float bias = l == 0 ? bias1 : l == 1 ? bias2 : bias3;
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fmaxf(acc[r] + bias, 0.f);
+            store(l == 0 ? a1 : l == 1 ? a2 : a3, l == 0 ? out.h1 : l == 1 ? out.h2 : out.h3);
+        } else if (l == 3) {
+            masked(a2);
+            store(a3, out.d2);
+        } else {
+            masked(a1);
+            store(nullptr, out.d1);
+        }
+        if (l != 2) continue;
+        __syncthreads();
+        // the output neuron: a thread per row
+        if (tid < R) {
+            float v = 0.f;
+#pragma unroll 16
+            for (int k = 0; k < kH; ++k) v = fmaf(a3[k * R + tid], s_w4[k], v);
+            const int m = m0 + tid;
+            const float f = 1.f / (1.f + __expf(-(v + b4)));
+            if (m < M) y[m] = f;
+            if (kTrain) {
+                const float e = m < M ? f - want : 0.f;
+                s_dy[tid] = 2.f * e / (float)M * f * (1.f - f);
+                s_l[tid] = e * e / (float)M;
+                if (m < M) out.dy[m] = s_dy[tid];
+            }
+        }
+        if (!kTrain) return;
+        __syncthreads();
+        if (tid == 0) {
+            float l = 0.f;
+            for (int r = 0; r < R; ++r) l += s_l[r];
+            out.loss[blockIdx.x] = l;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = s_dy[r] * w4;
+        masked(a3);
+        store(da, out.d3);
+    }
+}
+
+// Weight and bias gradients, one block a piece of them:
+//   block 0               the output neuron's bias (sum of dy);
+//   blocks 1-8            its weights, 16 inputs each;
+//   blocks 9-20           the other biases, 32 columns each: sums of 256
+//                         strided chains as a tree of shuffles would add them;
+//   the rest              16 x 16 tiles of A^T D (A = a layer's inputs, D =
+//                         the gradients of its pre-activations).
+// A weight's chain runs over the whole batch, so the parallelism is across
+// weights: 392 tiles of two warps, a thread holding 2 x 2 sums (16 x 32 tiles
+// of two warps: 19.6, of four: 17.1 against 15.7 us: fewer blocks than two
+// an SM leave some with one, and 2 x 4 sums leave a warp's issue the limit).
+// Both operands are read along their rows, so nothing is
+// transposed; 64-row stages arrive by cp.async three ahead.
+constexpr int kGradThreads = 64;
+constexpr int kGradM = 16, kGradN = 16;
+constexpr int kGradRows = 64;      // batch rows per stage
+constexpr int kGradStages = 4;
+constexpr int kGradNt = kH / kGradN;
+constexpr int kGradTiles1 = (kIn + kGradM - 1) / kGradM * kGradNt, kGradTilesH = kH / kGradM * kGradNt;
+constexpr int kGradBlocks = 21 + kGradTiles1 + 2 * kGradTilesH;
+constexpr int kGradStage = kGradRows * (kGradM + kGradN);          // floats
+constexpr int kGradSmem = (int)sizeof(float) * kGradStages * kGradStage;
+static_assert(kGradRows * 17 <= kGradStage, "16 inputs and dy fit a stage");
+
+__global__ void __launch_bounds__(kGradThreads) k_mlp_wgrad(const float* __restrict__ X, int M, const RowsOut in,
+                                                            float* __restrict__ grad)
+{
+    extern __shared__ __align__(16) float grad_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int steps = (M + kGradRows - 1) / kGradRows;
+    if (blockIdx.x == 0) {
+        for (int q = warp; q < 8; q += 2) {
+            float s = 0.f;
+            for (int m = 32 * q + lane; m < M; m += 256) s += __ldg(in.dy + m);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) grad_smem[q] = s;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            float t = 0.f;
+            for (int q = 0; q < 8; ++q) t += grad_smem[q];
+            grad[oB4] = t;
+        }
+        return;
+    }
+    if (blockIdx.x < 9) {
+        const int i0 = 16 * (blockIdx.x - 1);
+        auto issue = [&](int st) {
+            if (st < steps) {
+                float* a = grad_smem + (st % kGradStages) * kGradStage;
+                const int b = st * kGradRows, rows = min(kGradRows, M - b);
+                for (int i = tid; i < rows * 4; i += kGradThreads)
+                    cp_async16(a + 4 * i, in.h3 + (int64_t)(b + i / 4) * kH + i0 + 4 * (i % 4));
+                if (tid < rows) cp_async4(a + kGradRows * 16 + tid, in.dy + b + tid);
+            }
+            cp_commit();
+        };
+        for (int st = 0; st < kGradStages - 1; ++st) issue(st);
+        float s = 0.f;
+        for (int st = 0; st < steps; ++st) {
+            cp_wait<kGradStages - 2>();
+            __syncthreads();
+            issue(st + kGradStages - 1);
+            const float* a = grad_smem + (st % kGradStages) * kGradStage;
+            const int rows = min(kGradRows, M - st * kGradRows);
+            if (tid < 16)
+#pragma unroll 16
+                for (int r = 0; r < rows; ++r) s = fmaf(a[r * 16 + tid], a[kGradRows * 16 + r], s);
+        }
+        if (tid < 16) grad[oW4 + i0 + tid] = s;
+        return;
+    }
+    if (blockIdx.x < 21) {
+        const int l = (blockIdx.x - 9) / 4, n = 32 * ((blockIdx.x - 9) % 4) + lane;
+        const float* D = l == 0 ? in.d1 : l == 1 ? in.d2 : in.d3;
+        for (int q = warp; q < 8; q += 2) {
+            float s[32];
+#pragma unroll
+            for (int v = 0; v < 32; ++v) s[v] = 0.f;
+            for (int m = 32 * q; m < M; m += 256) {
+                float x[32];
+#pragma unroll
+                for (int v = 0; v < 32; ++v) x[v] = m + v < M ? __ldg(D + (int64_t)(m + v) * kH + n) : 0.f;
+#pragma unroll
+                for (int v = 0; v < 32; ++v) s[v] += x[v];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int v = 0; v < o; ++v) s[v] += s[v + o];
+            grad_smem[32 * q + lane] = s[0];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            float t = 0.f;
+            for (int q = 0; q < 8; ++q) t += grad_smem[32 * q + lane];
+            grad[(l == 0 ? oB1 : l == 1 ? oB2 : oB3) + n] = t;
+        }
+        return;
+    }
+    int tile = blockIdx.x - 21, ld = kH;
+    const float *A, *D;
+    int64_t oW;
+    if (tile < kGradTiles1) {
+        A = X, D = in.d1, ld = kIn, oW = oW1;
+    } else if ((tile -= kGradTiles1) < kGradTilesH) {
+        A = in.h1, D = in.d2, oW = oW2;
+    } else {
+        tile -= kGradTilesH;
+        A = in.h2, D = in.d3, oW = oW3;
+    }
+    const int m0 = tile / kGradNt * kGradM, n0 = tile % kGradNt * kGradN, width = min(kGradM, ld - m0);
+    const bool wide = (reinterpret_cast<uintptr_t>(A) & 15) == 0;   // ld and m0 are multiples of 4
+    // this thread's share of a stage: 4 of the 64 x 4 pieces of A and of D
+    const int ar = tid >> 2, aq = 4 * (tid & 3);
+    const float* asrc = A + (int64_t)ar * ld + m0 + aq;
+    const float* dsrc = D + (int64_t)ar * kH + n0 + aq;
+    auto issue = [&](int st) {
+        if (st < steps) {
+            float* a = grad_smem + (st % kGradStages) * kGradStage + ar * kGradM + aq;
+            float* d = a + kGradRows * kGradM;
+            const int b = st * kGradRows, rows = min(kGradRows, M - b);
+            const float* as = asrc + (int64_t)b * ld;
+            const float* ds = dsrc + (int64_t)b * kH;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+                if (ar + 16 * i < rows) {
+                    if (aq < width) {
+                        if (wide) cp_async16(a + 16 * i * kGradM, as + 16 * i * ld);
+                        else
+                            for (int e = 0; e < 4; ++e) cp_async4(a + 16 * i * kGradM + e, as + 16 * i * ld + e);
+                    }
+                    cp_async16(d + 16 * i * kGradN, ds + 16 * i * kH);
+                }
         }
+        cp_commit();
+    };
+    for (int st = 0; st < kGradStages - 1; ++st) issue(st);
+    // a warp covers 8 rows x 16 columns
+    const int mr = 8 * warp + 2 * (lane >> 3), nc = 2 * (lane & 7);
+    float acc[2][2] = {};
+    for (int st = 0; st < steps; ++st) {
+        cp_wait<kGradStages - 2>();
         __syncthreads();
-    }
+        issue(st + kGradStages - 1);
+        const float* a = grad_smem + (st % kGradStages) * kGradStage + mr;
+        const float* d = grad_smem + (st % kGradStages) * kGradStage + kGradRows * kGradM + nc;
+        auto rows8 = [&](int r0, int n) {   // n <= 8 rows, all reads before the products
+            float2 av[8], dv[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty * 4 + i;
-        if (m >= M) continue;
+            for (int r = 0; r < 8; ++r)
+                if (r < n) {
+                    av[r] = *reinterpret_cast<const float2*>(a + (r0 + r) * kGradM);
+                    dv[r] = *reinterpret_cast<const float2*>(d + (r0 + r) * kGradN);
+                }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tx * 4 + j;
-            if (n >= N) continue;
-            float v = acc[i][j] + (bias ? bias[n] : 0.f);
-            if (mask && !(mask[m * ldm + n] > 0.f)) v = 0.f;
-            if (act == 1) v = fmaxf(v, 0.f);
-            else if (act == 2) v = 1.f / (1.f + __expf(-v));
-            C[m * ldc + n] = v;
+            for (int r = 0; r < 8; ++r)
+                if (r < n) {
+                    acc[0][0] = fmaf(av[r].x, dv[r].x, acc[0][0]);
+                    acc[0][1] = fmaf(av[r].x, dv[r].y, acc[0][1]);
+                    acc[1][0] = fmaf(av[r].y, dv[r].x, acc[1][0]);
+                    acc[1][1] = fmaf(av[r].y, dv[r].y, acc[1][1]);
+                }
+        };
+        const int rows = min(kGradRows, M - st * kGradRows);
+        if (rows == kGradRows) {
+#pragma unroll
+            for (int r = 0; r < kGradRows; r += 8) rows8(r, 8);
+        } else {
+            for (int r = 0; r < rows; r += 8) rows8(r, rows - r);
         }
     }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)   // rows past `width` hold nothing that is used
+        if (mr + i < width)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) grad[oW + (int64_t)(m0 + mr + i) * kH + n0 + nc + j] = acc[i][j];
 }
 
-// column sums: out[n] = sum_m X[m][n] (bias gradients)
-__global__ void k_colsum(const float* __restrict__ X, int M, int N, float* __restrict__ out)
+// the loss: the blocks' sums, by the first warp in a fixed order
+__device__ __forceinline__ void sum_loss(const float* __restrict__ parts, int n, float* __restrict__ loss)
 {
-    const int n = blockIdx.x;
-    float s = 0.f;
-    for (int m = threadIdx.x; m < M; m += blockDim.x) s += X[(int64_t)m * N + n];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ float sh[32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += sh[i];
-        out[n] = t;
-    }
-}
-
-// dY = 2 (y - t) / B * y (1 - y); loss partial sums
-__global__ void k_out_grad(const float* __restrict__ y, const float* __restrict__ t, int B, float* __restrict__ dy,
-                           float* __restrict__ loss)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
     float l = 0.f;
-    if (i < B) {
-        const float e = y[i] - t[i];
-        dy[i] = 2.f * e / (float)B * y[i] * (1.f - y[i]);
-        l = e * e / (float)B;
-    }
+    for (int i = threadIdx.x; i < n; i += 32) l += parts[i];
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.f) atomicAdd(loss, l);
+    if (threadIdx.x == 0) *loss = l;
+}
+
+__global__ void k_loss(const float* __restrict__ parts, int n, float* __restrict__ loss) { sum_loss(parts, n, loss); }
+
+// the copies of weight i: FP16, its place in the tensor-core kernel's tiles,
+// and W2, W3 transposed
+__device__ __forceinline__ void store_weight_copies(int64_t i, float wi, __half* __restrict__ wh,
+                                                    __half* __restrict__ wtc, float* __restrict__ wt)
+{
+    const __half h = __float2half_rn(wi);
+    wh[i] = h;
+    if (i < oB1) {
+        const int n = (int)(i % kH), k = (int)(i / kH);
+        wtc[(k / kTcChunk) * kTcW1Chunk + tc_off(n, k % kTcChunk, kTcChunk) / 2] = h;
+    } else if ((i >= oW2 && i < oB2) || (i >= oW3 && i < oB3)) {
+        const int layer = i >= oW3, j = (int)(i - (layer ? oW3 : oW2)), n = j % kH, k = j / kH;
+        wtc[(kTcK1 / kTcChunk) * kTcW1Chunk + layer * kH * kH + tc_off(n, k, kH) / 2] = h;
+        wt[layer * kH * kH + n * kH + k] = wi;
+    }
 }
 
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
-                       __half* __restrict__ wh, int64_t n, float lr, float b1t, float b2t)
+                       __half* __restrict__ wh, __half* __restrict__ wtc, float* __restrict__ wt, int64_t n, float lr,
+                       float b1t, float b2t, const float* __restrict__ lparts, int n_l, float* __restrict__ loss)
 {
+    sum_loss(lparts, n_l, loss);
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -540,13 +839,20 @@ __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float
     const float mh = mi / (1.f - b1t), vh = vi / (1.f - b2t);
     const float wi = w[i] - lr * mh / (sqrtf(vh) + eps);
     w[i] = wi;
-    wh[i] = __float2half_rn(wi);
+    store_weight_copies(i, wi, wh, wtc, wt);
 }
 
-__global__ void k_to_half(const float* __restrict__ w, __half* __restrict__ wh, int64_t n)
+// every copy of the weights; zero: also the padding of the tensor-core tiles
+// (features 524 to 575, which no weight fills)
+__global__ void k_pack(const float* __restrict__ w, __half* __restrict__ wh, __half* __restrict__ wtc,
+                       float* __restrict__ wt, int zero)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) wh[i] = __float2half_rn(w[i]);
+    if (i < kParams) store_weight_copies(i, w[i], wh, wtc, wt);
+    if (zero && i < (int64_t)(kTcK1 - kIn) * kH) {
+        const int n = (int)(i % kH), k = kIn + (int)(i / kH);
+        wtc[(k / kTcChunk) * kTcW1Chunk + tc_off(n, k % kTcChunk, kTcChunk) / 2] = __float2half_rn(0.f);
+    }
 }
 
 // predicted outer volume = fraction x cells
@@ -569,29 +875,20 @@ __global__ void k_targets(const uint64_t* __restrict__ counts, const obb_qbox* _
     out[i] = fminf(fmaxf(t, 0.f), 1.f);
 }
 
-template <typename TB>
-void gemm(obb_ctx* ctx, int M, int N, int K, const float* A, int64_t sAm, int64_t sAk, const TB* B, int64_t sBk,
-          int64_t sBn, float* C, int64_t ldc, const float* bias, int act, const float* mask, int64_t ldm,
-          const int32_t* d_M)
-{
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
-    k_gemm<TB><<<grid, 256, 0, ctx->stream>>>(M, N, K, A, sAm, sAk, B, sBk, sBn, C, ldc, bias, act, mask, ldm, d_M);
-    note_launch(ctx);
-}
-
 }  // namespace
 
 struct MlpImpl {
     float* w = nullptr;    // FP32 master weights
     __half* wh = nullptr;  // FP16 inference copy
     __half* wtc = nullptr; // the FP16 weights transposed into the tensor-core kernel's shared tiles
+    float* wt = nullptr;   // W2 and W3 transposed (the backward pass)
     float* g = nullptr;    // gradients
     float* m = nullptr;    // Adam moments
     float* v = nullptr;
     int64_t step = 0;
     int64_t cap = 0;       // batch capacity of the activation buffers
     float *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *y = nullptr, *d1 = nullptr, *d2 = nullptr, *d3 = nullptr,
-          *dy = nullptr, *loss = nullptr;
+          *dy = nullptr, *loss = nullptr, *lparts = nullptr;
 };
 
 }  // namespace obbv
@@ -618,14 +915,32 @@ static obb_status mlp_reserve(obb_ctx* ctx, MlpImpl* P, int64_t B)
     }
     if (P->y) cudaFreeAsync(P->y, s);
     if (P->dy) cudaFreeAsync(P->dy, s);
+    if (P->lparts) cudaFreeAsync(P->lparts, s);
     OBB_CK(ctx, pool_alloc((void**)&P->y, sizeof(float) * B, s));
     OBB_CK(ctx, pool_alloc((void**)&P->dy, sizeof(float) * B, s));
+    OBB_CK(ctx, pool_alloc((void**)&P->lparts, sizeof(float) * ((B + 7) / 8), s));
     P->cap = B;
     return OBB_OK;
 }
 
-// forward pass into P->h1..h3, P->y (fraction); FP32 or FP16 weights
-static void mlp_forward(obb_ctx* ctx, const MlpImpl* P, const float* X, int B, const int32_t* d_B, bool half)
+// rows a block of k_mlp_rows carries: 8 up to two blocks' worth an SM, else 16
+static int rows_per_block(const obb_ctx* ctx, int B) { return B <= 16 * ctx->num_sms ? 8 : 16; }
+
+template <int R, bool kTrain>
+static cudaError_t launch_rows(obb_ctx* ctx, const MlpImpl* P, const float* X, int B, const int32_t* d_B,
+                               const float* T, const RowsOut& out)
+{
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_rows<R, kTrain>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               rows_smem(R, kTrain));
+    if (e != cudaSuccess) return e;
+    k_mlp_rows<R, kTrain><<<(unsigned)((B + R - 1) / R), kRowsThreads, rows_smem(R, kTrain), ctx->stream>>>(
+        X, B, d_B, P->w, P->wt, T, P->y, out);
+    note_launch(ctx);
+    return cudaGetLastError();
+}
+
+// forward pass into P->y (fraction); FP32 or FP16 weights
+static obb_status mlp_forward(obb_ctx* ctx, const MlpImpl* P, const float* X, int B, const int32_t* d_B, bool half)
 {
     if (half) {
         // all four layers in one tensor-core kernel (FP16 operands, FP32 accumulators)
@@ -635,46 +950,34 @@ static void mlp_forward(obb_ctx* ctx, const MlpImpl* P, const float* X, int B, c
         k_mlp_tc<<<(unsigned)((B + kTcRows - 1) / kTcRows), kTcRows, kTcSmem, ctx->stream>>>(X, B, d_B, P->wtc, P->wh,
                                                                                            P->w, P->y, ctx->d_err, stall);
         note_launch(ctx);
+        OBB_CK(ctx, cudaGetLastError());
+    } else if (rows_per_block(ctx, B) == 8) {
+        OBB_CK(ctx, (launch_rows<8, false>(ctx, P, X, B, d_B, nullptr, RowsOut{})));
     } else {
-        const float* w = P->w;
-        gemm<float>(ctx, B, kH, kIn, X, kIn, 1, w + oW1, kH, 1, P->h1, kH, w + oB1, 1, nullptr, 0, d_B);
-        gemm<float>(ctx, B, kH, kH, P->h1, kH, 1, w + oW2, kH, 1, P->h2, kH, w + oB2, 1, nullptr, 0, d_B);
-        gemm<float>(ctx, B, kH, kH, P->h2, kH, 1, w + oW3, kH, 1, P->h3, kH, w + oB3, 1, nullptr, 0, d_B);
-        gemm<float>(ctx, B, 1, kH, P->h3, kH, 1, w + oW4, 1, 1, P->y, 1, w + oB4, 2, nullptr, 0, d_B);
+        OBB_CK(ctx, (launch_rows<16, false>(ctx, P, X, B, d_B, nullptr, RowsOut{})));
     }
+    return OBB_OK;
 }
 
-// loss and gradients (FP32 weights) into P->g; loss into P->loss (device)
-static obb_status mlp_backward(obb_ctx* ctx, MlpImpl* P, const float* X, const float* T, int B)
+// gradients of the batch (FP32 weights) into P->g, the loss as *nl parts in P->lparts
+static obb_status mlp_backward(obb_ctx* ctx, MlpImpl* P, const float* X, const float* T, int B, int* nl)
 {
-    cudaStream_t s = ctx->stream;
-    mlp_forward(ctx, P, X, B, nullptr, false);
-    OBB_CK(ctx, cudaMemsetAsync(P->loss, 0, sizeof(float), s));
-    k_out_grad<<<(B + 255) / 256, 256, 0, s>>>(P->y, T, B, P->dy, P->loss);
-    note_launch(ctx);
-    float* g = P->g;
-    const float* w = P->w;
-    // layer 4: dW4 = H3^T dY, db4 = sum dY, dH3 = dY W4^T * (H3 > 0)
-    gemm<float>(ctx, kH, 1, B, P->h3, 1, kH, P->dy, 1, 1, g + oW4, 1, nullptr, 0, nullptr, 0, nullptr);
-    k_colsum<<<1, 256, 0, s>>>(P->dy, B, 1, g + oB4);
-    note_launch(ctx);
-    gemm<float>(ctx, B, kH, 1, P->dy, 1, 1, w + oW4, 1, 1, P->d3, kH, nullptr, 0, P->h3, kH, nullptr);
-    // layer 3
-    gemm<float>(ctx, kH, kH, B, P->h2, 1, kH, P->d3, kH, 1, g + oW3, kH, nullptr, 0, nullptr, 0, nullptr);
-    k_colsum<<<kH, 256, 0, s>>>(P->d3, B, kH, g + oB3);
-    note_launch(ctx);
-    gemm<float>(ctx, B, kH, kH, P->d3, kH, 1, w + oW3, 1, kH, P->d2, kH, nullptr, 0, P->h2, kH, nullptr);
-    // layer 2
-    gemm<float>(ctx, kH, kH, B, P->h1, 1, kH, P->d2, kH, 1, g + oW2, kH, nullptr, 0, nullptr, 0, nullptr);
-    k_colsum<<<kH, 256, 0, s>>>(P->d2, B, kH, g + oB2);
-    note_launch(ctx);
-    gemm<float>(ctx, B, kH, kH, P->d2, kH, 1, w + oW2, 1, kH, P->d1, kH, nullptr, 0, P->h1, kH, nullptr);
-    // layer 1
-    gemm<float>(ctx, kIn, kH, B, X, 1, kIn, P->d1, kH, 1, g + oW1, kH, nullptr, 0, nullptr, 0, nullptr);
-    k_colsum<<<kH, 256, 0, s>>>(P->d1, B, kH, g + oB1);
+    const RowsOut out{P->h1, P->h2, P->h3, P->d1, P->d2, P->d3, P->dy, P->lparts};
+    const int R = rows_per_block(ctx, B);
+    if (R == 8) OBB_CK(ctx, (launch_rows<8, true>(ctx, P, X, B, nullptr, T, out)));
+    else OBB_CK(ctx, (launch_rows<16, true>(ctx, P, X, B, nullptr, T, out)));
+    *nl = (B + R - 1) / R;
+    OBB_CK(ctx, cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem));
+    k_mlp_wgrad<<<kGradBlocks, kGradThreads, kGradSmem, ctx->stream>>>(X, B, out, P->g);
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
     return OBB_OK;
+}
+
+static void pack_weights(obb_ctx* ctx, MlpImpl* P, bool zero)
+{
+    k_pack<<<(unsigned)((kParams + 255) / 256), 256, 0, ctx->stream>>>(P->w, P->wh, P->wtc, P->wt, zero ? 1 : 0);
+    note_launch(ctx);
 }
 
 obb_status surrogate_predict(obb_ctx* ctx, const obb_mlp* mlp, const obb_lattice* lat, const obb_qbox* d_boxes,
@@ -685,7 +988,7 @@ obb_status surrogate_predict(obb_ctx* ctx, const obb_mlp* mlp, const obb_lattice
     k_features<<<(unsigned)cap, 128, 0, ctx->stream>>>(d_boxes, d_K, lat->d_words, lat->frame.N, lat->frame.W,
                                                        d_feats);
     note_launch(ctx);
-    mlp_forward(ctx, P, d_feats, (int)cap, d_K, true);
+    OBB_TRY(mlp_forward(ctx, P, d_feats, (int)cap, d_K, true));
     k_pred_obv<<<(unsigned)((cap + 255) / 256), 256, 0, ctx->stream>>>(P->y, d_boxes, d_K, d_pred);
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
@@ -736,6 +1039,7 @@ obb_status obb_mlp_create(obb_ctx* ctx, uint64_t seed, obb_mlp** out)
     cudaError_t e = pool_alloc((void**)&P->w, sizeof(float) * kParams, s);
     if (e == cudaSuccess) e = pool_alloc((void**)&P->wh, sizeof(__half) * kParams, s);
     if (e == cudaSuccess) e = pool_alloc((void**)&P->wtc, sizeof(__half) * kTcPacked, s);
+    if (e == cudaSuccess) e = pool_alloc((void**)&P->wt, sizeof(float) * 2 * kH * kH, s);
     if (e == cudaSuccess) e = pool_alloc((void**)&P->g, sizeof(float) * kParams, s);
     if (e == cudaSuccess) e = pool_alloc((void**)&P->m, sizeof(float) * kParams, s);
     if (e == cudaSuccess) e = pool_alloc((void**)&P->v, sizeof(float) * kParams, s);
@@ -744,9 +1048,7 @@ obb_status obb_mlp_create(obb_ctx* ctx, uint64_t seed, obb_mlp** out)
     if (e == cudaSuccess) e = cudaMemsetAsync(P->m, 0, sizeof(float) * kParams, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(P->v, 0, sizeof(float) * kParams, s);
     if (e == cudaSuccess) {
-        k_to_half<<<(unsigned)((kParams + 255) / 256), 256, 0, s>>>(P->w, P->wh, kParams);
-        k_pack_tc<<<(unsigned)((kTcPacked + 255) / 256), 256, 0, s>>>(P->wh, P->wtc);
-        note_launch(ctx, 2);
+        pack_weights(ctx, P, true);
         e = cudaStreamSynchronize(s);
     }
     if (e != cudaSuccess) {
@@ -763,7 +1065,7 @@ void obb_mlp_free(obb_mlp* m)
     cudaStream_t s = m->ctx ? m->ctx->stream : nullptr;
     if (m->p) {
         MlpImpl* P = m->p;
-        void* ptrs[] = {P->w, P->wh, P->wtc, P->g, P->m, P->v, P->h1, P->h2, P->h3, P->y, P->d1, P->d2, P->d3, P->dy, P->loss};
+        void* ptrs[] = {P->w, P->wh, P->wtc, P->g, P->m, P->v, P->h1, P->h2, P->h3, P->y, P->d1, P->d2, P->d3, P->dy, P->loss, P->wt, P->lparts};
         for (void* q : ptrs)
             if (q) cudaFreeAsync(q, s);
         delete P;
@@ -789,10 +1091,7 @@ obb_status obb_mlp_set_params(obb_ctx* ctx, obb_mlp* m, const float* in, int32_t
     MlpImpl* P = m->p;
     OBB_CK(ctx, cudaMemcpyAsync(P->w, in, sizeof(float) * kParams,
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->stream));
-    k_to_half<<<(unsigned)((kParams + 255) / 256), 256, 0, ctx->stream>>>(P->w, P->wh, kParams);
-    k_pack_tc<<<(unsigned)((kTcPacked + 255) / 256), 256, 0, ctx->stream>>>(P->wh, P->wtc);
-    note_launch(ctx);
-    note_launch(ctx);
+    pack_weights(ctx, P, false);
     OBB_CK(ctx, cudaMemsetAsync(P->m, 0, sizeof(float) * kParams, ctx->stream));
     OBB_CK(ctx, cudaMemsetAsync(P->v, 0, sizeof(float) * kParams, ctx->stream));
     P->step = 0;
@@ -859,8 +1158,7 @@ obb_status obb_mlp_forward(obb_ctx* ctx, const obb_mlp* m, const float* feats, i
     const float* dx;
     OBB_TRY(dev_in(ctx, feats, (size_t)B * kIn, on_device, &hx, &dx));
     OBB_TRY(mlp_reserve(ctx, m->p, B));
-    mlp_forward(ctx, m->p, dx, (int)B, nullptr, half_weights != 0);
-    OBB_CK(ctx, cudaGetLastError());
+    OBB_TRY(mlp_forward(ctx, m->p, dx, (int)B, nullptr, half_weights != 0));
     OBB_CK(ctx, cudaMemcpyAsync(out, m->p->y, sizeof(float) * B,
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, ctx->stream));
     if (hx) cudaFreeAsync(hx, ctx->stream);
@@ -878,7 +1176,12 @@ obb_status obb_mlp_gradients(obb_ctx* ctx, obb_mlp* m, const float* feats, const
     OBB_TRY(dev_in(ctx, feats, (size_t)B * kIn, on_device, &hx, &dx));
     OBB_TRY(dev_in(ctx, target, (size_t)B, on_device, &ht, &dt));
     OBB_TRY(mlp_reserve(ctx, m->p, B));
-    OBB_TRY(mlp_backward(ctx, m->p, dx, dt, (int)B));
+    MlpImpl* P = m->p;
+    int nl;
+    OBB_TRY(mlp_backward(ctx, P, dx, dt, (int)B, &nl));
+    k_loss<<<1, 32, 0, ctx->stream>>>(P->lparts, nl, P->loss);
+    note_launch(ctx);
+    OBB_CK(ctx, cudaGetLastError());
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (grads) OBB_CK(ctx, cudaMemcpyAsync(grads, m->p->g, sizeof(float) * kParams, kind, ctx->stream));
     if (loss) OBB_CK(ctx, cudaMemcpyAsync(loss, m->p->loss, sizeof(float), kind, ctx->stream));
@@ -900,13 +1203,13 @@ obb_status obb_mlp_train_step(obb_ctx* ctx, obb_mlp* m, const float* feats, cons
     OBB_TRY(dev_in(ctx, target, (size_t)B, on_device, &ht, &dt));
     MlpImpl* P = m->p;
     OBB_TRY(mlp_reserve(ctx, P, B));
-    OBB_TRY(mlp_backward(ctx, P, dx, dt, (int)B));
+    int nl;
+    OBB_TRY(mlp_backward(ctx, P, dx, dt, (int)B, &nl));
     P->step += 1;
     const float b1t = std::pow(0.9f, (float)P->step), b2t = std::pow(0.999f, (float)P->step);
-    k_adam<<<(unsigned)((kParams + 255) / 256), 256, 0, ctx->stream>>>(P->w, P->g, P->m, P->v, P->wh, kParams, lr,
-                                                                      b1t, b2t);
-    k_pack_tc<<<(unsigned)((kTcPacked + 255) / 256), 256, 0, ctx->stream>>>(P->wh, P->wtc);
-    note_launch(ctx, 2);
+    k_adam<<<(unsigned)((kParams + 255) / 256), 256, 0, ctx->stream>>>(P->w, P->g, P->m, P->v, P->wh, P->wtc, P->wt,
+                                                                      kParams, lr, b1t, b2t, P->lparts, nl, P->loss);
+    note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
     if (loss)
         OBB_CK(ctx, cudaMemcpyAsync(loss, P->loss, sizeof(float),
