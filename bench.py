@@ -134,7 +134,7 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-COUNTING_SOURCES = ("outer_volume.cu", "occupancy.cu", "internal.h")
+COUNTING_SOURCES = ("outer_volume.cu", "counting.cuh", "occupancy.cu", "internal.h")
 
 
 def counting_source_hash():

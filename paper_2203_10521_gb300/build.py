@@ -30,7 +30,7 @@ def nvcc() -> str:
 
 def _deps():
     files = [os.path.join(SRC, u) for u in UNITS]
-    files += [os.path.join(SRC, "internal.h"), os.path.join(HERE, "..", "include", "obbvar.h")]
+    files += [os.path.join(SRC, "internal.h"), os.path.join(SRC, "counting.cuh"), os.path.join(HERE, "..", "include", "obbvar.h")]
     return files
 
 

@@ -343,9 +343,14 @@ obb_status rebuild_occupancy(obb_ctx* ctx, obb_lattice* lat);
 obb_status quantize_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box* d_boxes, int64_t K,
                           obb_qbox* d_out);
 // counts / points (points may be null) for K boxes whose count is held on the device at
-// d_K (int32); K_cap bounds it for scratch sizing.  counts/points are zeroed here.
+// d_K (int32; null: K_cap boxes); K_cap bounds it for scratch sizing.  counts/points are zeroed here.
 obb_status count_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* d_boxes,
                        const int32_t* d_K, int64_t K_cap, uint64_t* d_counts, uint64_t* d_points);
+// the same for a count that the host knows: quantised boxes, and float boxes (quantised on the way)
+obb_status count_known(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* d_boxes, int64_t K, uint64_t* d_counts,
+                       uint64_t* d_points);
+obb_status count_float_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box* d_boxes, int64_t K,
+                             uint64_t* d_counts, uint64_t* d_points);
 // the same over boxes of several lattices: box k uses d_lats[d_lat_of_box[k]];
 // lattice_bytes (the lattices' occupancy words together) decides the spatial order
 obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats, const int32_t* d_lat_of_box,

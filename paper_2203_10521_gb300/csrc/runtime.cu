@@ -425,22 +425,15 @@ static obb_status outer_volume_impl(obb_ctx* ctx, const obb_lattice* lat, const 
     if (K < 0 || K > (int64_t(1) << 30)) return fail(ctx, OBB_ERR_ARG, "K out of range");
     if (K == 0) return OBB_OK;
     HostTmp hb(ctx), hc(ctx), hp(ctx);
+    const obb_box* db = nullptr;
     const obb_qbox* dq = nullptr;
-    if (boxes) {
-        const obb_box* db;
-        OBB_TRY(to_device(ctx, boxes, (size_t)K, on_device, hb, &db));
-        OBB_CK(ctx, ctx->qscratch.reserve(sizeof(obb_qbox) * K, ctx->stream));
-        OBB_TRY(quantize_boxes(ctx, lat, db, K, ctx->qscratch.as<obb_qbox>()));
-        dq = ctx->qscratch.as<obb_qbox>();
-    } else {
-        OBB_TRY(to_device(ctx, qboxes, (size_t)K, on_device, hb, &dq));
-    }
+    if (boxes) OBB_TRY(to_device(ctx, boxes, (size_t)K, on_device, hb, &db));
+    else OBB_TRY(to_device(ctx, qboxes, (size_t)K, on_device, hb, &dq));
     uint64_t *dc, *dp;
     OBB_TRY(out_device(ctx, counts, (size_t)K, on_device, hc, &dc));
     OBB_TRY(out_device(ctx, points, (size_t)K, on_device, hp, &dp));
-    OBB_CK(ctx, ctx->kdev.reserve(sizeof(int32_t), ctx->stream));
-    OBB_TRY(set_device_int(ctx, ctx->kdev.as<int32_t>(), (int32_t)K));
-    OBB_TRY(count_boxes(ctx, lat, dq, ctx->kdev.as<int32_t>(), K, dc, dp));
+    if (db) OBB_TRY(count_float_boxes(ctx, lat, db, K, dc, dp));
+    else OBB_TRY(count_known(ctx, lat, dq, K, dc, dp));
     OBB_TRY(copy_back(ctx, counts, dc, (size_t)K, on_device));
     OBB_TRY(copy_back(ctx, points, dp, (size_t)K, on_device));
     if (!on_device) return check_device_error(ctx);
