@@ -66,7 +66,8 @@ struct LatticeFrame {
     double h[3];
     double hmax;
     double center[3];   // lo + N h / 2
-    double s256[3];     // 256 rn(1 / h) (the snap's fast path)
+    double s256[3];     // 256 rn(1 / h)
+    float sf[3][2];     // s256 as two floats (the snap's fast path)
     int32_t N;
     int32_t W;          // uint64 words per row (even)
 };
