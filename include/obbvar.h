@@ -334,8 +334,9 @@ typedef struct {
     int64_t proposals;         /* over all rounds */
     int64_t moves;             /* accepted triangle moves */
     int64_t gain;              /* sum of accepted gains, lattice points */
-    int64_t box_evals;         /* exact box counts performed */
-    uint64_t points_counted;   /* lattice points inside the boxes counted */
+    int64_t box_evals;         /* exact box counts of its rounds and box update (every cluster takes part in every
+                                  round; sibling pairs that have settled keep their last counts) */
+    uint64_t points_counted;   /* lattice points inside those boxes */
     uint64_t total_obv;        /* sum of the layer's outer volumes after the step */
 } obb_step_stats;
 

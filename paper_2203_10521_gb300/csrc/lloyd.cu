@@ -25,8 +25,11 @@
 // Member lists: a stable least-significant-digit radix sort of the triangles
 // by cluster (per-tile digit counts, their exclusive scan, a stable scatter
 // that ranks equal digits with warp matches in triangle order).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
+#include "counting.cuh"
 #include "internal.h"
 
 namespace obbv {
@@ -36,6 +39,7 @@ constexpr int kNT = 128;   // threads of the block-per-cluster kernels
 
 enum { kCtrCand = 0, kCtrEval, kCtrCount };
 
+constexpr int kPairedSlot = 126;   // word of the pinned staging that check_pairs answers in
 constexpr int kMaxTopk = 16;   // candidates a surrogate may keep per source cluster
 
 struct Cand {
@@ -528,6 +532,33 @@ __device__ __forceinline__ void top2_add6(Top2 (&b)[8], const int64_t (&dmin)[3]
     }
 }
 
+// The eight states of every lane reduced and scattered over the warp: lane l
+// ends with state (l >> 2) & 7 of the whole warp.
+__device__ __forceinline__ Top2 top2_reduce(const Top2 (&b)[8], int l)
+{
+    // offset 16: keep states 0-3 (lanes 0-15) or 4-7; state parity (low or
+    // high side) is that of j
+    const bool u16 = (l >> 4) & 1, u8 = (l >> 3) & 1, u4 = (l >> 2) & 1;
+    Top2 t4[4];
+    for (int j = 0; j < 4; ++j) {
+        Top2 keep = u16 ? b[4 + j] : b[j];
+        top2_merge(keep, top2_shfl(u16 ? b[j] : b[4 + j], 16), (j & 1) == 0);
+        t4[j] = keep;
+    }
+    Top2 t2[2];
+    for (int j = 0; j < 2; ++j) {
+        Top2 keep = u8 ? t4[2 + j] : t4[j];
+        top2_merge(keep, top2_shfl(u8 ? t4[j] : t4[2 + j], 8), (j & 1) == 0);
+        t2[j] = keep;
+    }
+    Top2 w = u4 ? t2[1] : t2[0];
+    const bool low = !u4;
+    top2_merge(w, top2_shfl(u4 ? t2[0] : t2[1], 4), low);
+    top2_merge(w, top2_shfl(w, 2), low);
+    top2_merge(w, top2_shfl(w, 1), low);
+    return w;
+}
+
 // Small clusters: a warp per cluster, no block barrier.  Each lane takes
 // every 32nd member, two at a time with both triangles' loads issued before
 // either is projected.  The six states (padded to eight) are then reduced
@@ -576,26 +607,7 @@ __global__ void __launch_bounds__(128) k_extents_small(const int32_t* __restrict
             top2_add6(b, dmin, dmax, ta);
         }
     }
-    // offset 16: keep states 0-3 (lanes 0-15) or 4-7; state parity (low or
-    // high side) is that of j
-    const bool u16 = (l >> 4) & 1, u8 = (l >> 3) & 1, u4 = (l >> 2) & 1;
-    Top2 t4[4];
-    for (int j = 0; j < 4; ++j) {
-        Top2 keep = u16 ? b[4 + j] : b[j];
-        top2_merge(keep, top2_shfl(u16 ? b[j] : b[4 + j], 16), (j & 1) == 0);
-        t4[j] = keep;
-    }
-    Top2 t2[2];
-    for (int j = 0; j < 2; ++j) {
-        Top2 keep = u8 ? t4[2 + j] : t4[j];
-        top2_merge(keep, top2_shfl(u8 ? t4[j] : t4[2 + j], 8), (j & 1) == 0);
-        t2[j] = keep;
-    }
-    Top2 w = u4 ? t2[1] : t2[0];
-    const bool low = !u4;
-    top2_merge(w, top2_shfl(u4 ? t2[0] : t2[1], 4), low);
-    top2_merge(w, top2_shfl(w, 2), low);
-    top2_merge(w, top2_shfl(w, 1), low);
+    const Top2 w = top2_reduce(b, l);
     const int s = (l >> 2) & 7;
     if (live && (l & 3) == 0 && s < 6) {
         ext[k].v1[s] = w.v1;
@@ -785,6 +797,385 @@ __global__ void k_sum_points(const uint64_t* __restrict__ pts, const int32_t* __
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0 && s) atomicAdd((unsigned long long*)&stats[kStPoints], s);
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd((unsigned long long*)&stats[kStEvals], (unsigned long long)n);
+}
+
+// ------------------------------------------------------- rounds of sibling pairs
+//
+// The layers of a binary tree pair their clusters: 2i and 2i + 1 share a
+// parent and no other cluster does.  Moves stay inside a pair and both of its
+// clusters are in every one of them, so a pair accepts at most one move a
+// round, its rounds depend on no other pair, and the range of the member list
+// that its two clusters fill stays where it is.  A cluster of blocks per pair
+// therefore runs all of its rounds in one launch: extents, candidates, the
+// exact counts of their boxes, the best move, and at the end its members in
+// order.  A pair that accepts nothing has settled: its further rounds would
+// count the same boxes again (k_pair_finish adds them to the step's counters,
+// which cover every round of every pair).  Round by round the layer takes 13
+// launches and a round trip to the host each, all pairs in every round: three
+// iterations of 200k triangles in 1,024 clusters 3.3 ms a call, this way 1.3;
+// six with rotation descent of 2M in 16,384 clusters 13.9 and 11.1 ms.
+constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each
+constexpr int kPairMoves = 64;      // most rounds of a step that take this path
+constexpr int kPairGraphMin = 64;   // pairs of a layer whose captured iteration takes it (the launch counter of a small
+                                    // captured layer is read per round)
+
+struct PairArgs {
+    const int32_t *U, *F, *adj;
+    int32_t* assign;
+    obb_qbox* q;
+    uint64_t* obv;
+    int32_t *size, *start, *members, *mnew, *level, *ctr;
+    uint8_t* dirty;
+    int64_t* stats;
+    obb_qbox* evals;        // the last round's boxes and counts of every pair
+    uint64_t *ecount, *epoints;
+    int4* info;             // per pair: rounds run, boxes of its last round, their points (two words)
+    const LatRef* lats;
+    CountOpts o;
+    int32_t rounds, C;
+    unsigned long long* dom;
+    int32_t* err;
+};
+
+struct PairMove {
+    int32_t t, from, now;   // the triangle, its cluster of the pair (0 or 1) before the step and now
+};
+
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
+{
+    constexpr int kWarps = NT / 32;
+    __shared__ Top2 red[2][kWarps][6];
+    __shared__ Top2 ext[2][6];
+    __shared__ obb_qbox box[2], ev[kPairEvals];
+    __shared__ uint64_t obv[2];
+    __shared__ BoxPrep prep[kPairEvals];
+    __shared__ int64_t tiles[kPairEvals];
+    __shared__ unsigned long long sum[kPairEvals], pts[kPairEvals];
+    __shared__ PairMove moved[kPairMoves], mv[kPairMoves];   // the first block's, this block's copy
+    struct Control {
+        int32_t ne, n_moved, need, go;   // boxes to count; moves so far; clusters whose extents change (bits); another round
+        int32_t size[2];
+    };
+    __shared__ Control ctl, cc;          // the first block's, this block's copy
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int32_t C = p.C, pair = blockIdx.x / C, rank = blockIdx.x % C, k0 = 2 * pair;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto sync = [&] {
+        if (C > 1) cluster.sync();
+        else __syncthreads();
+    };
+    const int32_t A = p.start[k0], m0 = p.start[k0 + 1], B = p.start[k0 + 2];
+    if (tid < 2) {
+        box[tid] = p.q[k0 + tid];
+        obv[tid] = p.obv[k0 + tid];
+    }
+    if (tid == 0) {
+        ctl = Control{0, 0, 3, 1, {m0 - A, B - m0}};
+        cc = ctl;
+    }
+    __syncthreads();
+    const Control* ctl0 = cluster.map_shared_rank(&ctl, 0);
+    const PairMove* moved0 = cluster.map_shared_rank(&moved[0], 0);
+    const obb_qbox* ev0 = cluster.map_shared_rank(&ev[0], 0);
+    unsigned long long* sum0 = cluster.map_shared_rank(&sum[0], 0);
+    unsigned long long* pts0 = cluster.map_shared_rank(&pts[0], 0);
+    const bool lead = rank == 0 && warp == 0;   // the warp that chooses
+    // of the first warp's lanes 0-11: candidate of cluster lane / 6, side lane % 6
+    const int my_c = lane < 6 ? 0 : 1, my_side = lane < 6 ? lane : lane - 6;
+    unsigned long long proposals = 0, accepted = 0, gain = 0, e_sum = 0, p_sum = 0, p_last = 0, n_dom = 0;
+    int32_t e_last = 0, ran = 0;
+    for (;;) {
+        // extents of the clusters that lost a triangle (first round: both): the clusters' old segments without
+        // the triangles that have left, then those that have joined
+        for (int c = 0; c < 2; ++c) {
+            if (!(cc.need >> c & 1)) continue;
+            int32_t n[9];
+            for (int i = 0; i < 9; ++i) n[i] = box[c].n[i];
+            Top2 b[8];
+            for (int s = 0; s < 8; ++s) {
+                const int64_t e = (s & 1) ? INT64_MIN : INT64_MAX;
+                b[s] = Top2{e, e, INT32_MAX};
+            }
+            auto add = [&](int32_t t) {
+                int32_t P[9];
+                int64_t dmin[3], dmax[3];
+                load_tri(p.U, p.F, t, P);
+                proj_loaded(P, n, dmin, dmax);
+                top2_add6(b, dmin, dmax, t);
+            };
+            const int32_t s1 = c == 0 ? m0 : B;
+            for (int32_t i = (c == 0 ? A : m0) + rank * NT + tid; i < s1; i += NT * C) {
+                const int32_t t = p.members[i];
+                bool here = true;
+                for (int j = 0; j < cc.n_moved; ++j) here &= mv[j].t != t || mv[j].now == c;
+                if (here) add(t);
+            }
+            if (rank == 0)
+                for (int j = tid; j < cc.n_moved; j += NT)
+                    if (mv[j].from != c && mv[j].now == c) add(mv[j].t);
+            __syncwarp();
+            const Top2 w = top2_reduce(b, lane);
+            const int s = (lane >> 2) & 7;
+            if ((lane & 3) == 0 && s < 6) red[c][warp][s] = w;
+        }
+        sync();
+        if (rank == 0 && tid < 12 && (cc.need >> my_c & 1)) {
+            Top2 w = red[my_c][0][my_side];
+            for (int g = 0; g < C; ++g) {
+                const Top2* r = cluster.map_shared_rank(&red[0][0][0], g);
+                for (int i = g == 0 ? 1 : 0; i < kWarps; ++i)
+                    top2_merge(w, r[(my_c * kWarps + i) * 6 + my_side], (my_side & 1) == 0);
+            }
+            ext[my_c][my_side] = w;
+        }
+        // candidates: a triangle that alone attains a side of its cluster's box, taken by the first such side's
+        // lane, with an edge neighbour in the sibling
+        bool cand = false, grew = false;
+        int32_t t = -1;
+        unsigned vm = 0, gm = 0;
+        if (lead) {
+            __syncwarp();
+            if (lane < 12 && ctl.size[my_c] >= 2 && ext[my_c][my_side].v1 != ext[my_c][my_side].v2) {
+                t = ext[my_c][my_side].t1;
+                cand = true;
+                for (int side = 0; side < my_side; ++side)
+                    cand &= ext[my_c][side].t1 != t || ext[my_c][side].v2 == ext[my_c][side].v1;
+                bool near = false;
+                for (int i = 0; i < 3; ++i) near |= __ldcg(p.assign + p.adj[3 * (int64_t)t + i]) == k0 + 1 - my_c;
+                cand &= near;
+            }
+            int64_t dmin[3], dmax[3];   // the triangle along the sibling's axes
+            if (cand) {
+                int32_t P[9];
+                load_tri(p.U, p.F, t, P);
+                proj_loaded(P, box[1 - my_c].n, dmin, dmax);
+                for (int a = 0; a < 3; ++a)
+                    grew |= dmin[a] < box[1 - my_c].b[2 * a] || dmax[a] > box[1 - my_c].b[2 * a + 1];
+            }
+            vm = __ballot_sync(0xffffffffu, cand);
+            gm = __ballot_sync(0xffffffffu, grew);
+            const unsigned below = (1u << lane) - 1u;
+            if (cand) {
+                obb_qbox& E = ev[__popc(vm & below)];
+                E = box[my_c];
+                for (int side = 0; side < 6; ++side)
+                    if (ext[my_c][side].t1 == t && ext[my_c][side].v2 != ext[my_c][side].v1) E.b[side] = ext[my_c][side].v2;
+            }
+            if (grew) {
+                obb_qbox& E = ev[__popc(vm) + __popc(gm & below)];
+                E = box[1 - my_c];
+                for (int a = 0; a < 3; ++a) {
+                    E.b[2 * a] = min(E.b[2 * a], dmin[a]);
+                    E.b[2 * a + 1] = max(E.b[2 * a + 1], dmax[a]);
+                }
+            }
+            if (lane < kPairEvals) {
+                sum[lane] = 0;
+                pts[lane] = 0;
+            }
+            if (lane == 0) ctl.ne = __popc(vm) + __popc(gm);
+        }
+        sync();
+        const int ne = ctl0->ne;
+        if (warp == 0 && lane < ne)
+            tiles[lane] = prep_box(ev0[lane], 0, p.lats, 1, p.o, max(1, kWarps * C / max(ne, 1)), &prep[lane], p.err);
+        __syncthreads();
+        // the boxes' tiles one after another, dealt out over the warps
+        int64_t at = warp * C + rank;
+        for (int e = 0; e < ne; ++e) {
+            uint32_t x0 = 0, x1 = 0, x2 = 0;
+            unsigned long long empty = 0, inside = 0;
+            const int64_t nt = tiles[e];
+            const bool any = at < nt;
+            for (; at < nt; at += kWarps * C) {
+                const int32_t tk = (int32_t)(at / prep[e].ntj), tj = (int32_t)(at - (int64_t)tk * prep[e].ntj);
+                uint32_t em = 0, in = 0, in_dom = 0;
+                if (count_tile<false>(prep[e], tj, tk, em, in, x0, x1, x2, in_dom)) {
+                    empty += em;
+                    inside += in;
+                    n_dom += in_dom;
+                }
+            }
+            at -= nt;
+            if (!any) continue;   // warp-uniform
+            for (int s = 16; s > 0; s >>= 1) {
+                empty += __shfl_xor_sync(0xffffffffu, empty, s);
+                inside += __shfl_xor_sync(0xffffffffu, inside, s);
+            }
+            if (lane == 0) {
+                if (empty) atomicAdd(&sum0[e], empty);
+                if (inside) atomicAdd(&pts0[e], inside);
+            }
+        }
+        sync();
+        if (lead) {
+            // gains; the best proposal holds the largest key of both clusters and is accepted
+            int64_t g = 0;
+            const unsigned below = (1u << lane) - 1u;
+            const int es = __popc(vm & below), eg = __popc(vm) + __popc(gm & below);
+            if (cand) {
+                const int64_t rem = (int64_t)obv[my_c] - (int64_t)sum[es];
+                const int64_t add = grew ? (int64_t)sum[eg] - (int64_t)obv[1 - my_c] : 0;
+                g = rem - add;
+            }
+            const unsigned long long key =
+                g > 0 ? ((unsigned long long)g << 24) | (unsigned long long)(0xffffff - t) : 0ull;
+            proposals += __popc(__ballot_sync(0xffffffffu, key != 0));
+            unsigned long long best = key;
+            for (int s = 16; s > 0; s >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, s));
+            unsigned long long points = lane < ne ? pts[lane] : 0;
+            for (int s = 16; s > 0; s >>= 1) points += __shfl_xor_sync(0xffffffffu, points, s);
+            ++ran;
+            e_last = ne;
+            p_last = points;
+            e_sum += ne;
+            p_sum += points;
+            const int win = best ? __ffs(__ballot_sync(0xffffffffu, key == best)) - 1 : -1;
+            if (lane == win) {
+                const int to = 1 - my_c;
+                p.assign[t] = k0 + to;
+                for (int i = 0; i < 6; ++i) box[my_c].b[i] = ev[es].b[i];
+                obv[my_c] = sum[es];
+                if (grew) {
+                    for (int i = 0; i < 6; ++i) box[to].b[i] = ev[eg].b[i];
+                    obv[to] = sum[eg];
+                }
+                ctl.size[my_c] -= 1;
+                ctl.size[to] += 1;
+                int j = 0;
+                while (j < ctl.n_moved && moved[j].t != t) ++j;
+                if (j == ctl.n_moved) {
+                    moved[j] = PairMove{t, my_c, to};
+                    ctl.n_moved = j + 1;
+                } else {
+                    moved[j].now = to;
+                }
+                ctl.need = 1 << my_c;
+            }
+            const int32_t tw = __shfl_sync(0xffffffffu, t, max(win, 0));
+            const int to = 1 - __shfl_sync(0xffffffffu, my_c, max(win, 0));
+            if (win >= 0) {
+                accepted += 1;
+                gain += best >> 24;
+                if (lane < 6) {   // the joiner's place among its new cluster's extremes
+                    int32_t P[9];
+                    int64_t dmin[3], dmax[3];
+                    load_tri(p.U, p.F, tw, P);
+                    proj_loaded(P, box[to].n, dmin, dmax);
+                    const int a = lane >> 1;
+                    const int64_t lo = a == 0 ? dmin[0] : a == 1 ? dmin[1] : dmin[2],
+                                  hi = a == 0 ? dmax[0] : a == 1 ? dmax[1] : dmax[2];
+                    top2_add(ext[to][lane], (lane & 1) ? hi : lo, tw, (lane & 1) == 0);
+                }
+            }
+            if (lane == 0) ctl.go = win >= 0 && ran < p.rounds;
+        }
+        sync();
+        if (tid == 0) cc = *ctl0;
+        __syncthreads();
+        for (int j = tid; j < cc.n_moved; j += NT) mv[j] = moved0[j];
+        __syncthreads();
+        if (!cc.go) break;
+    }
+    // the pair's members in order: every triangle's place is its place among those that stay plus the joiners
+    // below it
+    bool net = false;
+    for (int j = 0; j < cc.n_moved; ++j) net |= mv[j].now != mv[j].from;
+    if (net) {
+        const int32_t seg[3] = {A, m0, B};
+        auto shift = [&](int c, int32_t t) {   // joiners minus leavers of cluster c below t
+            int32_t d = 0;
+            for (int j = 0; j < cc.n_moved; ++j)
+                if (mv[j].t < t && mv[j].now != mv[j].from) d += mv[j].now == c ? 1 : -1;
+            return d;
+        };
+        for (int32_t i = A + rank * NT + tid; i < B; i += NT * C) {
+            const int32_t t = p.members[i];
+            const int c = i >= m0;
+            bool stays = true;
+            for (int j = 0; j < cc.n_moved; ++j) stays &= mv[j].t != t || mv[j].now == c;
+            if (stays) p.mnew[(c ? A + cc.size[0] : A) + i - seg[c] + shift(c, t)] = t;
+        }
+        if (rank == 0)
+            for (int j = tid; j < cc.n_moved; j += NT)
+                if (mv[j].now != mv[j].from) {
+                    const int c = mv[j].now;
+                    const int32_t t = mv[j].t;
+                    int32_t lo = seg[c], hi = seg[c + 1];   // the first old member of c above t
+                    while (lo < hi) {
+                        const int32_t mid = (lo + hi) >> 1;
+                        if (p.members[mid] < t) lo = mid + 1;
+                        else hi = mid;
+                    }
+                    p.mnew[(c ? A + cc.size[0] : A) + lo - seg[c] + shift(c, t)] = t;
+                }
+        sync();
+        for (int32_t i = A + rank * NT + tid; i < B; i += NT * C) p.members[i] = __ldcg(p.mnew + i);
+    }
+    if (rank == 0) {
+        if (tid < 2) {
+            const int32_t k = k0 + tid;
+            for (int i = 0; i < 6; ++i) p.q[k].b[i] = box[tid].b[i];
+            p.obv[k] = obv[tid];
+            p.size[k] = cc.size[tid];
+            if (cc.n_moved > 0) {
+                p.dirty[k] = 1;
+                p.level[k] = 0;   // a new member set restarts the box-parameter search
+            }
+        }
+        if (tid == 0) p.start[k0 + 1] = A + cc.size[0];
+        if (warp == 0) {
+            int32_t base = 0;
+            if (lane == 0) {
+                p.info[pair] = make_int4(ran, e_last, (int32_t)(uint32_t)p_last, (int32_t)(uint32_t)(p_last >> 32));
+                base = atomicAdd(&p.ctr[kCtrEval], e_last);
+                atomicMax((unsigned long long*)&p.stats[kStRounds], (unsigned long long)ran);
+                if (proposals) atomicAdd((unsigned long long*)&p.stats[kStProposals], proposals);
+                if (accepted) atomicAdd((unsigned long long*)&p.stats[kStAccepted], accepted);
+                if (gain) atomicAdd((unsigned long long*)&p.stats[kStGain], gain);
+                atomicAdd((unsigned long long*)&p.stats[kStEvals], e_sum);
+                atomicAdd((unsigned long long*)&p.stats[kStPoints], p_sum);
+            }
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (lane < e_last) {
+                p.evals[base + lane] = ev[lane];
+                p.ecount[base + lane] = sum[lane];
+            }
+        }
+    }
+    for (int s = 16; s > 0; s >>= 1) n_dom += __shfl_xor_sync(0xffffffffu, n_dom, s);
+    if (lane == 0 && n_dom) atomicAdd(p.dom, n_dom);
+    if (C > 1) cluster.sync();   // no block leaves while the first one's shared memory is read
+}
+
+// the counters' share of the rounds that settled pairs sat out
+__global__ void k_pair_finish(const int4* __restrict__ info, int32_t pairs, int64_t* __restrict__ stats)
+{
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned long long e = 0, n = 0;
+    if (i < pairs) {
+        const int4 x = info[i];
+        const unsigned long long idle = (unsigned long long)stats[kStRounds] - (unsigned long long)x.x;
+        e = idle * (unsigned long long)x.y;
+        n = idle * ((unsigned long long)(uint32_t)x.z | (unsigned long long)(uint32_t)x.w << 32);
+    }
+    for (int s = 16; s > 0; s >>= 1) {
+        e += __shfl_xor_sync(0xffffffffu, e, s);
+        n += __shfl_xor_sync(0xffffffffu, n, s);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (e) atomicAdd((unsigned long long*)&stats[kStEvals], e);
+        if (n) atomicAdd((unsigned long long*)&stats[kStPoints], n);
+    }
+}
+
+// *paired = 0 unless clusters 2i and 2i + 1 share a parent and no others do (parents ascending by pairs)
+__global__ void k_check_pairs(const int32_t* __restrict__ parent, int32_t K, int32_t* __restrict__ paired)
+{
+    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (2 * i + 1 >= K) return;
+    if (parent[2 * i] != parent[2 * i + 1] || (i > 0 && parent[2 * i - 1] >= parent[2 * i])) *paired = 0;
 }
 
 // ------------------------------------------------------- refit (a9-a11)
@@ -1364,12 +1755,16 @@ struct LayerMem {
     int32_t cand_cap = 0, eval_cap = 0;
     // a whole Lloyd iteration captured as one CUDA graph (see lloyd_step_graph)
     cudaGraphExec_t gexec = nullptr;
-    int gkey[4] = {-1, -1, -1, -1};   // rounds, refit mode, descent steps, counting-tile generation
+    int gkey[5] = {-1, -1, -1, -1, -1};   // rounds, refit mode, descent steps, counting-tile generation, sibling pairs
     int64_t* loop = nullptr;          // [0] rounds run, [1] moves before the round, [2] rebuilds, [3] total
     CountScratch cscr{};              // the graph's own counting scratch (fixed addresses)
     void* cscr_mem = nullptr;
     int64_t g_round = 0, g_rebuild = 0, g_post = 0;   // kernel launches per round, per rebuild, after the loop
     bool members_valid = false;
+    // sibling pairs (k_pair_rounds): 1 / 0 known, -1 to be looked at (parents may have changed)
+    int paired = -1;
+    int4* pinfo = nullptr;      // [K / 2]
+    int32_t* dpaired = nullptr;
     // incremental member lists: mv [2K] the last round's leavers and joiners
     // per cluster (-1 = none), the new list and starts built beside the old
     int32_t* mv = nullptr;
@@ -1477,7 +1872,8 @@ void layer_destroy(obb_layer* L)
         void* mp[] = {M->skeys[0], M->skeys[1], M->svals[0], M->svals[1], M->scnt, M->soff, M->sbsum, M->sticket, M->ctr, M->cand, M->evals, M->ecount, M->epoints, M->mom,
                       M->newframe, M->newq, M->ncount, M->dK, M->feats, M->pred, M->skey,
                       M->slot, M->evals2, M->n2, M->map, M->dirty, M->keep, M->level,
-                      M->pframes, M->pq, M->pbest, M->pcount, M->mv, M->mnew, M->snew};
+                      M->pframes, M->pq, M->pbest, M->pcount, M->mv, M->mnew, M->snew, M->pinfo,
+                      M->dpaired};
         for (void* p : mp)
             if (p) cudaFreeAsync(p, s);
         delete M;
@@ -1507,6 +1903,98 @@ static obb_status init_boxes(obb_ctx* ctx, obb_layer* L, const double* d_frames,
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
     return count_boxes(ctx, lat, L->d_q, M->dK, K, L->d_obv, nullptr);
+}
+
+// Looks whether the layer's clusters are sibling pairs; the answer is on the
+// host (pairs_known) after the next synchronisation.
+static obb_status check_pairs(obb_ctx* ctx, obb_layer* L)
+{
+    LayerMem* M = mem_of(L);
+    int32_t* h = ctx->h_small + kPairedSlot;
+    *h = 0;
+    if (L->K < 2 || (L->K & 1)) return OBB_OK;
+    OBB_CK(ctx, cudaMemsetAsync(M->dpaired, 0xff, sizeof(int32_t), ctx->stream));
+    k_check_pairs<<<(L->K / 2 + 127) / 128, 128, 0, ctx->stream>>>(L->d_parent, L->K, M->dpaired);
+    note_launch(ctx);
+    OBB_CK(ctx, cudaMemcpyAsync(h, M->dpaired, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    return OBB_OK;
+}
+
+static void pairs_known(obb_ctx* ctx, obb_layer* L) { mem_of(L)->paired = ctx->h_small[kPairedSlot] != 0 ? 1 : 0; }
+
+void layer_parents_changed(obb_layer* L) { mem_of(L)->paired = -1; }
+
+// Whether the layer's rounds run pair by pair (k_pair_rounds).
+static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, bool* yes)
+{
+    LayerMem* M = mem_of(L);
+    *yes = false;
+    if (ctx->prof != 0 || ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
+    if (M->paired < 0) {
+        OBB_TRY(check_pairs(ctx, L));
+        OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
+        pairs_known(ctx, L);
+    }
+    *yes = M->paired == 1;
+    return OBB_OK;
+}
+
+// All partition rounds of a layer of sibling pairs, without host synchronisation (the counters zeroed here).
+static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
+{
+    cudaStream_t s = ctx->stream;
+    LayerMem* M = mem_of(L);
+    const obb_lattice* lat = L->lat;
+    const int32_t pairs = L->K / 2;
+    OBB_CK(ctx, cudaMemsetAsync(L->d_stats, 0, sizeof(int64_t) * kStCount, s));
+    OBB_CK(ctx, cudaMemsetAsync(M->ctr, 0, sizeof(int32_t) * kCtrCount, s));
+    PairArgs a{};
+    a.U = lat->d_fixed;
+    a.F = lat->mesh->d_tris;
+    a.adj = lat->mesh->d_adj;
+    a.assign = L->d_assign;
+    a.q = L->d_q;
+    a.obv = L->d_obv;
+    a.size = L->d_size;
+    a.start = L->d_start;
+    a.members = L->d_members;
+    a.mnew = M->mnew;
+    a.level = M->level;
+    a.ctr = M->ctr;
+    a.dirty = M->dirty;
+    a.stats = L->d_stats;
+    a.evals = M->evals;
+    a.ecount = M->ecount;
+    a.epoints = M->epoints;
+    a.info = M->pinfo;
+    a.lats = lat->d_ref;
+    a.o = CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank};
+    a.rounds = rounds;
+    a.dom = ctx->d_prof + 2;
+    a.err = ctx->d_err;
+    // Threads and blocks per pair: 128 threads, eight blocks a pair while there are few (a tree's upper levels;
+    // 256 threads lengthen the chooser's serial part: 5.1 against 4.7 ms for the tree of 7k triangles) and one
+    // from 1,024 pairs on (8,192 pairs: 11.05 against 12.07 ms for six iterations); in between 256 threads, as
+    // many blocks as are resident at once (512 pairs: 1.28 against 1.43 ms for three iterations).
+    const bool mid = pairs >= 128 && pairs < 1024;
+    int32_t C = 8;
+    while (C > 1 && (int64_t)C * pairs > (mid ? 2 : 8) * ctx->num_sms) C >>= 1;
+    a.C = C;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)pairs * C);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cfg.blockDim = dim3(mid ? 256 : 128);
+    OBB_CK(ctx, mid ? cudaLaunchKernelEx(&cfg, k_pair_rounds<256>, a) : cudaLaunchKernelEx(&cfg, k_pair_rounds<128>, a));
+    k_pair_finish<<<(pairs + 255) / 256, 256, 0, s>>>(M->pinfo, pairs, L->d_stats);
+    note_launch(ctx, 2);
+    OBB_CK(ctx, cudaGetLastError());
+    return OBB_OK;
 }
 
 obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_assign, const int32_t* d_parent,
@@ -1583,6 +2071,8 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     A_(dalloc(&M->pcount, (size_t)kProbes * K, s));
     A_(dalloc(&M->mv, 2 * (size_t)K, s));
     A_(dalloc(&M->mnew, T, s));
+    A_(dalloc(&M->pinfo, (size_t)(K + 1) / 2, s));
+    A_(dalloc(&M->dpaired, 1, s));
     A_(dalloc(&M->snew, (size_t)K + 1, s));
 #undef A_
     if (e != cudaSuccess) {
@@ -1600,7 +2090,9 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     if (st == OBB_OK) {
         k_check_nonempty<<<(K + 255) / 256, 256, 0, s>>>(L->d_size, K, ctx->d_err);
         note_launch(ctx);
-        st = check_device_error(ctx);   // assignment range / empty clusters before any box work
+        st = check_pairs(ctx, L);
+        if (st == OBB_OK) st = check_device_error(ctx);   // assignment range / empty clusters before any box work
+        if (st == OBB_OK) pairs_known(ctx, L);
     }
     if (st == OBB_OK) st = init_boxes(ctx, L, d_frames, d_fallback);
     if (st == OBB_OK) st = check_device_error(ctx);
@@ -1676,6 +2168,14 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
     const int refit_mode = opts ? opts->refit : 1;
     const int dsteps = (opts && opts->descent_steps > 0) ? opts->descent_steps : 2;
     if (opts && opts->graph && !L->mlp) return lloyd_step_graph(ctx, L, rounds, refit_mode, dsteps, st);
+    bool pairs = false;
+    OBB_TRY(pair_path(ctx, L, rounds, &pairs));
+    if (pairs) {
+        if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
+        OBB_TRY(pair_rounds(ctx, L, rounds));
+        OBB_TRY(layer_box_update(ctx, L, refit_mode, dsteps));
+        return layer_finish_stats(ctx, L, -1, st);
+    }
     OBB_CK(ctx, cudaMemsetAsync(L->d_stats, 0, sizeof(int64_t) * kStCount, s));
     int64_t* h = host_stats(ctx);
     int ran = 0;
@@ -1711,8 +2211,10 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
     const int K = L->K;
     cudaStream_t s = ctx->stream;
     if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
+    bool pairs = false;
+    if (K / 2 >= kPairGraphMin) OBB_TRY(pair_path(ctx, L, rounds, &pairs));
     if (!M->gexec || M->gkey[0] != rounds || M->gkey[1] != refit_mode || M->gkey[2] != dsteps ||
-        M->gkey[3] != ctx->tile_gen) {
+        M->gkey[3] != ctx->tile_gen || M->gkey[4] != (int)pairs) {
         if (M->gexec) {
             OBB_CK(ctx, cudaGraphExecDestroy(M->gexec));
             M->gexec = nullptr;
@@ -1750,6 +2252,31 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
             ctx->stream = cs[0];
             if (!ck(cudaStreamBeginCapture(cs[0], cudaStreamCaptureModeThreadLocal))) break;
             depth = 1;
+            // the box update and the layer total, after the rounds
+            auto finish = [&]() -> bool {
+                ctx->stream = cs[0];
+                const int64_t l2 = ctx->launches;
+                rc = layer_box_update(ctx, L, refit_mode, dsteps);
+                if (rc != OBB_OK) return false;
+                k_total<<<1, 1024, 0, cs[0]>>>(L->d_obv, K, M->loop + 3);
+                note_launch(ctx);
+                M->g_post = ctx->launches - l2;
+                if (!ck(cudaGetLastError())) return false;
+                if (!ck(cudaStreamEndCapture(cs[0], &g))) return false;
+                depth = 0;
+                return ck(cudaGraphInstantiate(&M->gexec, g, 0));
+            };
+            if (pairs) {
+                // sibling pairs: every round in one launch
+                ck(cudaMemsetAsync(M->loop, 0, sizeof(int64_t) * 4, cs[0]));
+                const int64_t l0 = ctx->launches;
+                rc = pair_rounds(ctx, L, rounds);
+                if (rc != OBB_OK) break;
+                const int64_t n = ctx->launches - l0;
+                M->g_round = M->g_rebuild = 0;
+                if (finish()) M->g_post += n;
+                break;
+            }
             ck(cudaMemsetAsync(L->d_stats, 0, sizeof(int64_t) * kStCount, cs[0]));
             ck(cudaMemsetAsync(M->loop, 0, sizeof(int64_t) * 4, cs[0]));
             cudaStreamCaptureStatus cst;
@@ -1806,18 +2333,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
             depth = 2;
             if (!ck(cudaStreamEndCapture(cs[1], &bg))) break;
             depth = 1;
-            // the box update and the layer total
-            ctx->stream = cs[0];
-            const int64_t l2 = ctx->launches;
-            rc = layer_box_update(ctx, L, refit_mode, dsteps);
-            if (rc != OBB_OK) break;
-            k_total<<<1, 1024, 0, cs[0]>>>(L->d_obv, K, M->loop + 3);
-            note_launch(ctx);
-            M->g_post = ctx->launches - l2;
-            if (!ck(cudaGetLastError())) break;
-            if (!ck(cudaStreamEndCapture(cs[0], &g))) break;
-            depth = 0;
-            if (!ck(cudaGraphInstantiate(&M->gexec, g, 0))) break;
+            finish();
         } while (false);
         // close whatever capture is still open, innermost first
         for (int d = depth; d >= 1; --d) {
@@ -1837,6 +2353,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
         M->gkey[1] = refit_mode;
         M->gkey[2] = dsteps;
         M->gkey[3] = ctx->tile_gen;
+        M->gkey[4] = (int)pairs;
     }
     OBB_CK(ctx, cudaGraphLaunch(M->gexec, s));
     int64_t* h = host_stats(ctx);
@@ -1844,7 +2361,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
     OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, M->loop, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost, s));
     OBB_TRY(check_device_error(ctx));
     M->members_valid = true;
-    const int64_t ran = h[kStCount], rebuilds = h[kStCount + 2];
+    const int64_t ran = pairs ? h[kStRounds] : h[kStCount], rebuilds = h[kStCount + 2];
     note_launch(ctx, (int)(M->g_round * ran + M->g_rebuild * rebuilds + M->g_post));
     if (st) {
         st->rounds_run = (int32_t)ran;
@@ -2368,7 +2885,7 @@ obb_status layer_finish_stats(obb_ctx* ctx, obb_layer* L, int ran, obb_step_stat
         OBB_CK(ctx, cudaMemcpyAsync(h, L->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
         OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, ctx->tmp_d.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         OBB_TRY(check_device_error(ctx));
-        st->rounds_run = ran;
+        st->rounds_run = ran >= 0 ? ran : (int32_t)h[kStRounds];   // < 0: counted on the device
         st->refits_accepted = (int32_t)h[kStRefits];
         st->proposals = h[kStProposals];
         st->moves = h[kStAccepted];

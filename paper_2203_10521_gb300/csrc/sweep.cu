@@ -426,6 +426,7 @@ obb_status unit_step(obb_ctx* ctx, obb_layer* up, obb_layer* low, const obb_step
         k_unit_assign<<<gT, 256, 0, s>>>(low->d_assign, low->d_parent, T, up->d_assign);
         note_launch(ctx);
         layer_members_changed(up);
+        layer_parents_changed(low);
     }
     OBB_TRY(layer_box_update(ctx, up, refit_mode, dsteps));
     return layer_finish_stats(ctx, up, ran, st);
