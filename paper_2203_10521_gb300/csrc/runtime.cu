@@ -819,16 +819,10 @@ obb_status obb_tree_score(obb_ctx* ctx, const obb_tree* tree, double* points, do
     if (!ctx || !tree) return fail(ctx, OBB_ERR_ARG, "null argument");
     if (tree->ctx != ctx) return fail(ctx, OBB_ERR_STATE, "tree belongs to another context");
     const int depth = (int)tree->layers.size() - 1;
+    uint64_t* h = reinterpret_cast<uint64_t*>(host_stats(ctx));
+    OBB_TRY(obbv::tree_totals(ctx, tree, h));
     double acc = 0.0;
-    for (int L = 0; L <= depth; ++L) {
-        const obb_layer* ly = tree->layers[L];
-        std::vector<uint64_t> o(ly->K);
-        OBB_CK(ctx, cudaMemcpyAsync(o.data(), ly->d_obv, sizeof(uint64_t) * ly->K, cudaMemcpyDeviceToHost, ctx->stream));
-        OBB_TRY(check_device_error(ctx));
-        double sum = 0.0;
-        for (uint64_t v : o) sum += (double)v;
-        acc += (double)(depth - L + 1) * sum;
-    }
+    for (int L = 0; L <= depth; ++L) acc += (double)(depth - L + 1) * (double)h[L];
     if (points) *points = acc;
     if (volume) {
         OBB_TRY(obbv::lattice_frame_host(tree->lat));

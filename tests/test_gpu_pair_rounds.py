@@ -121,3 +121,12 @@ def test_parents_changed_by_a_unit_step(ctx, torus, upper):
     assert out[0][0] == out[1][0]
     assert np.array_equal(out[0][1], out[1][1])
     _same(out[0][2], out[1][2])
+
+
+@pytest.mark.parametrize("depth", [0, 1, 9, 13])
+def test_tree_score_is_the_weighted_sum_of_its_levels(ctx, torus, depth):
+    lat, _ = torus
+    tree = ctx.build_tree(lat, depth, 0)
+    want = sum((depth - lev + 1) * int(ctx.tree_read(tree, lev)["obv"].sum()) for lev in range(depth + 1))
+    assert ctx.tree_score(tree)[0] == want
+    tree.free()
