@@ -1973,9 +1973,11 @@ static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
     a.dom = ctx->d_prof + 2;
     a.err = ctx->d_err;
     // Threads and blocks per pair: 128 threads, eight blocks a pair while there are few (a tree's upper levels;
-    // 256 threads lengthen the chooser's serial part: 5.1 against 4.7 ms for the tree of 7k triangles) and one
-    // from 1,024 pairs on (8,192 pairs: 11.05 against 12.07 ms for six iterations); in between 256 threads, as
-    // many blocks as are resident at once (512 pairs: 1.28 against 1.43 ms for three iterations).
+    // 256 threads lengthen the chooser's serial part: 5.1 against 4.7 ms for the tree of 7k triangles at 132^3)
+    // unless the boxes are large (from 32,768 lattice rows a pair on; four pairs at 1024^3: 2.36 against 3.22 ms
+    // for four iterations), and one from 1,024 pairs on (8,192 pairs: 11.05 against 12.07 ms for six iterations);
+    // in between 256 threads, as many blocks as are resident at once (512 pairs: 1.28 against 1.43 ms for three
+    // iterations).  Clusters of sixteen blocks: no faster.
     const bool mid = pairs >= 128 && pairs < 1024;
     int32_t C = 8;
     while (C > 1 && (int64_t)C * pairs > (mid ? 2 : 8) * ctx->num_sms) C >>= 1;
@@ -1989,8 +1991,9 @@ static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cfg.blockDim = dim3(mid ? 256 : 128);
-    OBB_CK(ctx, mid ? cudaLaunchKernelEx(&cfg, k_pair_rounds<256>, a) : cudaLaunchKernelEx(&cfg, k_pair_rounds<128>, a));
+    const bool big = mid || (int64_t)lat->frame.N * lat->frame.N >= 32768 * (int64_t)pairs;
+    cfg.blockDim = dim3(big ? 256 : 128);
+    OBB_CK(ctx, big ? cudaLaunchKernelEx(&cfg, k_pair_rounds<256>, a) : cudaLaunchKernelEx(&cfg, k_pair_rounds<128>, a));
     k_pair_finish<<<(pairs + 255) / 256, 256, 0, s>>>(M->pinfo, pairs, L->d_stats);
     note_launch(ctx, 2);
     OBB_CK(ctx, cudaGetLastError());

@@ -123,6 +123,26 @@ def test_parents_changed_by_a_unit_step(ctx, torus, upper):
     _same(out[0][2], out[1][2])
 
 
+@pytest.mark.parametrize("level", [1, 2, 3])
+def test_few_pairs_on_a_large_lattice(ctx, level):
+    """Two pairs or fewer at 257^3 take wider blocks, four do not."""
+    m = M.torus(1.0, 0.3, 60, 24, jitter=0.004, seed=11)
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, 257)
+    tree = ctx.build_tree(lat, level, 0)
+    r = ctx.tree_read(tree, level)
+    parent = (np.arange(1 << level) // 2).astype(np.int32)
+    out = []
+    for prof in (0, 2):
+        layer = ctx.layer_init(lat, r["assign"], parent, r["frames"])
+        out.append((_step(ctx, layer, prof, rounds=6, refit=2), ctx.layer_read(layer)))
+        layer.free()
+    assert out[0][0] == out[1][0]
+    _same(out[0][1], out[1][1])
+    for x in (tree, lat, mesh):
+        x.free()
+
+
 @pytest.mark.parametrize("depth", [0, 1, 9, 13])
 def test_tree_score_is_the_weighted_sum_of_its_levels(ctx, torus, depth):
     lat, _ = torus
