@@ -420,7 +420,7 @@ obb_status mesh_upload(obb_ctx* ctx, const float* verts, int64_t nv, const int32
 
 // tree.cu
 obb_status build_tree(obb_ctx* ctx, const obb_lattice* lat, const obb_tree_opts* opts, obb_tree* tree);
-obb_status split_layer(obb_ctx* ctx, const obb_layer* up, int32_t* d_child);
+obb_status split_layer(obb_ctx* ctx, const obb_layer* up, int32_t* d_child, bool even);
 // every level's total outer volume into host[0 .. levels) (at most kMaxLevels; synchronises)
 constexpr int kMaxLevels = 21;
 obb_status tree_totals(obb_ctx* ctx, const obb_tree* tree, uint64_t* host);

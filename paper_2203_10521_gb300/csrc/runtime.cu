@@ -766,7 +766,7 @@ obb_status obb_layer_split(obb_ctx* ctx, const obb_layer* L, int32_t* child, int
     HostTmp hc(ctx);
     int32_t* dc;
     OBB_TRY(out_device(ctx, child, (size_t)L->T, on_device, hc, &dc));
-    OBB_TRY(split_layer(ctx, L, dc));
+    OBB_TRY(split_layer(ctx, L, dc, false));
     OBB_TRY(copy_back(ctx, child, dc, (size_t)L->T, on_device));
     return check_device_error(ctx);
 }
