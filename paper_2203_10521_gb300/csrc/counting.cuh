@@ -24,6 +24,36 @@
 #endif
 
 namespace obbv {
+// rint(2^24 rn(rn(r h_b) / hmax)): an entry of a box's integer normals
+__device__ __noinline__ inline int32_t normal_exact(double r, const LatticeFrame* __restrict__ f, int b)
+{
+    return (int32_t)rint(__dmul_rn(__ddiv_rn(__dmul_rn(r, f->h[b]), f->hmax), 16777216.0));
+}
+
+// The same in integers: an FP64 instruction holds its scheduler for 64 cycles
+// however many lanes take part (measured: a dependent chain and four
+// independent ones both issue one in 64), and the defining sequence has
+// thirteen.  With |r| < 2, x = floor(2^61 |r|) and y = x ratio / 2^64 is
+// |r| h / hmax in units of 2^-60 within 258 of them (2^-53 of the ratio, the
+// truncations); the rounded sequence is within 2^-52 of its value, 512 units.
+// Farther than 4,096 units from a half-integer multiple of 2^36 both round to
+// the same integer; else (1 entry in 2^23), or out of range, the sequence decides.
+__device__ __forceinline__ int32_t normal_entry(double r, const LatticeFrame* __restrict__ f, int b)
+{
+    const uint64_t v = (uint64_t)__double_as_longlong(r);
+    const int sh = 1014 - ((int)(v >> 52) & 0x7ff);   // |r| 2^61 = m 2^-sh
+    if (sh >= -9) {
+        const uint64_t m = (v & ((1ull << 52) - 1)) | (1ull << 52);
+        const uint64_t x = sh <= 0 ? m << -sh : sh < 64 ? m >> sh : 0;
+        const uint64_t y = __umul64hi(x, f->ratio[b]) + (1ull << 35);
+        if ((y & ((1ull << 36) - 1)) - 4096 < (1ull << 36) - 8192) {
+            const int32_t n = (int32_t)(y >> 36);
+            return (int64_t)v < 0 ? -n : n;
+        }
+    }
+    return normal_exact(r, f, b);
+}
+
 // unroll factor of the row loop, margin rows of a box's rectangle
 constexpr int kCountUnroll = OBB_COUNT_UNROLL;
 constexpr int kRowMargin = OBB_ROW_MARGIN;

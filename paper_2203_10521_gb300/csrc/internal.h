@@ -68,6 +68,8 @@ struct LatticeFrame {
     double center[3];   // lo + N h / 2
     double s256[3];     // 256 rn(1 / h)
     float sf[3][2];     // s256 as two floats (the snap's fast path)
+    uint64_t ratio[3];  // 2^63 rn(h / hmax)
+    double s32;         // rn(2^32 / hmax)
     int32_t N;
     int32_t W;          // uint64 words per row (even)
 };
@@ -209,7 +211,7 @@ struct obb_ctx {
     int32_t tile_gen = 0;            // bumped when tile_k changes (captured steps recapture)
     int32_t* h_small = nullptr;      // pinned host staging (512 bytes; the first 64 hold the error word)
     // scratch reused across calls
-    obbv::DevBuf prep, chunk_off, qscratch, cscratch, pscratch, kdev, tmp_a, tmp_b, tmp_c, tmp_d,
+    obbv::DevBuf prep, chunk_off, cscratch, pscratch, kdev, tmp_a, tmp_b, tmp_c, tmp_d,
         cub_tmp, order;
     unsigned int* d_order_hist = nullptr;   // spatial-order buckets of the counting path
     // instrumentation: kernels launched by this context, and the optional
@@ -356,7 +358,8 @@ obb_status count_float_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box
 // lattice_bytes (the lattices' occupancy words together) decides the spatial order
 obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats, const int32_t* d_lat_of_box,
                              const obb_qbox* d_boxes, const int32_t* d_K, int64_t K_cap, uint64_t* d_counts,
-                             uint64_t* d_points, int64_t lattice_bytes);
+                             uint64_t* d_points, int64_t lattice_bytes,
+                             const obb_box* d_fboxes = nullptr, const LatticeFrame* d_frame = nullptr);
 obb_status set_device_int(obb_ctx* ctx, int32_t* d_dst, int32_t value);
 // Count the recorded requests in one multi-lattice launch: their boxes are
 // gathered into one list (device-side offsets from each request's box count),

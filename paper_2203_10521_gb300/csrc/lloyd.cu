@@ -1370,20 +1370,14 @@ __global__ void k_frames_from_moments(const double* __restrict__ mom, const doub
     jacobi3(c6, R);
 }
 
-// n_ab = rint(2^24 ((R_ab h_b) / h_max)), each step correctly rounded
+// n_ab = rint(2^24 ((R_ab h_b) / h_max)), each step correctly rounded (normal_entry)
 __global__ void k_normals(const double* __restrict__ frames, int32_t K, const LatticeFrame* __restrict__ f,
                           obb_qbox* __restrict__ q, const uint8_t* __restrict__ active)
 {
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K || (active && !active[k])) return;
-    const double hm = f->hmax;
     for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-            double t = __dmul_rn(frames[9 * (int64_t)k + 3 * a + b], f->h[b]);
-            t = __ddiv_rn(t, hm);
-            t = __dmul_rn(t, 16777216.0);
-            q[k].n[3 * a + b] = (int32_t)rint(t);
-        }
+        for (int b = 0; b < 3; ++b) q[k].n[3 * a + b] = normal_entry(frames[9 * (int64_t)k + 3 * a + b], f, b);
     q[k].reserved = 0;
 }
 

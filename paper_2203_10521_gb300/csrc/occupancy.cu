@@ -100,8 +100,12 @@ __global__ void __launch_bounds__(kAabbThreads) k_aabb_frame(const float* __rest
         f->sf[b][1] = (float)__dsub_rn(s, (double)sf);
     }
     __syncthreads();
+    const double hmax = fmax(0.0, fmax(f->h[0], fmax(f->h[1], f->h[2])));
+    if (threadIdx.x < 3)
+        f->ratio[threadIdx.x] = hmax > 0.0 ? (uint64_t)__dmul_rn(__ddiv_rn(f->h[threadIdx.x], hmax), 0x1p63) : 0;
+    if (threadIdx.x == 32) f->s32 = __ddiv_rn(4294967296.0, hmax);
     if (threadIdx.x == 0) {
-        f->hmax = fmax(0.0, fmax(f->h[0], fmax(f->h[1], f->h[2])));
+        f->hmax = hmax;
         f->N = N;
         f->W = 2 * ((N + 127) / 128);
         *ticket = 0;   // ready for the next launch

@@ -65,12 +65,10 @@ namespace {
 
 // ---------------------------------------------------------------- quantise
 
-__global__ void k_quantize(const obb_box* __restrict__ boxes, int64_t K, const LatticeFrame* __restrict__ f,
-                           obb_qbox* __restrict__ out, int32_t* err)
+// A box that is not finite, has a negative half-extent or does not fit 63 bits
+// becomes an empty one.
+__device__ __forceinline__ obb_qbox quantize_box(const obb_box& B, const LatticeFrame* __restrict__ f, int32_t* err)
 {
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const obb_box B = boxes[k];
     const float* raw = reinterpret_cast<const float*>(&B);
     bool bad = false;
     for (int q = 0; q < 12; ++q) bad |= !isfinite(raw[q]);
@@ -82,40 +80,37 @@ __global__ void k_quantize(const obb_box* __restrict__ boxes, int64_t K, const L
     R[6] = __dsub_rn(__dmul_rn(R[1], R[5]), __dmul_rn(R[2], R[4]));
     R[7] = __dsub_rn(__dmul_rn(R[2], R[3]), __dmul_rn(R[0], R[5]));
     R[8] = __dsub_rn(__dmul_rn(R[0], R[4]), __dmul_rn(R[1], R[3]));
-    const double hm = f->hmax;
-    const double s = __ddiv_rn(4294967296.0, hm);
+    double d[3];
+    for (int b = 0; b < 3; ++b) d[b] = __dsub_rn(__dsub_rn((double)B.c[b], f->lo[b]), 0.5 * f->h[b]);
     obb_qbox o;
     o.reserved = 0;
     for (int a = 0; a < 3; ++a) {
-        for (int b = 0; b < 3; ++b) {
-            double t = __dmul_rn(R[3 * a + b], f->h[b]);
-            t = __ddiv_rn(t, hm);
-            t = __dmul_rn(t, 16777216.0);
-            o.n[3 * a + b] = (int32_t)rint(t);
-        }
-        double half = (double)B.half[a];
-        bad |= !(half >= 0.0);
-        double m = 0.0;
-        for (int b = 0; b < 3; ++b) {
-            double d = __dsub_rn((double)B.c[b], f->lo[b]);
-            d = __dsub_rn(d, 0.5 * f->h[b]);
-            m = __dadd_rn(m, __dmul_rn(R[3 * a + b], d));
-        }
-        double lo = floor(__dmul_rn(__dsub_rn(m, half), s));
-        double hi = ceil(__dmul_rn(__dadd_rn(m, half), s));
-        if (!(fabs(lo) < 4.0e18 && fabs(hi) < 4.0e18)) bad = true;
-        o.b[2 * a] = bad ? 0 : (int64_t)lo;
-        o.b[2 * a + 1] = bad ? -1 : (int64_t)hi;
+        bad |= !(B.half[a] >= 0.0f);
+        const double half = (double)B.half[a];
+        double m = __dmul_rn(R[3 * a], d[0]);
+        for (int b = 1; b < 3; ++b) m = __dadd_rn(m, __dmul_rn(R[3 * a + b], d[b]));
+        const double lo = __dmul_rn(__dsub_rn(m, half), f->s32), hi = __dmul_rn(__dadd_rn(m, half), f->s32);
+        bad |= !(fabs(lo) < 4.0e18 && fabs(hi) < 4.0e18);   // whole numbers there: floor and ceil change nothing
+        o.b[2 * a] = __double2ll_rd(lo);
+        o.b[2 * a + 1] = __double2ll_ru(hi);
+        for (int b = 0; b < 3; ++b) o.n[3 * a + b] = normal_entry(R[3 * a + b], f, b);
     }
     if (bad) {
         atomicOr(err, kErrArg);
-        for (int q = 0; q < 9; ++q) o.n[q] = (q % 4 == 0) ? 1 : 0;
+        for (int q = 0; q < 9; ++q) o.n[q] = q % 4 == 0 ? 1 : 0;
         for (int a = 0; a < 3; ++a) {
             o.b[2 * a] = 0;
             o.b[2 * a + 1] = -1;   // empty
         }
     }
-    out[k] = o;
+    return o;
+}
+
+__global__ void k_quantize(const obb_box* __restrict__ boxes, int64_t K, const LatticeFrame* __restrict__ f,
+                           obb_qbox* __restrict__ out, int32_t* err)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k < K) out[k] = quantize_box(boxes[k], f, err);
 }
 
 // ------------------------------------------------------------------- prep
@@ -130,8 +125,13 @@ constexpr int32_t kShortTileBoxes = 128;
 // One box per thread (prep_box), counts zeroed on the way; then the last
 // block to finish (an atomic ticket, nothing waits) turns the tile counts into
 // offsets: off[0..K] exclusive, off[K + 1] = 0 (the counting kernel's work
-// counter).
+// counter).  kFloat: float boxes, quantised on the way (32,752 boxes at 1024^3:
+// 29.6 us, 42 with a quantisation launch before it; three warps a block that
+// share the FP64 work: 40 us).
+template <bool kFloat>
 __global__ void __launch_bounds__(kPrepThreads) k_prep(const obb_qbox* __restrict__ boxes,
+                                                       const obb_box* __restrict__ fboxes,
+                                                       const LatticeFrame* __restrict__ frame,
                                                        const int32_t* __restrict__ d_K, int32_t K_val,
                                                        const LatRef* __restrict__ lats, int32_t n_lats,
                                                        const int32_t* __restrict__ lat_of_box, const CountOpts o,
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(const obb_qbox* __restric
     if (k < K) {
         counts[k] = 0;
         if (points) points[k] = 0;
-        tiles[k] = prep_box(boxes[k], lat_of_box ? lat_of_box[k] : 0, lats, n_lats, o, warps, &prep[k], err);
+        tiles[k] = prep_box(kFloat ? quantize_box(fboxes[k], frame, err) : boxes[k], lat_of_box ? lat_of_box[k] : 0, lats, n_lats, o, warps, &prep[k], err);
         if (bucket) {
             // spatial order: the 16^3 Morton cell of the centre of the box's
             // index-space rectangle (clamped to the lattice)
@@ -253,11 +253,11 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(const obb_qbox* __restric
 // at the same place (the place within a bucket depends on scheduling; counts
 // do not depend on the order)
 __global__ void k_order_scatter(const uint32_t* __restrict__ bucket, const int64_t* __restrict__ tiles,
-                                const int32_t* __restrict__ d_K, unsigned int* __restrict__ hist,
+                                const int32_t* __restrict__ d_K, int32_t K_val, unsigned int* __restrict__ hist,
                                 int32_t* __restrict__ perm, int64_t* __restrict__ ptiles)
 {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int32_t K = *d_K;
+    const int32_t K = d_K ? *d_K : K_val;
     if (k >= K) return;
     const unsigned int pos = atomicAdd(&hist[bucket[k]], 1u);
     if (pos < (unsigned int)K) {
@@ -279,10 +279,11 @@ constexpr int kScanPer = 8;
 static_assert(256 * kScanPer == kScanBlock, "offset scan: 256 threads x kScanPer positions per block");
 
 __global__ void __launch_bounds__(256) k_tile_sums(const int64_t* __restrict__ tiles,
-                                                    const int32_t* __restrict__ d_K, int64_t* __restrict__ bsum)
+                                                    const int32_t* __restrict__ d_K, int32_t K_val,
+                                                    int64_t* __restrict__ bsum)
 {
     __shared__ int64_t ws[8];
-    const int32_t K = *d_K;
+    const int32_t K = d_K ? *d_K : K_val;
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
     int64_t v = 0;
 #pragma unroll
@@ -299,11 +300,12 @@ __global__ void __launch_bounds__(256) k_tile_sums(const int64_t* __restrict__ t
 
 __global__ void __launch_bounds__(256) k_tile_offsets(const int64_t* __restrict__ tiles,
                                                        const int64_t* __restrict__ bsum,
-                                                       const int32_t* __restrict__ d_K, int64_t* __restrict__ off)
+                                                       const int32_t* __restrict__ d_K, int32_t K_val,
+                                                       int64_t* __restrict__ off)
 {
     __shared__ int64_t ws[8];
     __shared__ int64_t before;
-    const int32_t K = *d_K;
+    const int32_t K = d_K ? *d_K : K_val;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     // the totals of the blocks before this one
     int64_t p = 0;
@@ -572,68 +574,39 @@ __global__ void __launch_bounds__(256, kMinB) k_count(const BoxPrep* __restrict_
 
 // ------------------------------------------------------------- few boxes
 
-// k_quantize's arithmetic for one box by one warp: an entry of n or a slab a lane
+// quantize_box's arithmetic for one box by one warp, an entry of n, a term of
+// a slab's centre or a bound a lane: 17 FP64 instructions in a row instead of
+// 75, of 64 cycles each.
 __device__ __forceinline__ void quantize_warp(const obb_box& B, const LatticeFrame* __restrict__ f, obb_qbox* out,
                                               int32_t* err)
 {
     const int lane = threadIdx.x & 31;
     const float* raw = reinterpret_cast<const float*>(&B);
     bool bad = lane < 12 && !isfinite(raw[lane < 12 ? lane : 0]);
-    const int a = lane < 9 ? lane / 3 : min(lane - 9, 2);   // lanes 0-8: n_ab, lanes 9-11: slab a
-    double R[3];
-    if (a < 2) {
-        const float* ax = a == 0 ? B.axis0 : B.axis1;
-        for (int b = 0; b < 3; ++b) R[b] = (double)ax[b];
-    } else {
-        double u[3], v[3];
-        for (int b = 0; b < 3; ++b) {
-            u[b] = (double)B.axis0[b];
-            v[b] = (double)B.axis1[b];
-        }
-        R[0] = __dsub_rn(__dmul_rn(u[1], v[2]), __dmul_rn(u[2], v[1]));
-        R[1] = __dsub_rn(__dmul_rn(u[2], v[0]), __dmul_rn(u[0], v[2]));
-        R[2] = __dsub_rn(__dmul_rn(u[0], v[1]), __dmul_rn(u[1], v[0]));
-    }
-    const double hm = f->hmax;
-    int32_t n = 0;
-    int64_t lo = 0, hi = -1;
-    if (lane < 9) {
-        const int b = lane % 3;
-        double t = __dmul_rn(b == 0 ? R[0] : b == 1 ? R[1] : R[2], f->h[b]);
-        t = __ddiv_rn(t, hm);
-        t = __dmul_rn(t, 16777216.0);
-        n = (int32_t)rint(t);
-    } else if (lane < 12) {
-        const double s = __ddiv_rn(4294967296.0, hm);
-        const double half = (double)B.half[a];
-        bad |= !(half >= 0.0);
-        double m = 0.0;
-        for (int b = 0; b < 3; ++b) {
-            double d = __dsub_rn((double)B.c[b], f->lo[b]);
-            d = __dsub_rn(d, 0.5 * f->h[b]);
-            m = __dadd_rn(m, __dmul_rn(R[b], d));
-        }
-        const double dlo = floor(__dmul_rn(__dsub_rn(m, half), s));
-        const double dhi = ceil(__dmul_rn(__dadd_rn(m, half), s));
-        if (!(fabs(dlo) < 4.0e18 && fabs(dhi) < 4.0e18)) bad = true;
-        else {
-            lo = (int64_t)dlo;
-            hi = (int64_t)dhi;
-        }
-    }
-    if (__any_sync(0xffffffffu, bad)) {   // an empty box, as k_quantize leaves it
+    const int e = lane < 9 ? lane : 0, a = e / 3, b = e - 3 * a, b1 = b == 2 ? 0 : b + 1, b2 = b == 0 ? 2 : b - 1;
+    double r = __dsub_rn(__dmul_rn((double)B.axis0[b1], (double)B.axis1[b2]),
+                         __dmul_rn((double)B.axis0[b2], (double)B.axis1[b1]));
+    if (a < 2) r = (double)(a == 0 ? B.axis0[b] : B.axis1[b]);
+    const int32_t n = normal_entry(r, f, b);
+    const double t = __dmul_rn(r, __dsub_rn(__dsub_rn((double)B.c[b], f->lo[b]), 0.5 * f->h[b]));
+    // lanes 0-5: bound lane & 1 of slab lane / 2
+    const int sl = lane < 6 ? lane >> 1 : 0;
+    double m = __shfl_sync(0xffffffffu, t, 3 * sl);
+    m = __dadd_rn(m, __shfl_sync(0xffffffffu, t, 3 * sl + 1));
+    m = __dadd_rn(m, __shfl_sync(0xffffffffu, t, 3 * sl + 2));
+    const float half = B.half[sl];
+    bad |= !(half >= 0.0f);
+    const double v = __dmul_rn(__dadd_rn(m, (double)((lane & 1) ? half : -half)), f->s32);
+    bad |= !(fabs(v) < 4.0e18);
+    int64_t bound = (lane & 1) ? __double2ll_ru(v) : __double2ll_rd(v);
+    const bool any = __any_sync(0xffffffffu, bad);   // an empty box then, as quantize_box leaves it
+    if (any) {
         if (lane == 0) atomicOr(err, kErrArg);
-        n = lane % 4 == 0 ? 1 : 0;
-        lo = 0;
-        hi = -1;
+        bound = -(lane & 1);
     }
-    if (lane < 9) out->n[lane] = n;
-    else if (lane < 12) {
-        out->b[2 * a] = lo;
-        out->b[2 * a + 1] = hi;
-    } else if (lane == 12) {
-        out->reserved = 0;
-    }
+    if (lane < 9) out->n[lane] = any ? (lane % 4 == 0 ? 1 : 0) : n;
+    if (lane < 6) out->b[lane] = bound;
+    if (lane == 12) out->reserved = 0;
 }
 
 // A few boxes (at most kFewMaxBoxes) in one launch: a cluster of kFewCluster
@@ -781,8 +754,7 @@ obb_status quantize_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box* d
                           obb_qbox* d_out)
 {
     if (K <= 0) return OBB_OK;
-    k_quantize<<<(unsigned)((K + 31) / 32), 32, 0, ctx->stream>>>(d_boxes, K, lat->d_frame, d_out,
-                                                                    ctx->d_err);
+    k_quantize<<<(unsigned)((K + 31) / 32), 32, 0, ctx->stream>>>(d_boxes, K, lat->d_frame, d_out, ctx->d_err);
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
     return OBB_OK;
@@ -869,9 +841,8 @@ obb_status count_float_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box
     if (few_boxes(ctx, K, (int64_t)lat->n_words * 8))
         return launch_few(ctx, lat->d_ref, 1, nullptr, nullptr, d_boxes, lat->d_frame, nullptr, K, d_counts, d_points,
                           ctx->d_prof + 2);
-    OBB_CK(ctx, ctx->qscratch.reserve(sizeof(obb_qbox) * K, ctx->stream));
-    OBB_TRY(quantize_boxes(ctx, lat, d_boxes, K, ctx->qscratch.as<obb_qbox>()));
-    return count_known(ctx, lat, ctx->qscratch.as<obb_qbox>(), K, d_counts, d_points);
+    return count_boxes_multi(ctx, lat->d_ref, 1, nullptr, nullptr, nullptr, K, d_counts, d_points,
+                             (int64_t)lat->n_words * 8, d_boxes, lat->d_frame);
 }
 
 obb_status count_known(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* d_boxes, int64_t K, uint64_t* d_counts,
@@ -898,14 +869,15 @@ obb_status count_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* d_b
 
 obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats, const int32_t* d_lat_of_box,
                              const obb_qbox* d_boxes, const int32_t* d_K, int64_t K_cap, uint64_t* d_counts,
-                             uint64_t* d_points, int64_t lattice_bytes)
+                             uint64_t* d_points, int64_t lattice_bytes, const obb_box* d_fboxes,
+                             const LatticeFrame* d_frame)
 {
     cudaStream_t s = ctx->stream;
     if (K_cap <= 0) return OBB_OK;
     if (K_cap > (int64_t(1) << 30)) return fail(ctx, OBB_ERR_RANGE, "too many boxes in one call");
     if (few_boxes(ctx, K_cap, lattice_bytes))
-        return launch_few(ctx, d_lats, n_lats, d_lat_of_box, d_boxes, nullptr, nullptr, d_K, K_cap, d_counts, d_points,
-                          ctx->d_prof + 2);
+        return launch_few(ctx, d_lats, n_lats, d_lat_of_box, d_boxes, d_fboxes, d_frame, d_K, K_cap, d_counts,
+                          d_points, ctx->d_prof + 2);
     BoxPrep* prep;
     int64_t *tiles, *off;
     unsigned int* ticket = ctx->d_ticket;
@@ -940,31 +912,30 @@ obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
         }
     }
     const bool scan = !perm && K_cap <= kPrepScanBoxes;
-    if (!d_K && !scan) {   // the other kernels read the count from the device
-        OBB_CK(ctx, ctx->kdev.reserve(sizeof(int32_t), s));
-        OBB_TRY(set_device_int(ctx, ctx->kdev.as<int32_t>(), (int32_t)K_cap));
-        d_K = ctx->kdev.as<int32_t>();
-    }
     // the preparation kernel also zeroes counts and points (accumulated with atomics)
-    k_prep<<<(unsigned)((K_cap + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
-        d_boxes, d_K, (int32_t)K_cap, d_lats, n_lats, d_lat_of_box,
-        CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank}, count_grid_warps(ctx), prep, tiles, off,
-        reinterpret_cast<unsigned long long*>(d_counts), reinterpret_cast<unsigned long long*>(d_points), ticket,
-        bucket, bucket ? ctx->d_order_hist : nullptr, scan ? 1 : 0, ctx->d_err);
+    const auto run_prep = [&](auto kernel) {
+        kernel<<<(unsigned)((K_cap + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
+            d_boxes, d_fboxes, d_frame, d_K, (int32_t)K_cap, d_lats, n_lats, d_lat_of_box,
+            CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank}, count_grid_warps(ctx), prep, tiles, off,
+            reinterpret_cast<unsigned long long*>(d_counts), reinterpret_cast<unsigned long long*>(d_points), ticket,
+            bucket, bucket ? ctx->d_order_hist : nullptr, scan ? 1 : 0, ctx->d_err);
+    };
+    if (d_fboxes) run_prep(k_prep<true>);
+    else run_prep(k_prep<false>);
     note_launch(ctx);
     // tile offsets (unless the preparation's last block has scanned them): an exclusive scan of the tile counts in counting order
     // (the spatial order's permuted copy, else the boxes' own order)
     const int64_t* scan_in = tiles;
     if (perm) {
-        k_order_scatter<<<(unsigned)((K_cap + 255) / 256), 256, 0, s>>>(bucket, tiles, d_K, ctx->d_order_hist, perm,
-                                                                      ptiles);
+        k_order_scatter<<<(unsigned)((K_cap + 255) / 256), 256, 0, s>>>(bucket, tiles, d_K, (int32_t)K_cap,
+                                                                        ctx->d_order_hist, perm, ptiles);
         note_launch(ctx);
         scan_in = ptiles;
     }
     if (!scan) {
         const unsigned nsb = (unsigned)(K_cap / kScanBlock + 1);
-        k_tile_sums<<<nsb, 256, 0, s>>>(scan_in, d_K, bsum);
-        k_tile_offsets<<<nsb, 256, 0, s>>>(scan_in, bsum, d_K, off);
+        k_tile_sums<<<nsb, 256, 0, s>>>(scan_in, d_K, (int32_t)K_cap, bsum);
+        k_tile_offsets<<<nsb, 256, 0, s>>>(scan_in, bsum, d_K, (int32_t)K_cap, off);
         note_launch(ctx, 2);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1126,8 +1097,8 @@ extern "C" obb_status obb_outer_volume_q_noalloc(obb_ctx* ctx, const obb_lattice
     // (zero at load; every launch leaves it at zero again)
     unsigned int* ticket = reinterpret_cast<unsigned int*>(base + kNoAllocOffsetK + 128);
     // the preparation kernel also zeroes counts and points (accumulated with atomics)
-    k_prep<<<(unsigned)((K + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
-        d_boxes, nullptr, (int32_t)K, lat->d_ref, 1, nullptr,
+    k_prep<false><<<(unsigned)((K + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
+        d_boxes, nullptr, nullptr, nullptr, (int32_t)K, lat->d_ref, 1, nullptr,
         CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank}, count_grid_warps(ctx), prep, chunks, off,
         reinterpret_cast<unsigned long long*>(d_counts), reinterpret_cast<unsigned long long*>(d_points), ticket,
         nullptr, nullptr, 1, ctx->d_err);

@@ -251,7 +251,7 @@ void obb_destroy(obb_ctx* ctx)
 {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->stream);
-    DevBuf* bufs[] = {&ctx->prep, &ctx->chunk_off, &ctx->qscratch, &ctx->cscratch, &ctx->pscratch, &ctx->kdev,
+    DevBuf* bufs[] = {&ctx->prep, &ctx->chunk_off, &ctx->cscratch, &ctx->pscratch, &ctx->kdev,
                       &ctx->tmp_a, &ctx->tmp_b, &ctx->tmp_c, &ctx->tmp_d, &ctx->cub_tmp, &ctx->order};
     for (DevBuf* b : bufs) b->release(ctx->stream);
     cudaStreamSynchronize(ctx->stream);
@@ -583,9 +583,7 @@ obb_status obb_outer_volume_multi(obb_ctx* ctx, const obb_lattice* const* lats, 
     uint64_t *dc, *dp;
     OBB_TRY(out_device(ctx, counts, (size_t)K, on_device, hc, &dc));
     OBB_TRY(out_device(ctx, points, (size_t)K, on_device, hp, &dp));
-    OBB_CK(ctx, ctx->kdev.reserve(sizeof(int32_t), ctx->stream));
-    OBB_TRY(set_device_int(ctx, ctx->kdev.as<int32_t>(), (int32_t)K));
-    OBB_TRY(count_boxes_multi(ctx, dt, n_lats, dl, db, ctx->kdev.as<int32_t>(), K, dc, dp, lattice_bytes));
+    OBB_TRY(count_boxes_multi(ctx, dt, n_lats, dl, db, nullptr, K, dc, dp, lattice_bytes));
     OBB_TRY(copy_back(ctx, counts, dc, (size_t)K, on_device));
     OBB_TRY(copy_back(ctx, points, dp, (size_t)K, on_device));
     // the lattice table lives in a temporary: wait before it is released
