@@ -1351,34 +1351,164 @@ __device__ void jacobi3(const double c6[6], double R[9])
     R[8] = R[0] * R[4] - R[1] * R[3];
 }
 
+__device__ __forceinline__ void put_normals(const double* R, const LatticeFrame* __restrict__ f, obb_qbox* q)
+{
+    for (int i = 0; i < 9; ++i) q->n[i] = normal_entry(R[i], f, i % 3);
+    q->reserved = 0;
+}
+
+// Frames of clusters from their moments, and the frames' integer normals:
+// n_ab = rint(2^24 ((R_ab h_b) / h_max)), each step correctly rounded
+// (normal_entry).  A thread a cluster.
 __global__ void k_frames_from_moments(const double* __restrict__ mom, const double* __restrict__ fallback,
-                                      int32_t K, double* __restrict__ out, const uint8_t* __restrict__ dirty)
+                                      int32_t K, double* __restrict__ out, const LatticeFrame* __restrict__ f,
+                                      obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty)
 {
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K || (dirty && !dirty[k])) return;
     const double* m = mom + 10 * (int64_t)k;
-    double* R = out + 9 * (int64_t)k;
+    double R[9];
     const double A = m[0];
     if (!(A > 0.0)) {
         for (int i = 0; i < 9; ++i) R[i] = fallback ? fallback[9 * (int64_t)k + i] : (i % 4 == 0 ? 1.0 : 0.0);
-        return;
+    } else {
+        const double mu[3] = {m[1] / A, m[2] / A, m[3] / A};
+        const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
+        double c6[6];
+        for (int q = 0; q < 6; ++q) c6[q] = m[4 + q] / A - mu[ia[q]] * mu[ib[q]];
+        jacobi3(c6, R);
     }
-    const double mu[3] = {m[1] / A, m[2] / A, m[3] / A};
-    const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
-    double c6[6];
-    for (int q = 0; q < 6; ++q) c6[q] = m[4 + q] / A - mu[ia[q]] * mu[ib[q]];
-    jacobi3(c6, R);
+    for (int i = 0; i < 9; ++i) out[9 * (int64_t)k + i] = R[i];
+    put_normals(R, f, q + k);
 }
 
-// n_ab = rint(2^24 ((R_ab h_b) / h_max)), each step correctly rounded (normal_entry)
+// The same, bit for bit, by eight lanes a cluster: the loops over rows and the
+// divisions by A run on a lane each.  An FP64 instruction costs a warp 64
+// cycles whatever its lanes, so a cluster's chain shortens with its
+// instructions as long as every scheduler has a warp or two.  Lanes 0-2 hold
+// the rows of the covariance, 3-5 those of the eigenvectors; the products and
+// sums are fused as the compiler fuses jacobi3's.
+constexpr int kFrameLanes = 8;
+__global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ mom,
+                                                     const double* __restrict__ fallback, int32_t K,
+                                                     double* __restrict__ out, const LatticeFrame* __restrict__ f,
+                                                     obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, r = lane & (kFrameLanes - 1), g0 = lane - r;
+    const int32_t k = (blockIdx.x * 32 + lane) / kFrameLanes;
+    const bool on = k < K && !(dirty && !dirty[k]);
+    if (!__any_sync(kAll, on)) return;
+    const double* m = mom + 10 * (int64_t)(on ? k : 0);
+    const double A = on ? m[0] : 0.0;
+    const bool solve = A > 0.0;
+    auto get = [&](double x, int from) { return __shfl_sync(kAll, x, g0 + from); };
+    // lanes 0-5: an entry of the covariance (xx, yy, zz, xy, xz, yz)
+    const double mu = (solve ? m[1 + min(r, 2)] : 0.0) / (solve ? A : 1.0);
+    const int ia = r == 5 ? 1 : r > 2 ? 0 : r, ib = r == 3 ? 1 : r > 3 ? 2 : r;
+    const double mx = get(mu, ia), my = get(mu, min(ib, 2));
+    const double c = (solve ? m[4 + min(r, 5)] : 0.0) / (solve ? A : 1.0) - mx * my;
+    double M[3];
+    {
+        const double xx = get(c, 0), yy = get(c, 1), zz = get(c, 2), xy = get(c, 3), xz = get(c, 4), yz = get(c, 5);
+        M[0] = r == 0 ? xx : r == 1 ? xy : r == 2 ? xz : r == 3 ? 1.0 : 0.0;
+        M[1] = r == 0 ? xy : r == 1 ? yy : r == 2 ? yz : r == 4 ? 1.0 : 0.0;
+        M[2] = r == 0 ? xz : r == 1 ? yz : r == 2 ? zz : r == 5 ? 1.0 : 0.0;
+    }
+    double fro = 0.0;
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) {
+            const double x = get(M[j], i);
+            fro += x * x;
+        }
+    for (int sweep = 0; sweep < 16; ++sweep) {
+        const double a01 = get(M[1], 0), a02 = get(M[2], 0), a12 = get(M[2], 1);
+        const double off = 2.0 * (a01 * a01 + a02 * a02 + a12 * a12);
+        const bool go = solve && !(off <= 1e-30 * fro);
+        if (!__any_sync(kAll, go)) break;
+#pragma unroll
+        for (int rot = 0; rot < 3; ++rot) {
+            const int p = rot == 2 ? 1 : 0, qq = rot == 0 ? 1 : 2;
+            const double apq = get(M[qq], p), app = get(M[p], p), aqq = get(M[qq], qq);
+            const bool turn = go && apq != 0.0;
+            const double theta = (aqq - app) / (2.0 * apq);
+            const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+            const double cs = 1.0 / sqrt(t * t + 1.0);
+            const double sn = t * cs;
+            // columns p and q of the lane's row
+            const double x = M[p], y = M[qq];
+            const double xn = __fma_rn(cs, x, -__dmul_rn(sn, y)), yn = __fma_rn(sn, x, __dmul_rn(cs, y));
+            if (turn) {
+                M[p] = xn;
+                M[qq] = yn;
+            }
+            // rows p and q of the covariance: the two lanes exchange theirs
+            const int other = r == p ? qq : r == qq ? p : r;
+            double o[3];
+            for (int j = 0; j < 3; ++j) o[j] = get(M[j], other);
+            // row p: c row_p - s row_q; row q: s row_p + c row_q
+            for (int j = 0; j < 3; ++j) {
+                const double rp = r == p ? M[j] : o[j], rq = r == p ? o[j] : M[j];
+                const double u = r == p ? cs : sn, w = r == p ? -sn : cs;
+                const double v = __fma_rn(u, rp, __dmul_rn(w, rq));
+                if (turn && (r == p || r == qq)) M[j] = v;
+            }
+        }
+    }
+    const double ev[3] = {get(M[0], 0), get(M[1], 1), get(M[2], 2)};
+    int o[3] = {0, 1, 2};
+    for (int i = 0; i < 3; ++i)
+        for (int j = i + 1; j < 3; ++j)
+            if ((o[j] == 0 ? ev[0] : o[j] == 1 ? ev[1] : ev[2]) > (o[i] == 0 ? ev[0] : o[i] == 1 ? ev[1] : ev[2])) {
+                const int tmp = o[i];
+                o[i] = o[j];
+                o[j] = tmp;
+            }
+    double R[9];
+    for (int a = 0; a < 2; ++a) {
+        const double mine = o[a] == 0 ? M[0] : o[a] == 1 ? M[1] : M[2];
+        double row[3];
+        for (int b = 0; b < 3; ++b) row[b] = get(mine, 3 + b);
+        double big = row[0];
+        for (int b = 1; b < 3; ++b)
+            if (fabs(row[b]) > fabs(big)) big = row[b];
+        for (int b = 0; b < 3; ++b) R[3 * a + b] = big < 0.0 ? -row[b] : row[b];
+    }
+    R[6] = R[1] * R[5] - R[2] * R[4];
+    R[7] = R[2] * R[3] - R[0] * R[5];
+    R[8] = R[0] * R[4] - R[1] * R[3];
+    if (!on) return;
+    for (int i = r; i < 9; i += kFrameLanes) {
+        double x = R[0];
+#pragma unroll
+        for (int j = 1; j < 9; ++j)
+            if (i == j) x = R[j];
+        if (!solve) x = fallback ? fallback[9 * (int64_t)k + i] : (i % 4 == 0 ? 1.0 : 0.0);
+        out[9 * (int64_t)k + i] = x;
+        q[k].n[i] = normal_entry(x, f, i % 3);
+    }
+    if (r == 0) q[k].reserved = 0;
+}
+
+// integer normals of given frames
 __global__ void k_normals(const double* __restrict__ frames, int32_t K, const LatticeFrame* __restrict__ f,
-                          obb_qbox* __restrict__ q, const uint8_t* __restrict__ active)
+                          obb_qbox* __restrict__ q)
 {
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K || (active && !active[k])) return;
-    for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) q[k].n[3 * a + b] = normal_entry(frames[9 * (int64_t)k + 3 * a + b], f, b);
-    q[k].reserved = 0;
+    if (k < K) put_normals(frames + 9 * (int64_t)k, f, q + k);
+}
+
+static void launch_frames(obb_ctx* ctx, const double* mom, const double* fallback, int32_t K, double* frames,
+                          const LatticeFrame* f, obb_qbox* q, const uint8_t* dirty)
+{
+    // eight lanes a cluster against a thread: 18.0 against 24.4 us for 64 clusters, 25.8 against 33.1 for 1,024, 26.8
+    // against 33.3 for 2,048; from 3,072 on (33.4, 33.3) a scheduler has several of the lanes' warps and falls behind
+    // (16,384: 141 against 36)
+    if (K <= 2048)
+        k_frames_lanes<<<(K * kFrameLanes + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty);
+    else
+        k_frames_from_moments<<<(K + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty);
+    note_launch(ctx);
 }
 
 template <int NT>
@@ -1629,28 +1759,42 @@ constexpr int kProbes = 6;
 constexpr int kDescentMaxLevel = 8;
 
 __global__ void k_probe_frames(const double* __restrict__ frames, const int32_t* __restrict__ level, int32_t K,
-                               double* __restrict__ pf, uint8_t* __restrict__ active)
+                               double* __restrict__ pf, uint8_t* __restrict__ active,
+                               const LatticeFrame* __restrict__ f, obb_qbox* __restrict__ pq)
 {
+    // the levels' rotations, by the first warp
+    __shared__ double tc[kDescentMaxLevel], ts[kDescentMaxLevel];
+    if (threadIdx.x < kDescentMaxLevel) {
+        const double t = ldexp(1.0, -(5 + (int)threadIdx.x));
+        const double t2 = __dmul_rn(t, t);
+        const double den = __dadd_rn(1.0, t2);
+        tc[threadIdx.x] = __ddiv_rn(__dsub_rn(1.0, t2), den);
+        ts[threadIdx.x] = __ddiv_rn(__dmul_rn(2.0, t), den);
+    }
+    __syncthreads();
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= K * kProbes) return;
     const int32_t k = i / kProbes, p = i % kProbes;
-    const bool on = level[k] < kDescentMaxLevel;
+    const int32_t lev = level[k];
+    const bool on = lev < kDescentMaxLevel;
     active[i] = on;
     if (!on) return;
-    const double t = ldexp(1.0, -(5 + level[k]));
-    const double t2 = __dmul_rn(t, t);
-    const double den = __dadd_rn(1.0, t2);
-    const double c = __ddiv_rn(__dsub_rn(1.0, t2), den);
-    const double sn = __ddiv_rn(__dmul_rn(2.0, t), den);
+    const double c = tc[lev], sn = ts[lev];
     const double ss = (p & 1) ? -sn : sn;
     const int a = p >> 1, b1 = (a + 1) % 3, b2 = (a + 2) % 3;
     const double* R = frames + 9 * (int64_t)k;
     double* O = pf + 9 * (int64_t)i;
+    obb_qbox* q = pq + i;
+    auto put = [&](int a, int j, double x) {
+        O[3 * a + j] = x;
+        q->n[3 * a + j] = normal_entry(x, f, j);
+    };
     for (int j = 0; j < 3; ++j) {
-        O[3 * a + j] = R[3 * a + j];
-        O[3 * b1 + j] = __dadd_rn(__dmul_rn(c, R[3 * b1 + j]), __dmul_rn(ss, R[3 * b2 + j]));
-        O[3 * b2 + j] = __dsub_rn(__dmul_rn(c, R[3 * b2 + j]), __dmul_rn(ss, R[3 * b1 + j]));
+        put(a, j, R[3 * a + j]);
+        put(b1, j, __dadd_rn(__dmul_rn(c, R[3 * b1 + j]), __dmul_rn(ss, R[3 * b2 + j])));
+        put(b2, j, __dsub_rn(__dmul_rn(c, R[3 * b2 + j]), __dmul_rn(ss, R[3 * b1 + j])));
     }
+    q->reserved = 0;
 }
 
 // surrogate screen of the probes: keep the m lowest predicted outer volumes of each cluster
@@ -1884,15 +2028,14 @@ static obb_status init_boxes(obb_ctx* ctx, obb_layer* L, const double* d_frames,
     const int K = L->K;
     if (d_frames) {
         OBB_CK(ctx, cudaMemcpyAsync(L->d_frames, d_frames, sizeof(double) * 9 * K, cudaMemcpyDeviceToDevice, s));
+        k_normals<<<(K + 31) / 32, 32, 0, s>>>(L->d_frames, K, lat->d_frame, L->d_q);
+        note_launch(ctx);
     } else {
         k_moments<kNT><<<K, kNT, 0, s>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start,
                                          lat->d_frame, M->mom, nullptr);
         note_launch(ctx);
-        k_frames_from_moments<<<(K + 31) / 32, 32, 0, s>>>(M->mom, d_fallback, K, L->d_frames, nullptr);
-        note_launch(ctx);
+        launch_frames(ctx, M->mom, d_fallback, K, L->d_frames, lat->d_frame, L->d_q, nullptr);
     }
-    k_normals<<<(K + 31) / 32, 32, 0, s>>>(L->d_frames, K, lat->d_frame, L->d_q, nullptr);
-    note_launch(ctx);
     launch_tight(ctx, L, L->d_q, 1, nullptr, s);
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
@@ -2387,10 +2530,9 @@ static obb_status refit_covariance(obb_ctx* ctx, obb_layer* L, int phase)
         if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
         k_moments<kNT><<<K, kNT, 0, s>>>(mesh->d_verts, mesh->d_tris, L->d_members, L->d_start, lat->d_frame,
                                          M->mom, M->dirty);
-        k_frames_from_moments<<<(K + 31) / 32, 32, 0, s>>>(M->mom, L->d_frames, K, M->newframe, M->dirty);
-        k_normals<<<(K + 31) / 32, 32, 0, s>>>(M->newframe, K, lat->d_frame, M->newq, M->dirty);
+        launch_frames(ctx, M->mom, L->d_frames, K, M->newframe, lat->d_frame, M->newq, M->dirty);
         launch_tight(ctx, L, M->newq, 1, M->dirty, s);
-        note_launch(ctx, 4);
+        note_launch(ctx, 2);
         const uint8_t* screen = nullptr;
         if (L->mlp) {
             // surrogate screen: exact counts only for the boxes predicted to improve
@@ -2432,10 +2574,10 @@ obb_status layer_box_update(obb_ctx* ctx, obb_layer* L, int refit_mode, int dste
         if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
         const int32_t KP = kProbes * K;
         for (int step = 0; step < dsteps; ++step) {
-            k_probe_frames<<<(KP + 127) / 128, 128, 0, s>>>(L->d_frames, M->level, K, M->pframes, M->keep);
-            k_normals<<<(KP + 31) / 32, 32, 0, s>>>(M->pframes, KP, lat->d_frame, M->pq, M->keep);
+            k_probe_frames<<<(KP + 127) / 128, 128, 0, s>>>(L->d_frames, M->level, K, M->pframes, M->keep, lat->d_frame,
+                                                            M->pq);
             launch_tight(ctx, L, M->pq, kProbes, M->keep, s);
-            note_launch(ctx, 3);
+            note_launch(ctx, 2);
             if (L->mlp) {
                 OBB_CK(ctx, ctx->kdev.reserve(sizeof(int32_t), s));
                 OBB_TRY(set_device_int(ctx, ctx->kdev.as<int32_t>(), KP));
