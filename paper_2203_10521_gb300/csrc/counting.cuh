@@ -95,6 +95,25 @@ __device__ __forceinline__ int choose_axis(const obb_qbox& q)
     return best;
 }
 
+// floor(x / d) and its remainder in [0, d), for 0 < d <= 2^24 and |x| < 2^62,
+// by the integer reciprocal M = floor((2^64 - 1) / d): the high half of y M
+// is at most one below floor(y / d) (M d > 2^64 - d - 1, y < 2^63), so one
+// correction makes it exact.  All integer: 64-bit int <-> float conversions
+// issue on the FP64 pipe, a small fraction of the integer rate on this GPU.
+__device__ __forceinline__ void floordiv_rcp(int64_t x, int32_t d, uint64_t M, int64_t& q, int32_t& r)
+{
+    const bool neg = x < 0;
+    const uint64_t y = neg ? (uint64_t)(-x) + (uint64_t)(d - 1) : (uint64_t)x;   // x < 0: floor(x/d) = -floor(y/d)
+    uint64_t qq = __umul64hi(y, M);
+    uint64_t rr = y - qq * (uint64_t)d;
+    if (rr >= (uint64_t)d) {
+        rr -= (uint64_t)d;
+        ++qq;
+    }
+    q = neg ? -(int64_t)qq : (int64_t)qq;
+    r = neg ? d - 1 - (int32_t)rr : (int32_t)rr;
+}
+
 // How a launch's boxes are counted: rows per lane per tile, row axis mode,
 // rank rows on or off.
 struct CountOpts {
@@ -146,6 +165,8 @@ __device__ __noinline__ int64_t prep_box(const obb_qbox& qin, int32_t li, const 
         empty |= p.Lq[a] > p.Hq[a];
         const int32_t d = p.n[3 * a];
         p.dd[a] = d >= 0 ? d : -d;
+        p.qw[a] = 0;
+        p.rw[a] = 0;
         p.qstep[a] = 0;
         p.rstep[a] = 0;
         p.fmul[a] = 0;
@@ -360,6 +381,7 @@ __device__ __noinline__ int64_t prep_box(const obb_qbox& qin, int32_t li, const 
             uint64_t fr = (uint64_t)rs * (uint32_t)(M >> 32) + __umulhi(rs, (uint32_t)M);
             if ((fr + 1) * (uint64_t)p.dd[a] <= ((uint64_t)rs << 32)) ++fr;
             p.fstep[a] = (int64_t)qs * 4294967296LL + (int64_t)fr;
+            floordiv_rcp(p.Hq[a] - p.Lq[a] - p.dd[a] + 1, p.dd[a], M, p.qw[a], p.rw[a]);
         }
     // A quotient saturated at +-2^30 must stay outside [0, span] for a whole
     // tile: its tk - 1 steps of at most |qstep| + 1 each stay below 2^29.  With
@@ -391,25 +413,6 @@ __device__ __forceinline__ int64_t fixed_frac(int32_t r, uint64_t M)   // 0 <= r
 {
     const uint32_t ru = (uint32_t)r;
     return (int64_t)((uint64_t)ru * (uint32_t)(M >> 32) + __umulhi(ru, (uint32_t)M));
-}
-
-// floor(x / d) and its remainder in [0, d), for 0 < d <= 2^24 and |x| < 2^62,
-// by the integer reciprocal M = floor((2^64 - 1) / d): the high half of y M
-// is at most one below floor(y / d) (M d > 2^64 - d - 1, y < 2^63), so one
-// correction makes it exact.  All integer: 64-bit int <-> float conversions
-// issue on the FP64 pipe, a small fraction of the integer rate on this GPU.
-__device__ __forceinline__ void floordiv_rcp(int64_t x, int32_t d, uint64_t M, int64_t& q, int32_t& r)
-{
-    const bool neg = x < 0;
-    const uint64_t y = neg ? (uint64_t)(-x) + (uint64_t)(d - 1) : (uint64_t)x;   // x < 0: floor(x/d) = -floor(y/d)
-    uint64_t qq = __umul64hi(y, M);
-    uint64_t rr = y - qq * (uint64_t)d;
-    if (rr >= (uint64_t)d) {
-        rr -= (uint64_t)d;
-        ++qq;
-    }
-    q = neg ? -(int64_t)qq : (int64_t)qq;
-    r = neg ? d - 1 - (int32_t)rr : (int32_t)rr;
 }
 
 // Intersect [lo, hi] with { i : L <= d i + c <= H } exactly (d != 0), by
@@ -449,6 +452,12 @@ __device__ __forceinline__ uint32_t popc_range(const uint64_t* __restrict__ row,
     return cnt + __popcll(first & mlo) + __popcll(last & (one ? 0ull : mhi));
 }
 
+// bits of the end words up to e, less those before a (mod 2^32)
+__device__ __forceinline__ uint32_t rank_bits(uint64_t first, uint64_t last, int32_t a, int32_t e)
+{
+    return (uint32_t)__popcll(last << (~e & 63)) - (uint32_t)__popcll(first & ~(~0ull << (a & 63)));
+}
+
 // The same count through the row's rank table (rk[w ws] = occupied bits in
 // words 0..w-1): the bits before e + 1 minus the bits before a, each a rank
 // entry plus the popcount of its word below the bit -- four loads whatever
@@ -460,8 +469,14 @@ __device__ __forceinline__ uint32_t popc_rank(const uint64_t* __restrict__ row, 
     const uint64_t first = __ldg(row + wa * ws);
     const uint64_t last = __ldg(row + we * ws);
     const uint32_t ra = __ldg(rk + wa * ws), rb = __ldg(rk + we * ws);
-    return rb - ra + (uint32_t)__popcll(last & (~0ull >> (63 - (e & 63)))) -
-           (uint32_t)__popcll(first & ~(~0ull << (a & 63)));
+    return rb - ra + rank_bits(first, last, a, e);
+}
+
+// occupied bits of [a, e] from its two end words, when it has no others: the
+// bits from a on and those up to e (shifts, no masks); in one word, less all
+__device__ __forceinline__ uint32_t short_bits(uint64_t first, uint64_t last, int32_t a, int32_t e)
+{
+    return __popcll(first >> (a & 63)) + __popcll(last << (~e & 63)) - ((a ^ e) < 64 ? __popcll(first) : 0);
 }
 
 // occupied bits of [a, e] when it lies within two consecutive words
@@ -470,11 +485,7 @@ __device__ __forceinline__ uint32_t popc_short(const uint64_t* __restrict__ row,
     const int32_t wa = a >> 6, we = e >> 6;
     const uint64_t first = __ldg(row + wa * ws);
     const uint64_t last = __ldg(row + we * ws);
-    uint64_t mlo = ~0ull << (a & 63);
-    const uint64_t mhi = ~0ull >> (63 - (e & 63));
-    const bool one = wa == we;
-    mlo = one ? (mlo & mhi) : mlo;
-    return __popcll(first & mlo) + __popcll(last & (one ? 0ull : mhi));
+    return short_bits(first, last, a, e);
 }
 
 // Row counting modes of a box (BoxPrep::rank).
@@ -500,50 +511,94 @@ __device__ __forceinline__ uint32_t popc_mode(const uint64_t* __restrict__ row, 
     else return popc_range(row, ws, a, e);
 }
 
+// The first row's interval of a lane, relative to i0, from the six bounds of
+// the DDA; the bounds step to the next row.
+__device__ __forceinline__ void dda_step(int64_t (&Al)[3], int64_t (&Ah)[3], const int64_t (&Bs)[3], int32_t span,
+                                         int32_t& lo, int32_t& hi)
+{
+    lo = max(max((int32_t)(Al[0] >> 32), (int32_t)(Al[1] >> 32)), max((int32_t)(Al[2] >> 32), 0));
+    hi = min(min((int32_t)(Ah[0] >> 32), (int32_t)(Ah[1] >> 32)), min((int32_t)(Ah[2] >> 32), span));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        Al[a] += Bs[a];
+        Ah[a] += Bs[a];
+    }
+}
+
 // One pass of a lane over its rows r0..r1 of a tile of a box whose three
 // slabs all step by DDA: each of the six bounds is a 32.32 fixed-point value
 // whose integer part is the quotient, so a bound costs one 64-bit add per
-// row.  kMode: how a row's occupied bits are counted; kInterior: the tile's
-// rows and x-intervals all lie in the lattice (no clamps); kProf: algorithmic
-// bytes and rows are added up.
+// row.  The loop is bound by issue slots, most of them integer ones: a row's
+// place is a 32-bit offset (at, mod 2^32: rows outside the lattice are not
+// read, and the largest copy has 2^27 words) and the bits are counted by
+// shifts where a mask can be saved.  32,767 tree boxes at 1024^3: 257 us, 285
+// with 64-bit row pointers, masks, two divisions a slab and the in-domain
+// points of interior rows added up twice.
+//
+// dda_interior: rows whose words are the two at their ends (kMode kRowRank or
+// kRowShort) of a tile that lies in the lattice with all of its x-intervals
+// (an idle lane's span is -1).  A row's words are counted a row later, behind
+// the next row's bounds (261 -> 257 us).
+template <int kMode, bool kProf>
+__device__ __forceinline__ void dda_interior(int64_t (&Al)[3], int64_t (&Ah)[3], const int64_t (&Bs)[3],
+                                             const uint64_t* __restrict__ words, const uint16_t* __restrict__ ranks,
+                                             uint32_t at, uint32_t rstride, int32_t rows, int32_t i0, int32_t span,
+                                             int32_t N, uint32_t& empty, uint32_t& inbox, uint32_t& my_bytes,
+                                             uint32_t& my_rows, uint32_t& my_rank, uint32_t& my_dom)
+{
+    uint32_t in = 0, occ = 0, rk = 0;
+    uint64_t first = 0, last = 0;
+    int32_t a = 0, e = 0;
+    const auto take = [&] {
+        occ += kMode == kRowRank ? rk + rank_bits(first, last, a, e) : short_bits(first, last, a, e);
+    };
+    for (int32_t r = 0; r < rows; ++r, at += rstride) {
+        int32_t lo, hi;
+        dda_step(Al, Ah, Bs, span, lo, hi);
+        take();
+        first = last = 0;
+        rk = 0;
+        if (lo <= hi) {
+            a = i0 + lo;
+            e = i0 + hi;
+            in += (uint32_t)(hi - lo + 1);
+            const uint32_t pa = at + (a >> 6) * N, pe = at + (e >> 6) * N;
+            first = __ldg(words + pa);
+            last = __ldg(words + pe);
+            if (kMode == kRowRank) rk = (uint32_t)__ldg(ranks + pe) - (uint32_t)__ldg(ranks + pa);
+            if (kProf) {
+                my_bytes += row_bytes<kMode>(a, e);
+                my_rows += 1;
+                my_rank += kMode == kRowRank ? 1u : 0u;
+            }
+        }
+    }
+    take();
+    inbox += in;
+    empty += in - occ;
+    my_dom += in;
+}
+
+// dda_rows: any other tile.  kInterior: as above, with words between the ends.
 template <int kMode, bool kInterior, bool kProf>
 __device__ __forceinline__ void dda_rows(int64_t (&Al)[3], int64_t (&Ah)[3], const int64_t (&Bs)[3],
-                                         const uint64_t* __restrict__ rowp, const uint16_t* __restrict__ rkp,
-                                         int64_t rstride, int32_t r0, int32_t r1, int32_t k, int32_t wk, int32_t kend,
-                                         bool jvalid, bool jin, int32_t i0, int32_t span, int32_t N,
+                                         const uint64_t* __restrict__ words, const uint16_t* __restrict__ ranks,
+                                         uint32_t at, uint32_t rstride, int32_t rows, int32_t k, int32_t wk,
+                                         int32_t kend, bool jvalid, bool jin, int32_t i0, int32_t span, int32_t N,
                                          uint32_t& empty, uint32_t& inbox, uint32_t& my_bytes, uint32_t& my_rows,
                                          uint32_t& my_rank, uint32_t& my_dom)
 {
-    const int32_t spanl = kInterior ? (jvalid ? span : -1) : span;
 #pragma unroll kCountUnroll
-    for (int r = r0; r <= r1; ++r, k += wk, rowp += rstride, rkp += rstride) {
-        const int32_t lo = max(max((int32_t)(Al[0] >> 32), (int32_t)(Al[1] >> 32)), max((int32_t)(Al[2] >> 32), 0));
-        const int32_t hi = min(min((int32_t)(Ah[0] >> 32), (int32_t)(Ah[1] >> 32)), min((int32_t)(Ah[2] >> 32), spanl));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            Al[a] += Bs[a];
-            Ah[a] += Bs[a];
-        }
-        if (kInterior) {
-            if (lo <= hi) {
-                const int32_t a = i0 + lo, e = i0 + hi;
-                const uint32_t len = (uint32_t)(hi - lo + 1);
-                empty += len - popc_mode<kMode>(rowp, rkp, N, a, e);
-                inbox += len;
-                my_dom += len;
-                if (kProf) {
-                    my_bytes += row_bytes<kMode>(a, e);
-                    my_rows += 1;
-                    my_rank += kMode == kRowRank ? 1u : 0u;
-                }
-            }
-        } else if (jvalid && k < kend && lo <= hi) {
+    for (int32_t r = 0; r < rows; ++r, k += wk, at += rstride) {
+        int32_t lo, hi;
+        dda_step(Al, Ah, Bs, span, lo, hi);
+        if (kInterior ? lo <= hi : jvalid && k < kend && lo <= hi) {
             const uint32_t len = (uint32_t)(hi - lo + 1);
             uint32_t occ = 0;
-            if (jin && (uint32_t)k < (uint32_t)N) {
-                const int32_t a = max(i0 + lo, 0), e = min(i0 + hi, N - 1);
-                if (a <= e) {
-                    occ = popc_mode<kMode>(rowp, rkp, N, a, e);
+            if (kInterior || (jin && (uint32_t)k < (uint32_t)N)) {
+                const int32_t a = kInterior ? i0 + lo : max(i0 + lo, 0), e = kInterior ? i0 + hi : min(i0 + hi, N - 1);
+                if (kInterior || a <= e) {
+                    occ = popc_mode<kMode>(words + at, ranks + at, N, a, e);
                     my_dom += (uint32_t)(e - a + 1);
                     if (kProf) my_bytes += row_bytes<kMode>(a, e);
                 }
@@ -639,10 +694,15 @@ __device__ __forceinline__ bool count_tile(const BoxPrep& p, int32_t tj, int32_t
             qs[a] = p.qstep[a];
             const int64_t cc = (int64_t)p.n[3 * a + 1] * j + (int64_t)p.n[3 * a + 2] * kb0;
             const int64_t xlo = p.n[3 * a] > 0 ? p.Lq[a] - cc : cc - p.Hq[a];
-            const int64_t xhi = p.n[3 * a] > 0 ? p.Hq[a] - cc : cc - p.Lq[a];
-            int64_t wlo, whi;
+            int64_t wlo;
             floordiv_rcp(xlo + dd[a] - 1, dd[a], p.fmul[a], wlo, ra[a]);   // ceil(xlo / dd)
-            floordiv_rcp(xhi, dd[a], p.fmul[a], whi, rb[a]);               // floor(xhi / dd)
+            // the upper bound floor(xhi / dd): xhi = (xlo + dd - 1) + (H - L - dd + 1)
+            int64_t whi = wlo + p.qw[a];
+            rb[a] = ra[a] + p.rw[a];
+            if (rb[a] >= dd[a]) {
+                rb[a] -= dd[a];
+                ++whi;
+            }
             const int64_t lim = int64_t(1) << 30;
             qa[a] = (int32_t)min(max(wlo - i0, -lim), lim);
             qb[a] = (int32_t)min(max(whi - i0, -lim), lim);
@@ -662,24 +722,30 @@ __device__ __forceinline__ bool count_tile(const BoxPrep& p, int32_t tj, int32_t
         }
         // count copies interleave the rows of a slice by column: word w of
         // row (slice k, column j) at (k W + w) N + j
-        const int64_t roff = (int64_t)kb0 * W * N + j;
-        const int64_t rstride = (int64_t)wk * W * N;
+        const uint32_t at = (uint32_t)kb0 * (uint32_t)(W * N) + (uint32_t)j;
+        const uint32_t rstride = (uint32_t)wk * (uint32_t)(W * N);
+        const int32_t rows = r1 - r0 + 1;
         // an interior box's full-height tile: every row is in the lattice
         // and so is every x-interval; an idle lane gets an empty range
         const bool interior = (mode & 0x100) && (tk + 1) * wk * tkr <= p.nk;
-#define OBB_DDA_ROWS(MODE, INTERIOR)                                                                             \
-dda_rows<MODE, INTERIOR, kProf>(Al, Ah, Bs, words + roff, p.ranks + roff, rstride, r0, r1, kb0, wk, kend, jvalid, \
-                                jin, i0, span, N, empty, inbox, my_bytes, my_rows, my_rank, my_dom)
+        const int32_t spanl = jvalid ? span : -1;
+#define OBB_DDA_INTERIOR(MODE)                                                                                       \
+dda_interior<MODE, kProf>(Al, Ah, Bs, words, p.ranks, at, rstride, rows, i0, spanl, N, empty, inbox, my_bytes, my_rows, \
+                          my_rank, my_dom)
+#define OBB_DDA_ROWS(MODE, INTERIOR)                                                                               \
+dda_rows<MODE, INTERIOR, kProf>(Al, Ah, Bs, words, p.ranks, at, rstride, rows, kb0, wk, kend, jvalid, jin, i0,       \
+                                INTERIOR ? spanl : span, N, empty, inbox, my_bytes, my_rows, my_rank, my_dom)
         if (p.rank == kRowRank) {
-            if (interior) OBB_DDA_ROWS(kRowRank, true);
+            if (interior) OBB_DDA_INTERIOR(kRowRank);
             else OBB_DDA_ROWS(kRowRank, false);
         } else if (p.rank == kRowShort) {
-            if (interior) OBB_DDA_ROWS(kRowShort, true);
+            if (interior) OBB_DDA_INTERIOR(kRowShort);
             else OBB_DDA_ROWS(kRowShort, false);
         } else {
             if (interior) OBB_DDA_ROWS(kRowWalk, true);
             else OBB_DDA_ROWS(kRowWalk, false);
         }
+#undef OBB_DDA_INTERIOR
 #undef OBB_DDA_ROWS
     } else
 #pragma unroll kCountUnroll

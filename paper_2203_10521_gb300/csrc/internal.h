@@ -112,6 +112,8 @@ struct alignas(128) BoxPrep {
     // ... by the exact seeds of a tile's first row
     int64_t Lq[3], Hq[3];    // ceil(lo / 256), floor(hi / 256)
     uint64_t fmul[3];        // floor((2^64 - 1) / dd): remainder -> 32-bit fraction
+    int64_t qw[3];           // quotient and remainder of H - L - dd + 1 by dd: from a slab's lower bound to its upper
+    int32_t rw[3];
     int64_t fstep[3];        // floor(step * 2^32), step = qstep + rstep / dd (32.32 fixed point)
     // ... and by the general row loop only
     int32_t rstep[3];        // remainder of that step, in [0, dd)

@@ -537,10 +537,8 @@ __global__ void __launch_bounds__(256, kMinB) k_count(const BoxPrep* __restrict_
             ++c;
             continue;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            empty += __shfl_xor_sync(0xffffffffu, empty, o);
-            inbox += __shfl_xor_sync(0xffffffffu, inbox, o);
-        }
+        empty = __reduce_add_sync(0xffffffffu, empty);
+        inbox = __reduce_add_sync(0xffffffffu, inbox);
         if (lane == 0) {
             if (empty) atomicAdd(&counts[bi], (unsigned long long)empty);
             if (points && inbox) atomicAdd(&points[bi], (unsigned long long)inbox);
