@@ -680,8 +680,11 @@ __global__ void __launch_bounds__(kRunThreads) k_fl_run(
         cluster.sync();
         const int ne = *ne_at;
         if (ne < 0) break;
-        if (warp < ne && lane == 0)
-            tiles[warp] = prep_box(ev_at[warp], 0, lats, 1, o, max(1, kWarps * C / ne), &prep[warp], err);
+        if (warp < ne) {
+            const int64_t nt = prep_box(lane < 4 ? &ev_at[warp] : nullptr, 0, lats, 1, o, max(1, kWarps * C / ne),
+                                        &prep[warp], err);
+            if (lane == 0) tiles[warp] = nt;
+        }
         __syncthreads();
         // the boxes' tiles one after another, dealt out over the cluster's warps
         int64_t t = warp * C + rank;

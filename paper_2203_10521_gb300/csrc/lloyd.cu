@@ -815,7 +815,7 @@ __global__ void k_sum_points(const uint64_t* __restrict__ pts, const int32_t* __
 // launches and a round trip to the host each, all pairs in every round: three
 // iterations of 200k triangles in 1,024 clusters 3.3 ms a call, this way 1.3;
 // six with rotation descent of 2M in 16,384 clusters 13.9 and 11.1 ms.
-constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each
+constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each (prepared by three warps, eight each)
 constexpr int kPairMoves = 64;      // most rounds of a step that take this path
 constexpr int kPairGraphMin = 64;   // pairs of a layer whose captured iteration takes it (the launch counter of a small
                                     // captured layer is read per round)
@@ -979,8 +979,12 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
         }
         sync();
         const int ne = ctl0->ne;
-        if (warp == 0 && lane < ne)
-            tiles[lane] = prep_box(ev0[lane], 0, p.lats, 1, p.o, max(1, kWarps * C / max(ne, 1)), &prep[lane], p.err);
+        if (8 * warp < ne) {   // eight boxes a warp
+            const int e = 8 * warp + (lane >> 2);
+            const int64_t nt = prep_box(e < ne ? &ev0[e] : nullptr, 0, p.lats, 1, p.o, max(1, kWarps * C / ne),
+                                        &prep[min(e, kPairEvals - 1)], p.err);
+            if (e < ne && (lane & 3) == 0) tiles[e] = nt;
+        }
         __syncthreads();
         // the boxes' tiles one after another, dealt out over the warps
         int64_t at = warp * C + rank;

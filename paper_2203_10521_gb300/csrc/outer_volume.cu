@@ -56,7 +56,8 @@
 namespace obbv {
 constexpr int64_t kOrderMinBoxes = OBB_ORDER_MIN_BOXES;
 constexpr int64_t kOrderMinLatticeBytes = int64_t(OBB_ORDER_MIN_MB) << 20;
-constexpr int kPrepThreads = 32;   // one warp per preparation block: its per-box work spreads over many SMs
+constexpr int kPrepThreads = 128;   // four lanes prepare a box (prep_box)
+constexpr int kPrepBoxes = kPrepThreads / 4;
 constexpr int kGrab = OBB_GRAB;   // tiles per work grab
 }  // namespace obbv
 
@@ -122,7 +123,7 @@ __global__ void k_quantize(const obb_box* __restrict__ boxes, int64_t K, const L
 // against 68.8).
 constexpr int32_t kShortTileBoxes = 128;
 
-// One box per thread (prep_box), counts zeroed on the way; then the last
+// Four lanes a box (prep_box), counts zeroed on the way; then the last
 // block to finish (an atomic ticket, nothing waits) turns the tile counts into
 // offsets: off[0..K] exclusive, off[K + 1] = 0 (the counting kernel's work
 // counter).  kFloat: float boxes, quantised on the way (32,752 boxes at 1024^3:
@@ -144,14 +145,27 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(const obb_qbox* __restric
                                                        uint32_t* __restrict__ bucket, unsigned int* __restrict__ hist,
                                                        int32_t scan_tiles, int32_t* err)
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    static_assert(kPrepBoxes == 32, "a warp quantises the block's boxes");
+    const int64_t k = blockIdx.x * (int64_t)kPrepBoxes + (threadIdx.x >> 2);
     const int32_t K = d_K ? *d_K : K_val;
+    __shared__ obb_qbox sq[kFloat ? kPrepBoxes : 1];
+    if (kFloat) {
+        const int64_t f = blockIdx.x * (int64_t)kPrepBoxes + threadIdx.x;
+        if (threadIdx.x < 32 && f < K) sq[threadIdx.x] = quantize_box(fboxes[f], frame, err);
+        __syncthreads();
+    }
     // warps of the counting grid per box, when there are few boxes
     const int32_t warps = K > 0 && K <= kShortTileBoxes ? grid_warps / K : 0;
-    if (k < K) {
+    const bool on = k < K;
+    int64_t nt = 0;
+    if (__any_sync(0xffffffffu, on))
+        nt = prep_box(!on ? nullptr : kFloat ? &sq[threadIdx.x >> 2] : boxes + k, on && lat_of_box ? lat_of_box[k] : 0,
+                      lats, n_lats, o, warps, on ? &prep[k] : nullptr, err);
+    __syncwarp();   // the box's preparation is its four lanes' work
+    if (on && (threadIdx.x & 3) == 0) {
         counts[k] = 0;
         if (points) points[k] = 0;
-        tiles[k] = prep_box(kFloat ? quantize_box(fboxes[k], frame, err) : boxes[k], lat_of_box ? lat_of_box[k] : 0, lats, n_lats, o, warps, &prep[k], err);
+        tiles[k] = nt;
         if (bucket) {
             // spatial order: the 16^3 Morton cell of the centre of the box's
             // index-space rectangle (clamped to the lattice)
@@ -188,7 +202,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep(const obb_qbox* __restric
         if (last) __threadfence();
     }
     __syncthreads();
-    if (!last) return;
+    if (!last || threadIdx.x >= 32) return;
     if (bucket) {
         // spatial order: the bucket counts become bucket starts (exclusive
         // scan, one warp, 128 buckets a lane); k_order_scatter,
@@ -658,9 +672,9 @@ __global__ void __launch_bounds__(kFewThreads) k_count_few(const obb_qbox* __res
             quantize_warp(fboxes[k], frame, &q, err);
             __syncwarp();
         }
-        if (lane == 0)
-            s_tiles = prep_box(fboxes ? q : boxes[k], lat_of_box ? lat_of_box[k] : 0, lats, n_lats, o, kWarps * C, &p,
-                               err);
+        const int64_t nt = prep_box(lane >= 4 ? nullptr : fboxes ? &q : boxes + k, lat_of_box ? lat_of_box[k] : 0, lats,
+                                    n_lats, o, kWarps * C, &p, err);
+        if (lane == 0) s_tiles = nt;
     }
     __syncthreads();
     unsigned long long v[3] = {0, 0, 0};
@@ -912,7 +926,7 @@ obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
     const bool scan = !perm && K_cap <= kPrepScanBoxes;
     // the preparation kernel also zeroes counts and points (accumulated with atomics)
     const auto run_prep = [&](auto kernel) {
-        kernel<<<(unsigned)((K_cap + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
+        kernel<<<(unsigned)((K_cap + kPrepBoxes - 1) / kPrepBoxes), kPrepThreads, 0, s>>>(
             d_boxes, d_fboxes, d_frame, d_K, (int32_t)K_cap, d_lats, n_lats, d_lat_of_box,
             CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank}, count_grid_warps(ctx), prep, tiles, off,
             reinterpret_cast<unsigned long long*>(d_counts), reinterpret_cast<unsigned long long*>(d_points), ticket,
@@ -1095,7 +1109,7 @@ extern "C" obb_status obb_outer_volume_q_noalloc(obb_ctx* ctx, const obb_lattice
     // (zero at load; every launch leaves it at zero again)
     unsigned int* ticket = reinterpret_cast<unsigned int*>(base + kNoAllocOffsetK + 128);
     // the preparation kernel also zeroes counts and points (accumulated with atomics)
-    k_prep<false><<<(unsigned)((K + kPrepThreads - 1) / kPrepThreads), kPrepThreads, 0, s>>>(
+    k_prep<false><<<(unsigned)((K + kPrepBoxes - 1) / kPrepBoxes), kPrepThreads, 0, s>>>(
         d_boxes, nullptr, nullptr, nullptr, (int32_t)K, lat->d_ref, 1, nullptr,
         CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank}, count_grid_warps(ctx), prep, chunks, off,
         reinterpret_cast<unsigned long long*>(d_counts), reinterpret_cast<unsigned long long*>(d_points), ticket,

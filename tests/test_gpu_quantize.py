@@ -97,3 +97,21 @@ def test_float_boxes_count_as_quantised_ones(ctx, lat, K):
     c = ctx.outer_volume_q(L, ctx.quantize_boxes(L, b), want_points=True)
     for x, y in zip(a, c):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("K", [2, 9, 33, 600])
+@pytest.mark.parametrize("every", [1, 2, 3, 8])
+def test_empty_boxes_among_others(ctx, lat, K, every):
+    """Boxes without a point, axis-aligned ones and rotated ones prepared by one warp."""
+    L, verts = lat
+    b = boxes_of(np.random.default_rng(K + every), K, verts)
+    b[::every, 9:] = 0.0                                       # no lattice point inside, unless by chance
+    b[1::5, 3:9] = np.r_[1.0, 0, 0, 0, 1, 0]
+    q = ctx.quantize_boxes(L, b)
+    got = ctx.outer_volume(L, b, want_points=True)
+    again = ctx.outer_volume_q(L, q, want_points=True)
+    one = [ctx.outer_volume_q(L, q[k:k + 1], want_points=True) for k in range(min(K, 40))]
+    for i in range(2):
+        assert np.array_equal(got[i], again[i])
+        assert np.array_equal(got[i][:len(one)], np.concatenate([o[i] for o in one]))
+    assert np.all(got[0][::every] <= 8)
