@@ -391,16 +391,17 @@ obb_status batch_create(obb_ctx* ctx, obb_layer* const* layers, int32_t n, obb_b
 void batch_destroy(obb_batch* B);
 obb_status batch_lloyd_step(obb_ctx* ctx, obb_batch* B, const obb_step_opts* opts, obb_step_stats* stats);
 // pieces of the Lloyd step that the step between levels (sweep.cu) reuses
-enum { kStProposals = 0, kStAccepted, kStGain, kStEvals, kStRefits, kStPoints, kStRounds, kStCount };
+enum { kStProposals = 0, kStAccepted, kStGain, kStEvals, kStRefits, kStPoints, kStRounds, kStCount,
+       kStTotal = kStCount, kStErr, kStWords };   // read with them: total outer volume, the error word
 obb_status layer_box_update(obb_ctx* ctx, obb_layer* L, int refit_mode, int dsteps);
 obb_status layer_finish_stats(obb_ctx* ctx, obb_layer* L, int ran, obb_step_stats* st);
+obb_status read_stats(obb_ctx* ctx, const int64_t* d_stats, int64_t* h);
 uint8_t* layer_dirty(obb_layer* L);      // [K] membership changed since the last covariance refit
 int32_t* layer_level(obb_layer* L);      // [K] rotation-descent level
 const int32_t* layer_dev_K(obb_layer* L);   // device copy of K
 obb_status layer_members(obb_ctx* ctx, obb_layer* L);   // member lists valid on return
 void layer_members_changed(obb_layer* L);
 void layer_parents_changed(obb_layer* L);
-void launch_sum_points(obb_ctx* ctx, const uint64_t* d_pts, const int32_t* d_n, int64_t* d_stats);
 
 // surrogate.cu: features of boxes [0, *d_K) and predicted outer volumes (FP16 weights)
 obb_status surrogate_predict(obb_ctx* ctx, const obb_mlp* mlp, const obb_lattice* lat, const obb_qbox* d_boxes,

@@ -1364,12 +1364,14 @@ __device__ __forceinline__ void put_normals(const double* R, const LatticeFrame*
 
 // Frames of clusters from their moments, and the frames' integer normals:
 // n_ab = rint(2^24 ((R_ab h_b) / h_max)), each step correctly rounded
-// (normal_entry).  A thread a cluster.
+// (normal_entry).  A thread a cluster.  zero: a counter the next launches need at zero.
 __global__ void k_frames_from_moments(const double* __restrict__ mom, const double* __restrict__ fallback,
                                       int32_t K, double* __restrict__ out, const LatticeFrame* __restrict__ f,
-                                      obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty)
+                                      obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty,
+                                      int32_t* __restrict__ zero)
 {
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (zero && k == 0) *zero = 0;
     if (k >= K || (dirty && !dirty[k])) return;
     const double* m = mom + 10 * (int64_t)k;
     double R[9];
@@ -1397,9 +1399,11 @@ constexpr int kFrameLanes = 8;
 __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ mom,
                                                      const double* __restrict__ fallback, int32_t K,
                                                      double* __restrict__ out, const LatticeFrame* __restrict__ f,
-                                                     obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty)
+                                                     obb_qbox* __restrict__ q, const uint8_t* __restrict__ dirty,
+                                                     int32_t* __restrict__ zero)
 {
     constexpr unsigned kAll = 0xffffffffu;
+    if (zero && blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;
     const int lane = threadIdx.x & 31, r = lane & (kFrameLanes - 1), g0 = lane - r;
     const int32_t k = (blockIdx.x * 32 + lane) / kFrameLanes;
     const bool on = k < K && !(dirty && !dirty[k]);
@@ -1504,15 +1508,15 @@ __global__ void k_normals(const double* __restrict__ frames, int32_t K, const La
 }
 
 static void launch_frames(obb_ctx* ctx, const double* mom, const double* fallback, int32_t K, double* frames,
-                          const LatticeFrame* f, obb_qbox* q, const uint8_t* dirty)
+                          const LatticeFrame* f, obb_qbox* q, const uint8_t* dirty, int32_t* zero)
 {
     // eight lanes a cluster against a thread: 18.0 against 24.4 us for 64 clusters, 25.8 against 33.1 for 1,024, 26.8
     // against 33.3 for 2,048; from 3,072 on (33.4, 33.3) a scheduler has several of the lanes' warps and falls behind
     // (16,384: 141 against 36)
     if (K <= 2048)
-        k_frames_lanes<<<(K * kFrameLanes + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty);
+        k_frames_lanes<<<(K * kFrameLanes + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty, zero);
     else
-        k_frames_from_moments<<<(K + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty);
+        k_frames_from_moments<<<(K + 31) / 32, 32, 0, ctx->stream>>>(mom, fallback, K, frames, f, q, dirty, zero);
     note_launch(ctx);
 }
 
@@ -1613,7 +1617,9 @@ void launch_tight(obb_ctx* ctx, const obb_layer* L, obb_qbox* q, int32_t per_clu
                                           active);
 }
 
-__global__ void k_total(const uint64_t* __restrict__ obv, int32_t K, int64_t* __restrict__ out)
+// *out = total outer volume; err: the error word behind it, for the same copy
+__global__ void k_total(const uint64_t* __restrict__ obv, int32_t K, int64_t* __restrict__ out,
+                        const int32_t* __restrict__ err)
 {
     unsigned long long s = 0;
     for (int32_t i = threadIdx.x; i < K; i += blockDim.x) s += obv[i];
@@ -1624,7 +1630,8 @@ __global__ void k_total(const uint64_t* __restrict__ obv, int32_t K, int64_t* __
     if (threadIdx.x == 0) {
         unsigned long long t = 0;
         for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += sh[i];
-        *out = (int64_t)t;
+        out[0] = (int64_t)t;
+        if (err) out[1] = *err;
     }
 }
 
@@ -1717,20 +1724,34 @@ __global__ void k_screen_compact(Cand* __restrict__ cand, const int32_t* __restr
 }
 
 __global__ void k_refit_accept_mapped(const double* __restrict__ newframe, const obb_qbox* __restrict__ newq,
-                                      const uint64_t* __restrict__ cnt, const int32_t* __restrict__ map,
-                                      const int32_t* __restrict__ n2, double* __restrict__ frames,
-                                      obb_qbox* __restrict__ q, uint64_t* __restrict__ obv,
+                                      const uint64_t* __restrict__ cnt, const uint64_t* __restrict__ pts,
+                                      const int32_t* __restrict__ map, const int32_t* __restrict__ n2, int32_t K,
+                                      double* __restrict__ frames, obb_qbox* __restrict__ q,
+                                      uint64_t* __restrict__ obv, uint8_t* __restrict__ dirty,
                                       int64_t* __restrict__ stats)
 {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= *n2) return;
-    const int32_t k = map[i];
-    if (cnt[i] < obv[k]) {
-        for (int t = 0; t < 9; ++t) frames[9 * (int64_t)k + t] = newframe[9 * (int64_t)k + t];
-        q[k] = newq[k];
-        obv[k] = cnt[i];
-        atomicAdd((unsigned long long*)&stats[kStRefits], 1ull);
+    const int32_t n = *n2;
+    unsigned long long points = 0;
+    bool kept = false;
+    if (i < K) dirty[i] = 0;
+    if (i < n) {
+        const int32_t k = map[i];
+        points = pts[i];
+        kept = cnt[i] < obv[k];
+        if (kept) {
+            for (int t = 0; t < 9; ++t) frames[9 * (int64_t)k + t] = newframe[9 * (int64_t)k + t];
+            q[k] = newq[k];
+            obv[k] = cnt[i];
+        }
     }
+    for (int o = 16; o > 0; o >>= 1) points += __shfl_xor_sync(0xffffffffu, points, o);
+    const unsigned n_kept = __popc(__ballot_sync(0xffffffffu, kept));
+    if ((threadIdx.x & 31) == 0) {
+        if (points) atomicAdd((unsigned long long*)&stats[kStPoints], points);
+        if (n_kept) atomicAdd((unsigned long long*)&stats[kStRefits], (unsigned long long)n_kept);
+    }
+    if (i == 0) atomicAdd((unsigned long long*)&stats[kStEvals], (unsigned long long)n);
 }
 
 // clusters whose membership changed since their last covariance refit
@@ -2218,7 +2239,7 @@ static obb_status init_boxes(obb_ctx* ctx, obb_layer* L, const double* d_frames,
         k_moments<kNT><<<K, kNT, 0, s>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start,
                                          lat->d_frame, M->mom, nullptr);
         note_launch(ctx);
-        launch_frames(ctx, M->mom, d_fallback, K, L->d_frames, lat->d_frame, L->d_q, nullptr);
+        launch_frames(ctx, M->mom, d_fallback, K, L->d_frames, lat->d_frame, L->d_q, nullptr, nullptr);
     }
     launch_tight(ctx, L, L->d_q, 1, nullptr, s);
     note_launch(ctx);
@@ -2359,7 +2380,7 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     A_(dalloc(&L->d_members, T, s));
     A_(dalloc(&L->d_ext, K, s));
     A_(dalloc(&L->d_best, K, s));
-    A_(dalloc(&L->d_stats, kStCount, s));
+    A_(dalloc(&L->d_stats, kStWords, s));
     for (int p = 0; p + 1 < M->sort_passes; ++p) {
         A_(dalloc(&M->skeys[p], T, s));
         A_(dalloc(&M->svals[p], T, s));
@@ -2582,7 +2603,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
                 const int64_t l2 = ctx->launches;
                 rc = layer_box_update(ctx, L, refit_mode, dsteps);
                 if (rc != OBB_OK) return false;
-                k_total<<<1, 1024, 0, cs[0]>>>(L->d_obv, K, M->loop + 3);
+                k_total<<<1, 1024, 0, cs[0]>>>(L->d_obv, K, M->loop + 3, nullptr);
                 note_launch(ctx);
                 M->g_post = ctx->launches - l2;
                 if (!ck(cudaGetLastError())) return false;
@@ -2714,7 +2735,7 @@ static obb_status refit_covariance(obb_ctx* ctx, obb_layer* L, int phase)
         if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
         k_moments<kNT><<<K, kNT, 0, s>>>(mesh->d_verts, mesh->d_tris, L->d_members, L->d_start, lat->d_frame,
                                          M->mom, M->dirty);
-        launch_frames(ctx, M->mom, L->d_frames, K, M->newframe, lat->d_frame, M->newq, M->dirty);
+        launch_frames(ctx, M->mom, L->d_frames, K, M->newframe, lat->d_frame, M->newq, M->dirty, M->n2);
         launch_tight(ctx, L, M->newq, 1, M->dirty, s);
         note_launch(ctx, 2);
         const uint8_t* screen = nullptr;
@@ -2725,17 +2746,14 @@ static obb_status refit_covariance(obb_ctx* ctx, obb_layer* L, int phase)
             note_launch(ctx);
             screen = M->keep;
         }
-        OBB_CK(ctx, cudaMemsetAsync(M->n2, 0, sizeof(int32_t), s));
         k_dirty_compact<<<(K + 127) / 128, 128, 0, s>>>(M->dirty, screen, K, M->newq, M->evals2, M->map, M->n2);
         note_launch(ctx);
         OBB_TRY(count_boxes(ctx, lat, M->evals2, M->n2, K, M->ncount, M->epoints));
     }
     if (phase & kPost) {
-        k_sum_points<<<32, 256, 0, s>>>(M->epoints, M->n2, L->d_stats);
-        k_refit_accept_mapped<<<(K + 127) / 128, 128, 0, s>>>(M->newframe, M->newq, M->ncount, M->map, M->n2,
-                                                              L->d_frames, L->d_q, L->d_obv, L->d_stats);
-        note_launch(ctx, 2);
-        OBB_CK(ctx, cudaMemsetAsync(M->dirty, 0, K, s));
+        k_refit_accept_mapped<<<(K + 127) / 128, 128, 0, s>>>(M->newframe, M->newq, M->ncount, M->epoints, M->map, M->n2,
+                                                              K, L->d_frames, L->d_q, L->d_obv, M->dirty, L->d_stats);
+        note_launch(ctx);
     }
     OBB_CK(ctx, cudaGetLastError());
     return OBB_OK;
@@ -3212,18 +3230,25 @@ obb_status batch_lloyd_step(obb_ctx* ctx, obb_batch* B, const obb_step_opts* opt
 
 // Copies the layer's device counters and total outer volume into *st (if
 // non-null) after a step that ran `ran` partition rounds; synchronises.
+// Waits for a layer's counters (kStWords of them, the error word last, put
+// there by the kernel before); an error goes its usual way.
+obb_status read_stats(obb_ctx* ctx, const int64_t* d_stats, int64_t* h)
+{
+    OBB_CK(ctx, cudaMemcpyAsync(h, d_stats, sizeof(int64_t) * kStWords, cudaMemcpyDeviceToHost, ctx->stream));
+    OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
+    return h[kStErr] ? check_device_error(ctx) : OBB_OK;
+}
+
 obb_status layer_finish_stats(obb_ctx* ctx, obb_layer* L, int ran, obb_step_stats* st)
 {
     cudaStream_t s = ctx->stream;
     const int K = L->K;
     int64_t* h = host_stats(ctx);
     if (st) {
-        OBB_CK(ctx, ctx->tmp_d.reserve(sizeof(int64_t), s));
-        k_total<<<1, 1024, 0, s>>>(L->d_obv, K, ctx->tmp_d.as<int64_t>());
+        // counters, total and error word in one copy
+        k_total<<<1, 1024, 0, s>>>(L->d_obv, K, L->d_stats + kStTotal, ctx->d_err);
         note_launch(ctx);
-        OBB_CK(ctx, cudaMemcpyAsync(h, L->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
-        OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, ctx->tmp_d.p, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        OBB_TRY(check_device_error(ctx));
+        OBB_TRY(read_stats(ctx, L->d_stats, h));
         st->rounds_run = ran >= 0 ? ran : (int32_t)h[kStRounds];   // < 0: counted on the device
         st->refits_accepted = (int32_t)h[kStRefits];
         st->proposals = h[kStProposals];
@@ -3231,7 +3256,7 @@ obb_status layer_finish_stats(obb_ctx* ctx, obb_layer* L, int ran, obb_step_stat
         st->gain = h[kStGain];
         st->box_evals = h[kStEvals];
         st->points_counted = (uint64_t)h[kStPoints];
-        st->total_obv = (uint64_t)h[kStCount];
+        st->total_obv = (uint64_t)h[kStTotal];
     }
     return OBB_OK;
 }
@@ -3250,12 +3275,6 @@ void layer_members_changed(obb_layer* L)
 {
     mem_of(L)->members_valid = false;
     mem_of(L)->incr_ok = false;   // moved by something that keeps no move records
-}
-
-void launch_sum_points(obb_ctx* ctx, const uint64_t* d_pts, const int32_t* d_n, int64_t* d_stats)
-{
-    k_sum_points<<<32, 256, 0, ctx->stream>>>(d_pts, d_n, d_stats);
-    note_launch(ctx);
 }
 
 obb_status layer_set_surrogate(obb_ctx* ctx, obb_layer* L, const obb_mlp* mlp, int32_t topk)

@@ -61,10 +61,13 @@ __global__ void k_check_nesting(const int32_t* __restrict__ up_assign, const int
 }
 
 __global__ void k_unit_init(int32_t K, int64_t* __restrict__ m1, int64_t* __restrict__ m2,
-                            int32_t* __restrict__ cnt1, int32_t* __restrict__ usize)
+                            int32_t* __restrict__ cnt1, int32_t* __restrict__ usize,
+                            unsigned long long* __restrict__ best, int32_t* __restrict__ ctr)
 {
     int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kUCtrCount) ctr[k] = 0;
     if (k >= K) return;
+    best[k] = 0;
     for (int side = 0; side < 6; ++side) {
         const int64_t sent = (side & 1) ? INT64_MIN : INT64_MAX;
         m1[6 * (int64_t)k + side] = sent;
@@ -279,9 +282,20 @@ __global__ void k_unit_evals(const UnitScan* __restrict__ scan, const int32_t* _
 
 __global__ void k_unit_gains(UnitCand* __restrict__ cand, const int32_t* __restrict__ ctr,
                              const uint64_t* __restrict__ obv, const uint64_t* __restrict__ ecount,
-                             unsigned long long* __restrict__ best, int64_t* __restrict__ stats)
+                             const uint64_t* __restrict__ epoints, unsigned long long* __restrict__ best,
+                             int64_t* __restrict__ stats, const int32_t* __restrict__ err)
 {
     int32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    // the counters of the round's boxes, and the error word behind them
+    const int32_t ne = ctr[kUCtrEval];
+    unsigned long long points = 0;
+    for (int32_t i = r; i < ne; i += gridDim.x * blockDim.x) points += epoints[i];
+    for (int o = 16; o > 0; o >>= 1) points += __shfl_xor_sync(0xffffffffu, points, o);
+    if ((threadIdx.x & 31) == 0 && points) atomicAdd((unsigned long long*)&stats[kStPoints], points);
+    if (r == 0) {
+        atomicAdd((unsigned long long*)&stats[kStEvals], (unsigned long long)ne);
+        stats[kStErr] = *err;
+    }
     if (r >= ctr[kUCtrCand]) return;
     const UnitCand c = cand[r];
     const int64_t rem = (int64_t)obv[c.s] - (int64_t)ecount[c.e_shr];
@@ -397,27 +411,23 @@ obb_status unit_step(obb_ctx* ctx, obb_layer* up, obb_layer* low, const obb_step
     int ran = 0;
     int64_t before = 0;
     for (int r = 0; r < rounds; ++r) {
-        k_unit_init<<<(K + 127) / 128, 128, 0, s>>>(K, m1, m2, cnt1, usize);
+        k_unit_init<<<(K + 127) / 128, 128, 0, s>>>(K, m1, m2, cnt1, usize, up->d_best, ctr);
         k_unit_scan<<<Ku, kUT, 0, s>>>(lat->d_fixed, mesh->d_tris, mesh->d_adj, low->d_assign, low->d_members,
                                        low->d_start, low->d_parent, up->d_parent, up->d_q, usize, scan, ctx->d_err);
         k_unit_m1<<<gU, 128, 0, s>>>(scan, low->d_parent, Ku, m1);
         k_unit_m2<<<gU, 128, 0, s>>>(scan, low->d_parent, Ku, m1, m2, cnt1);
         note_launch(ctx, 4);
-        OBB_CK(ctx, cudaMemsetAsync(ctr, 0, sizeof(int32_t) * kUCtrCount, s));
-        OBB_CK(ctx, cudaMemsetAsync(up->d_best, 0, sizeof(unsigned long long) * K, s));
         k_unit_evals<<<gU, 128, 0, s>>>(scan, low->d_parent, Ku, usize, m1, m2, cnt1, up->d_q, cand, evals, ctr,
                                         cand_cap, eval_cap, ctx->d_err);
         note_launch(ctx);
         OBB_TRY(count_boxes(ctx, lat, evals, ctr + kUCtrEval, eval_cap, ecount, epoints));
-        launch_sum_points(ctx, epoints, ctr + kUCtrEval, up->d_stats);
         const unsigned cb = (unsigned)((cand_cap + 127) / 128);
-        k_unit_gains<<<cb, 128, 0, s>>>(cand, ctr, up->d_obv, ecount, up->d_best, up->d_stats);
+        k_unit_gains<<<cb, 128, 0, s>>>(cand, ctr, up->d_obv, ecount, epoints, up->d_best, up->d_stats, ctx->d_err);
         k_unit_accept<<<cb, 128, 0, s>>>(cand, ctr, up->d_best, evals, ecount, low->d_parent, up->d_q, up->d_obv,
                                          up->d_stats, layer_dirty(up), layer_level(up));
         note_launch(ctx, 2);
         OBB_CK(ctx, cudaGetLastError());
-        OBB_CK(ctx, cudaMemcpyAsync(h, up->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
-        OBB_TRY(check_device_error(ctx));
+        OBB_TRY(read_stats(ctx, up->d_stats, h));
         ++ran;
         const int64_t moved = h[kStAccepted] - before;
         before = h[kStAccepted];
