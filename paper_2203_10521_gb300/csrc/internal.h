@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstring>
 #include <functional>
 #include <map>
 #include <string>
@@ -177,6 +178,29 @@ struct BatchReq {
 // pool for the next allocation instead of going back to the driver at every
 // synchronisation).  Same contract as cudaMallocAsync; cudaFreeAsync frees.
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
+// Several arrays in one allocation, 256-byte aligned each: `add` them, then
+// `alloc`; freed as one (base).  An allocation and its release cost the host
+// about 1.3 us: 45 of a layer and ten of a unit step took 0.8 ms of a tree of
+// 511 boxes with one sweep.
+struct Slab {
+    std::vector<std::pair<void*, size_t>> parts;   // the pointer variable, its array's offset
+    size_t bytes = 0;
+    template <class T>
+    void add(T** p, size_t n)
+    {
+        parts.emplace_back(p, bytes);
+        bytes += (sizeof(T) * (n > 0 ? n : 1) + 255) / 256 * 256;
+    }
+    cudaError_t alloc(void** base, cudaStream_t s)
+    {
+        const cudaError_t e = pool_alloc(base, bytes, s);
+        for (const auto& p : parts) {
+            char* at = e == cudaSuccess ? static_cast<char*>(*base) + p.second : nullptr;
+            std::memcpy(p.first, &at, sizeof(at));
+        }
+        return e;
+    }
+};
 template <class T>
 inline cudaError_t pool_alloc(T** p, size_t bytes, cudaStream_t s)
 {

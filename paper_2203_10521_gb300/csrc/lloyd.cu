@@ -2102,6 +2102,7 @@ struct LayerMem {
     int64_t* loop = nullptr;          // [0] rounds run, [1] moves before the round, [2] rebuilds, [3] total
     CountScratch cscr{};              // the graph's own counting scratch (fixed addresses)
     void* cscr_mem = nullptr;
+    void* slab = nullptr;             // the arrays of the layer that are allocated with it
     int64_t g_round = 0, g_rebuild = 0, g_post = 0;   // kernel launches per round, per rebuild, after the loop
     bool members_valid = false;
     // sibling pairs (k_pair_rounds): 1 / 0 known, -1 to be looked at (parents may have changed)
@@ -2204,20 +2205,11 @@ void layer_destroy(obb_layer* L)
     if (!L) return;
     cudaStream_t s = L->ctx ? L->ctx->stream : nullptr;
     LayerMem* M = mem_of(L);
-    void* ptrs[] = {L->d_assign, L->d_parent, L->d_frames, L->d_q, L->d_obv, L->d_size, L->d_start,
-                    L->d_members, L->d_ext, L->d_best, L->d_stats};
-    for (void* p : ptrs)
-        if (p) cudaFreeAsync(p, s);
     if (M) {
         if (M->gexec) cudaGraphExecDestroy(M->gexec);
         if (M->loop) cudaFreeAsync(M->loop, s);
         if (M->cscr_mem) cudaFreeAsync(M->cscr_mem, s);
-        void* mp[] = {M->skeys[0], M->skeys[1], M->svals[0], M->svals[1], M->scnt, M->soff, M->sbsum, M->sticket, M->ctr, M->cand, M->evals, M->ecount, M->epoints, M->mom,
-                      M->newframe, M->newq, M->ncount, M->dK, M->feats, M->pred, M->skey,
-                      M->slot, M->evals2, M->n2, M->map, M->dirty, M->keep, M->level,
-                      M->pframes, M->pq, M->pbest, M->pcount, M->mv, M->mnew, M->snew, M->pinfo,
-                      M->dpaired};
-        for (void* p : mp)
+        for (void* p : {(void*)M->slab, (void*)M->feats, (void*)M->pred, (void*)M->skey, (void*)M->slot})
             if (p) cudaFreeAsync(p, s);
         delete M;
     }
@@ -2367,59 +2359,57 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     }
     const int64_t sort_tiles = (T + kSortTile - 1) / kSortTile;
     const int64_t sort_nc = ((int64_t)1 << M->sort_bits) * sort_tiles;
-    cudaError_t e = cudaSuccess;
-#define A_(x)                        \
-    if (e == cudaSuccess) e = (x);
-    A_(dalloc(&L->d_assign, T, s));
-    A_(dalloc(&L->d_parent, K, s));
-    A_(dalloc(&L->d_frames, 9 * (size_t)K, s));
-    A_(dalloc(&L->d_q, K, s));
-    A_(dalloc(&L->d_obv, K, s));
-    A_(dalloc(&L->d_size, K, s));
-    A_(dalloc(&L->d_start, (size_t)K + 1, s));
-    A_(dalloc(&L->d_members, T, s));
-    A_(dalloc(&L->d_ext, K, s));
-    A_(dalloc(&L->d_best, K, s));
-    A_(dalloc(&L->d_stats, kStWords, s));
+    Slab slab;
+    slab.add(&L->d_assign, T);
+    slab.add(&L->d_parent, K);
+    slab.add(&L->d_frames, 9 * (size_t)K);
+    slab.add(&L->d_q, K);
+    slab.add(&L->d_obv, K);
+    slab.add(&L->d_size, K);
+    slab.add(&L->d_start, (size_t)K + 1);
+    slab.add(&L->d_members, T);
+    slab.add(&L->d_ext, K);
+    slab.add(&L->d_best, K);
+    slab.add(&L->d_stats, kStWords);
     for (int p = 0; p + 1 < M->sort_passes; ++p) {
-        A_(dalloc(&M->skeys[p], T, s));
-        A_(dalloc(&M->svals[p], T, s));
+        slab.add(&M->skeys[p], T);
+        slab.add(&M->svals[p], T);
     }
-    A_(dalloc(&M->scnt, sort_nc, s));
-    A_(dalloc(&M->soff, sort_nc, s));
-    A_(dalloc(&M->sbsum, (sort_nc + kSortScanBlock - 1) / kSortScanBlock, s));
-    A_(dalloc(&M->sticket, 1, s));
+    slab.add(&M->scnt, sort_nc);
+    slab.add(&M->soff, sort_nc);
+    slab.add(&M->sbsum, (sort_nc + kSortScanBlock - 1) / kSortScanBlock);
+    slab.add(&M->sticket, 1);
+    slab.add(&M->ctr, kCtrCount);
+    slab.add(&M->cand, M->cand_cap);
+    slab.add(&M->evals, M->eval_cap);
+    slab.add(&M->ecount, M->eval_cap);
+    slab.add(&M->epoints, std::max<int64_t>(M->eval_cap, (int64_t)kProbes * K));
+    slab.add(&M->mom, 10 * (size_t)K);
+    slab.add(&M->newframe, 9 * (size_t)K);
+    slab.add(&M->newq, K);
+    slab.add(&M->ncount, K);
+    slab.add(&M->dK, 1);
+    const size_t cap2 = (size_t)std::max<int64_t>(M->eval_cap, (int64_t)kProbes * K);
+    slab.add(&M->evals2, cap2);
+    slab.add(&M->map, cap2);
+    slab.add(&M->n2, 1);
+    slab.add(&M->dirty, K);
+    slab.add(&M->keep, (size_t)kProbes * K);
+    slab.add(&M->level, K);
+    slab.add(&M->pframes, (size_t)9 * kProbes * K);
+    slab.add(&M->pq, (size_t)kProbes * K);
+    slab.add(&M->pbest, K);
+    slab.add(&M->pcount, (size_t)kProbes * K);
+    slab.add(&M->mv, 2 * (size_t)K);
+    slab.add(&M->mnew, T);
+    slab.add(&M->pinfo, (size_t)(K + 1) / 2);
+    slab.add(&M->dpaired, 1);
+    slab.add(&M->snew, (size_t)K + 1);
+    cudaError_t e = slab.alloc(&M->slab, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(M->sticket, 0, sizeof(unsigned int), s);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sort_scatter_smem(1 << kSortMaxBits));
-    A_(dalloc(&M->ctr, kCtrCount, s));
-    A_(dalloc(&M->cand, M->cand_cap, s));
-    A_(dalloc(&M->evals, M->eval_cap, s));
-    A_(dalloc(&M->ecount, M->eval_cap, s));
-    A_(dalloc(&M->epoints, std::max<int64_t>(M->eval_cap, (int64_t)kProbes * K), s));
-    A_(dalloc(&M->mom, 10 * (size_t)K, s));
-    A_(dalloc(&M->newframe, 9 * (size_t)K, s));
-    A_(dalloc(&M->newq, K, s));
-    A_(dalloc(&M->ncount, K, s));
-    A_(dalloc(&M->dK, 1, s));
-    const size_t cap2 = (size_t)std::max<int64_t>(M->eval_cap, (int64_t)kProbes * K);
-    A_(dalloc(&M->evals2, cap2, s));
-    A_(dalloc(&M->map, cap2, s));
-    A_(dalloc(&M->n2, 1, s));
-    A_(dalloc(&M->dirty, K, s));
-    A_(dalloc(&M->keep, (size_t)kProbes * K, s));
-    A_(dalloc(&M->level, K, s));
-    A_(dalloc(&M->pframes, (size_t)9 * kProbes * K, s));
-    A_(dalloc(&M->pq, (size_t)kProbes * K, s));
-    A_(dalloc(&M->pbest, K, s));
-    A_(dalloc(&M->pcount, (size_t)kProbes * K, s));
-    A_(dalloc(&M->mv, 2 * (size_t)K, s));
-    A_(dalloc(&M->mnew, T, s));
-    A_(dalloc(&M->pinfo, (size_t)(K + 1) / 2, s));
-    A_(dalloc(&M->dpaired, 1, s));
-    A_(dalloc(&M->snew, (size_t)K + 1, s));
-#undef A_
     if (e != cudaSuccess) {
         layer_destroy(L);
         return cuda_fail(ctx, e, "layer allocation");

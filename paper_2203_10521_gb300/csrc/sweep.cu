@@ -357,19 +357,10 @@ __global__ void k_unit_assign(const int32_t* __restrict__ low_assign, const int3
 // Scratch of one unit step, released when it returns.
 struct UnitMem {
     obb_ctx* ctx = nullptr;
-    std::vector<void*> ptrs;
-    cudaError_t e = cudaSuccess;
-    template <class T>
-    T* get(size_t n)
-    {
-        void* p = nullptr;
-        if (e == cudaSuccess) e = pool_alloc(&p, sizeof(T) * (n > 0 ? n : 1), ctx->stream);
-        if (e == cudaSuccess) ptrs.push_back(p);
-        return static_cast<T*>(p);
-    }
+    void* base = nullptr;
     ~UnitMem()
     {
-        for (void* p : ptrs) cudaFreeAsync(p, ctx->stream);
+        if (base) cudaFreeAsync(base, ctx->stream);
     }
 };
 
@@ -395,17 +386,24 @@ obb_status unit_step(obb_ctx* ctx, obb_layer* up, obb_layer* low, const obb_step
     UnitMem mem;
     mem.ctx = ctx;
     const int32_t cand_cap = Ku + 32, eval_cap = (1 + kMaxUnitCand) * cand_cap;
-    UnitScan* scan = mem.get<UnitScan>(Ku);
-    int64_t* m1 = mem.get<int64_t>(6 * (size_t)K);
-    int64_t* m2 = mem.get<int64_t>(6 * (size_t)K);
-    int32_t* cnt1 = mem.get<int32_t>(6 * (size_t)K);
-    int32_t* usize = mem.get<int32_t>(K);
-    UnitCand* cand = mem.get<UnitCand>(cand_cap);
-    obb_qbox* evals = mem.get<obb_qbox>(eval_cap);
-    uint64_t* ecount = mem.get<uint64_t>(eval_cap);
-    uint64_t* epoints = mem.get<uint64_t>(eval_cap);
-    int32_t* ctr = mem.get<int32_t>(kUCtrCount);
-    if (mem.e != cudaSuccess) return cuda_fail(ctx, mem.e, "unit step scratch");
+    UnitScan* scan;
+    int64_t *m1, *m2;
+    int32_t *cnt1, *usize, *ctr;
+    UnitCand* cand;
+    obb_qbox* evals;
+    uint64_t *ecount, *epoints;
+    Slab slab;
+    slab.add(&scan, Ku);
+    slab.add(&m1, 6 * (size_t)K);
+    slab.add(&m2, 6 * (size_t)K);
+    slab.add(&cnt1, 6 * (size_t)K);
+    slab.add(&usize, K);
+    slab.add(&cand, cand_cap);
+    slab.add(&evals, eval_cap);
+    slab.add(&ecount, eval_cap);
+    slab.add(&epoints, eval_cap);
+    slab.add(&ctr, kUCtrCount);
+    OBB_CK(ctx, slab.alloc(&mem.base, s));
     OBB_CK(ctx, cudaMemsetAsync(up->d_stats, 0, sizeof(int64_t) * kStCount, s));
     int64_t* h = host_stats(ctx);
     int ran = 0;
