@@ -848,14 +848,16 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
     constexpr int kWarps = NT / 32;
     __shared__ Top2 red[2][kWarps][6];
     __shared__ Top2 ext[2][6];
-    __shared__ obb_qbox box[2], ev[kPairEvals];
+    __shared__ obb_qbox box[2], ev[2][kPairEvals];                     // this round's boxes and the last one's
     __shared__ uint64_t obv[2];
     __shared__ BoxPrep prep[kPairEvals];
     __shared__ int64_t tiles[kPairEvals];
-    __shared__ unsigned long long sum[kPairEvals], pts[kPairEvals];
+    __shared__ unsigned long long sum[2][kPairEvals], pts[2][kPairEvals];
+    __shared__ int32_t todo[kPairEvals], slot[kPairEvals];             // those of this round that are counted; a copy
     __shared__ PairMove moved[kPairMoves], mv[kPairMoves];   // the first block's, this block's copy
     struct Control {
         int32_t ne, n_moved, need, go;   // boxes to count; moves so far; clusters whose extents change (bits); another round
+        int32_t cur;                     // which of the two box lists is this round's
         int32_t size[2];
     };
     __shared__ Control ctl, cc;          // the first block's, this block's copy
@@ -872,20 +874,22 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
         obv[tid] = p.obv[k0 + tid];
     }
     if (tid == 0) {
-        ctl = Control{0, 0, 3, 1, {m0 - A, B - m0}};
+        ctl = Control{0, 0, 3, 1, 0, {m0 - A, B - m0}};
         cc = ctl;
     }
     __syncthreads();
     const Control* ctl0 = cluster.map_shared_rank(&ctl, 0);
     const PairMove* moved0 = cluster.map_shared_rank(&moved[0], 0);
-    const obb_qbox* ev0 = cluster.map_shared_rank(&ev[0], 0);
-    unsigned long long* sum0 = cluster.map_shared_rank(&sum[0], 0);
-    unsigned long long* pts0 = cluster.map_shared_rank(&pts[0], 0);
+    const int32_t* todo0 = cluster.map_shared_rank(&todo[0], 0);
+    const obb_qbox* ev0 = cluster.map_shared_rank(&ev[0][0], 0);
+    unsigned long long* sum0 = cluster.map_shared_rank(&sum[0][0], 0);
+    unsigned long long* pts0 = cluster.map_shared_rank(&pts[0][0], 0);
     const bool lead = rank == 0 && warp == 0;   // the warp that chooses
     // of the first warp's lanes 0-11: candidate of cluster lane / 6, side lane % 6
     const int my_c = lane < 6 ? 0 : 1, my_side = lane < 6 ? lane : lane - 6;
     unsigned long long proposals = 0, accepted = 0, gain = 0, e_sum = 0, p_sum = 0, p_last = 0, n_dom = 0;
     int32_t e_last = 0, ran = 0;
+    int32_t old_s = -1, old_g = -1;      // places of this lane's boxes in the last round's list
     for (;;) {
         // extents of the clusters that lost a triangle (first round: both): the clusters' old segments without
         // the triangles that have left, then those that have joined
@@ -957,33 +961,67 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
             vm = __ballot_sync(0xffffffffu, cand);
             gm = __ballot_sync(0xffffffffu, grew);
             const unsigned below = (1u << lane) - 1u;
+            // A move changes the box of the cluster it leaves and often not the other one's: a candidate box that
+            // its lane had in the last round too keeps its count (10,000 triangles, depth 8, 16 steps of pair rounds:
+            // 3.32 -> 3.11 ms).
+            const int cur = ran & 1;
+            const int es = __popc(vm & below), eg = __popc(vm) + __popc(gm & below);
+            const auto as_before = [&](int e, int old) {
+                bool same = old >= 0;
+                for (int i = 0; i < 6 && same; ++i) same = ev[cur][e].b[i] == ev[cur ^ 1][old].b[i];
+                return same;
+            };
+            bool new_s = cand, new_g = grew;
+            if (lane < kPairEvals) {
+                sum[cur][lane] = 0;
+                pts[cur][lane] = 0;
+            }
+            __syncwarp();
             if (cand) {
-                obb_qbox& E = ev[__popc(vm & below)];
+                obb_qbox& E = ev[cur][es];
                 E = box[my_c];
                 for (int side = 0; side < 6; ++side)
                     if (ext[my_c][side].t1 == t && ext[my_c][side].v2 != ext[my_c][side].v1) E.b[side] = ext[my_c][side].v2;
+                if (as_before(es, old_s)) {
+                    new_s = false;
+                    sum[cur][es] = sum[cur ^ 1][old_s];
+                    pts[cur][es] = pts[cur ^ 1][old_s];
+                }
             }
             if (grew) {
-                obb_qbox& E = ev[__popc(vm) + __popc(gm & below)];
+                obb_qbox& E = ev[cur][eg];
                 E = box[1 - my_c];
                 for (int a = 0; a < 3; ++a) {
                     E.b[2 * a] = min(E.b[2 * a], dmin[a]);
                     E.b[2 * a + 1] = max(E.b[2 * a + 1], dmax[a]);
                 }
+                if (as_before(eg, old_g)) {
+                    new_g = false;
+                    sum[cur][eg] = sum[cur ^ 1][old_g];
+                    pts[cur][eg] = pts[cur ^ 1][old_g];
+                }
             }
-            if (lane < kPairEvals) {
-                sum[lane] = 0;
-                pts[lane] = 0;
+            old_s = cand ? es : -1;
+            old_g = grew ? eg : -1;
+            const unsigned ns = __ballot_sync(0xffffffffu, new_s), ng = __ballot_sync(0xffffffffu, new_g);
+            if (new_s) todo[__popc(ns & below)] = es;
+            if (new_g) todo[__popc(ns) + __popc(ng & below)] = eg;
+            if (lane == 0) {
+                ctl.ne = __popc(ns) + __popc(ng);
+                ctl.cur = cur;
             }
-            if (lane == 0) ctl.ne = __popc(vm) + __popc(gm);
         }
         sync();
-        const int ne = ctl0->ne;
+        const int ne = ctl0->ne, base = ctl0->cur * kPairEvals;
         if (8 * warp < ne) {   // eight boxes a warp
             const int e = 8 * warp + (lane >> 2);
-            const int64_t nt = prep_box(e < ne ? &ev0[e] : nullptr, 0, p.lats, 1, p.o, max(1, kWarps * C / ne),
+            const int32_t at_e = e < ne ? base + todo0[e] : 0;
+            const int64_t nt = prep_box(e < ne ? &ev0[at_e] : nullptr, 0, p.lats, 1, p.o, max(1, kWarps * C / ne),
                                         &prep[min(e, kPairEvals - 1)], p.err);
-            if (e < ne && (lane & 3) == 0) tiles[e] = nt;
+            if (e < ne && (lane & 3) == 0) {
+                tiles[e] = nt;
+                slot[e] = at_e;
+            }
         }
         __syncthreads();
         // the boxes' tiles one after another, dealt out over the warps
@@ -1009,8 +1047,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
                 inside += __shfl_xor_sync(0xffffffffu, inside, s);
             }
             if (lane == 0) {
-                if (empty) atomicAdd(&sum0[e], empty);
-                if (inside) atomicAdd(&pts0[e], inside);
+                if (empty) atomicAdd(&sum0[slot[e]], empty);
+                if (inside) atomicAdd(&pts0[slot[e]], inside);
             }
         }
         sync();
@@ -1018,10 +1056,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
             // gains; the best proposal holds the largest key of both clusters and is accepted
             int64_t g = 0;
             const unsigned below = (1u << lane) - 1u;
+            const int cur = ran & 1, nb = __popc(vm) + __popc(gm);
             const int es = __popc(vm & below), eg = __popc(vm) + __popc(gm & below);
             if (cand) {
-                const int64_t rem = (int64_t)obv[my_c] - (int64_t)sum[es];
-                const int64_t add = grew ? (int64_t)sum[eg] - (int64_t)obv[1 - my_c] : 0;
+                const int64_t rem = (int64_t)obv[my_c] - (int64_t)sum[cur][es];
+                const int64_t add = grew ? (int64_t)sum[cur][eg] - (int64_t)obv[1 - my_c] : 0;
                 g = rem - add;
             }
             const unsigned long long key =
@@ -1029,22 +1068,22 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
             proposals += __popc(__ballot_sync(0xffffffffu, key != 0));
             unsigned long long best = key;
             for (int s = 16; s > 0; s >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, s));
-            unsigned long long points = lane < ne ? pts[lane] : 0;
+            unsigned long long points = lane < nb ? pts[cur][lane] : 0;
             for (int s = 16; s > 0; s >>= 1) points += __shfl_xor_sync(0xffffffffu, points, s);
             ++ran;
-            e_last = ne;
+            e_last = nb;
             p_last = points;
-            e_sum += ne;
+            e_sum += nb;
             p_sum += points;
             const int win = best ? __ffs(__ballot_sync(0xffffffffu, key == best)) - 1 : -1;
             if (lane == win) {
                 const int to = 1 - my_c;
                 p.assign[t] = k0 + to;
-                for (int i = 0; i < 6; ++i) box[my_c].b[i] = ev[es].b[i];
-                obv[my_c] = sum[es];
+                for (int i = 0; i < 6; ++i) box[my_c].b[i] = ev[cur][es].b[i];
+                obv[my_c] = sum[cur][es];
                 if (grew) {
-                    for (int i = 0; i < 6; ++i) box[to].b[i] = ev[eg].b[i];
-                    obv[to] = sum[eg];
+                    for (int i = 0; i < 6; ++i) box[to].b[i] = ev[cur][eg].b[i];
+                    obv[to] = sum[cur][eg];
                 }
                 ctl.size[my_c] -= 1;
                 ctl.size[to] += 1;
@@ -1144,8 +1183,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_pair_rounds(const PairArgs p)
             }
             base = __shfl_sync(0xffffffffu, base, 0);
             if (lane < e_last) {
-                p.evals[base + lane] = ev[lane];
-                p.ecount[base + lane] = sum[lane];
+                p.evals[base + lane] = ev[(ran - 1) & 1][lane];
+                p.ecount[base + lane] = sum[(ran - 1) & 1][lane];
             }
         }
     }
