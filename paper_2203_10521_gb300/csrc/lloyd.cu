@@ -814,7 +814,8 @@ __global__ void k_sum_points(const uint64_t* __restrict__ pts, const int32_t* __
 // which cover every round of every pair).  Round by round the layer takes 13
 // launches and a round trip to the host each, all pairs in every round: three
 // iterations of 200k triangles in 1,024 clusters 3.3 ms a call, this way 1.3;
-// six with rotation descent of 2M in 16,384 clusters 13.9 and 11.1 ms.
+// six with rotation descent of 2M in 16,384 clusters 13.9 and 11.1 ms (1.1 and
+// 8.2 since the boxes' preparation, the counts and the box update got cheaper).
 constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each (prepared by three warps, eight each)
 constexpr int kPairMoves = 64;      // most rounds of a step that take this path
 constexpr int kPairGraphMin = 64;   // pairs of a layer whose captured iteration takes it (the launch counter of a small

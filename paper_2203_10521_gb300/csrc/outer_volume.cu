@@ -13,8 +13,8 @@
 //          x wk * tk (z) rows of one box, wj * wk = 32 lanes.  A tile outside
 //          the box's shadow is skipped and the rows of a tile are clipped to
 //          it.  Each lane owns one j and walks tk rows along z: it divides the
-//          six slab bounds exactly once per tile (integer reciprocal) and then
-//          steps them as 32.32 fixed-point values (boxes whose three slabs are
+//          lower slab bounds exactly once per tile (integer reciprocal; the
+//          upper ones follow from the slabs' widths) and then steps all six as 32.32 fixed-point values (boxes whose three slabs are
 //          DDA slabs) or with a remainder carry (the general loop), so each
 //          row's exact x-interval costs adds and compares only.  The occupied
 //          bits of the interval are popcounted over 64-bit words; outer volume
@@ -626,7 +626,7 @@ __device__ __forceinline__ void quantize_warp(const obb_box& B, const LatticeFra
 // cluster's warps.  Such a call is latency: of the general path's six launches
 // (box count, quantisation, preparation, two for the tile offsets, counting)
 // and of lanes that walk 32 rows one after another.  Five boxes on 64^3: 27 us
-// of kernels and 39 a call that way, 12 and 23 this way.  No scratch, no zeroed
+// of kernels and 37 a call that way, 10 and 12 this way.  No scratch, no zeroed
 // outputs: the cluster's sums meet in distributed shared memory and its first
 // block writes them.  Boxes are quantised ones, or float ones quantised on the
 // way (frame given).
