@@ -150,3 +150,23 @@ def test_tree_score_is_the_weighted_sum_of_its_levels(ctx, torus, depth):
     want = sum((depth - lev + 1) * int(ctx.tree_read(tree, lev)["obv"].sum()) for lev in range(depth + 1))
     assert ctx.tree_score(tree)[0] == want
     tree.free()
+
+
+@pytest.mark.parametrize("level,refit", [(1, 1), (2, 3), (3, 2), (4, 1)])
+def test_captured_rounds_of_few_large_pairs(ctx, level, refit):
+    """20,000 to 5,000 triangles a cluster take the pairs' rounds in a graph too, 2,500 do not."""
+    m = M.torus(1.0, 0.3, 200, 100, jitter=0.004, seed=10)
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, 90)
+    tree = ctx.build_tree(lat, level, 0)
+    r = ctx.tree_read(tree, level)
+    parent = (np.arange(1 << level) // 2).astype(np.int32)
+    layers = [ctx.layer_init(lat, r["assign"], parent, r["frames"]) for _ in range(3)]
+    for it in range(3):
+        st = [_step(ctx, layers[0], 0, rounds=16, refit=refit), _step(ctx, layers[1], 2, rounds=16, refit=refit),
+              _step(ctx, layers[2], 0, rounds=16, refit=refit, graph=True)]
+        assert st[0] == st[1] == st[2]
+        for x in layers[1:]:
+            _same(ctx.layer_read(layers[0]), ctx.layer_read(x))
+    for x in layers + [tree, lat, mesh]:
+        x.free()
