@@ -56,3 +56,26 @@ def test_frames_do_not_depend_on_the_number_of_clusters(ctx, kind, jitter, share
         assert np.array_equal(out[0][key][:shared], out[1][key][:shared]), key
     lat.free()
     mesh.free()
+
+
+@pytest.mark.parametrize("members", [1, 2, 127, 128, 129, 257, 513, 641, 5000])
+def test_frames_do_not_depend_on_how_members_are_loaded(ctx, members):
+    """Layers of large clusters load their members ahead; the sums keep their order."""
+    m = M.torus(1.0, 0.3, 200, 100, jitter=0.004, seed=8)    # 40,000 triangles
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, 64)
+    T = len(m.tris)
+    pick = np.random.default_rng(members).permutation(T)
+    out = []
+    for K in (3, 300):                                       # 13,333 and 133 triangles a cluster
+        a = np.empty(T, np.int32)
+        a[pick[:members]] = 0
+        a[pick[members:]] = 1 + np.arange(T - members) % (K - 1)
+        layer = ctx.layer_init(lat, a, np.zeros(K, np.int32))
+        r = ctx.layer_read(layer)
+        out.append([r[key][0] for key in ("frames", "qboxes", "obv")])
+        layer.free()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+    lat.free()
+    mesh.free()
