@@ -225,7 +225,7 @@ __device__ __forceinline__ bool dir_rect(const float3 A, const float3 B, const f
 // issue (64 boxes, 10k triangles, m = 32: 42.2 ms); a triangle meets only the
 // rays inside its projection, so a thread projects a triangle onto the faces
 // and only the texels it covers are tested, with the same ray-triangle test,
-// each ray keeping its sums in shared memory (the same call: 0.073 ms).  What
+// each ray keeping its sums in shared memory (the same call: 0.066 ms).  What
 // is left is the walk over the mesh (gathers from L2) and the boxes near the
 // surface, where a few triangles cover many texels.
 // - Triangles beyond the box's farthest exit are left out.
