@@ -411,6 +411,9 @@ __device__ __noinline__ int64_t prep_box(const obb_qbox* __restrict__ qin, int32
         const int32_t smax = max(geti(own, 0), max(geti(own, 1), geti(own, 2)));
         if (smax > 0 && (int64_t)(tk - 1) * smax >= (int64_t(1) << 29)) tk = max(1, min(tk, (1 << 29) / smax));
     }
+    // A warp adds up its tile's points in 32 bits: 32 lanes, tk rows each, rows
+    // of at most span + 1 points.  Only rows beyond 2^20 points cut a tile.
+    if ((int64_t)tk * (span + 1) >= (int64_t(1) << 27)) tk = ((1 << 27) - 1) / (span + 1);
     if (!on) return 0;
     if (lane < 3) {
         out->sat_nu[a][0] = nu_j;
