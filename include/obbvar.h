@@ -109,7 +109,7 @@ const char* obb_last_error(const obb_ctx* ctx);
 
 /* Instrumentation.  `launches` counts every kernel this context has enqueued
  * (library kernels and the radix-sort kernels compiled into the library).
- * With profiling enabled, each launch of the outer-volume counting kernel is
+ * With profiling enabled, each launch of an outer-volume counting kernel is
  * bracketed by CUDA events on the context stream (launches inside a Lloyd
  * iteration run as a CUDA graph are not) and the kernel adds up its
  * algorithmic traffic (16 bytes per 128-bit occupancy chunk that a box row's
@@ -121,10 +121,12 @@ const char* obb_last_error(const obb_ctx* ctx);
  * its boxes that lie inside the lattice domain [0, N)^3: the points whose
  * occupancy bit it reads (points outside the domain are empty by definition
  * and cost no memory).  obb_profile_enable resets the totals: on = 1 times
- * every counting launch and adds up its bytes and rows, on = 2 only times it
- * (the kernel then runs without the byte and row counters, as it does with
- * profiling off), on = 0 stops; obb_profile_read synchronises and reports
- * the totals. */
+ * every counting launch and adds up its bytes and rows (every count that is
+ * not part of a captured iteration is then a launch of the counting kernel of
+ * its own), on = 2 only times the counting launches and changes nothing else
+ * (counts made inside another kernel -- the rounds of sibling pairs, exact
+ * flooding -- are no launches of their own and are not timed), on = 0 stops;
+ * obb_profile_read synchronises and reports the totals. */
 typedef struct {
     int64_t launches;        /* kernels enqueued by the context since creation */
     int64_t count_launches;  /* counting-kernel launches since profiling was enabled */

@@ -339,7 +339,8 @@ class Context:
     # ------------------------------------------------------- instrumentation
     def profile_enable(self, on=True):
         """True/1: time every counting launch and add up its algorithmic bytes
-        and rows; 2: time only (the kernel without its counters); False/0: off."""
+        and rows (every count is then a launch of its own); 2: time the counting
+        launches that there are, nothing else changes; False/0: off."""
         self.check(self.lib.obb_profile_enable(self.h, int(on)))
 
     def profile_read(self):

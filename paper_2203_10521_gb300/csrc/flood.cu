@@ -923,8 +923,8 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     OBB_TRY(set_device_int(ctx, ctr + 2, (int32_t)(T - K)));
     obb_flood_stats st{};
     int64_t evals_total = 0;
-    // profiled launches keep the counting kernel's own launches and counters, a wave at a time
-    const bool run = mode == 0 && ctx->prof == 0;
+    // with profiling counters (mode 1) the counting kernel's own launches, a wave at a time
+    const bool run = mode == 0 && ctx->prof != 1;
     if (run) OBB_TRY(flood_exact(ctx, L, mem, group, gstart, gbox, key, nassign, &st.waves, &evals_total));
     while (!run) {
         OBB_CK(ctx, cudaMemcpyAsync(hi, ctr + 2, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -2375,7 +2375,7 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, bool* yes)
 {
     LayerMem* M = mem_of(L);
     *yes = false;
-    if (ctx->prof != 0 || ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
+    if (ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -2616,7 +2616,8 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
     const int dsteps = (opts && opts->descent_steps > 0) ? opts->descent_steps : 2;
     if (opts && opts->graph && !L->mlp) return lloyd_step_graph(ctx, L, rounds, refit_mode, dsteps, st);
     bool pairs = false;
-    OBB_TRY(pair_path(ctx, L, rounds, &pairs));
+    // profiling with counters (mode 1) counts in launches of the counting kernel
+    if (ctx->prof != 1) OBB_TRY(pair_path(ctx, L, rounds, &pairs));
     if (pairs) {
         if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
         OBB_TRY(pair_rounds(ctx, L, rounds));

@@ -14,12 +14,13 @@
 //          the box's shadow is skipped and the rows of a tile are clipped to
 //          it.  Each lane owns one j and walks tk rows along z: it divides the
 //          lower slab bounds exactly once per tile (integer reciprocal; the
-//          upper ones follow from the slabs' widths) and then steps all six as 32.32 fixed-point values (boxes whose three slabs are
-//          DDA slabs) or with a remainder carry (the general loop), so each
-//          row's exact x-interval costs adds and compares only.  The occupied
-//          bits of the interval are popcounted over 64-bit words; outer volume
-//          = interval length - occupied bits, and rows or points outside
-//          [0, N)^3 are all empty.
+//          upper ones follow from the slabs' widths) and then steps all six as
+//          32.32 fixed-point values (boxes whose three slabs are DDA slabs) or
+//          with a remainder carry (the general loop), so each row's exact
+//          x-interval costs adds and compares only.  The occupied bits of the
+//          interval are popcounted over 64-bit words; outer volume = interval
+//          length - occupied bits, and rows or points outside [0, N)^3 are all
+//          empty.
 // Counts are integer sums (warp reduction + one 64-bit atomic per tile), so
 // the result does not depend on scheduling.
 #include <cooperative_groups.h>
@@ -639,7 +640,7 @@ constexpr int kFewThreads = 256;
 // cluster per box cannot share a large box out over the whole machine as the
 // general path's tile queue does (31 boxes of a tree's top levels at 1024^3: 267
 // against 106 us; 255 boxes at 544^3: 134 against 84 us; seven at 340^3: 60
-// against 73 us).  Profiled launches keep the general path and its counters.
+// against 73 us).  Profiling with counters (mode 1) needs the general path's.
 constexpr int64_t kFewMaxBoxes = 512;
 constexpr int64_t kFewMaxLatticeBytes = int64_t(2) << 20;
 constexpr int64_t kFewMaxWork = int64_t(64) << 20;
@@ -819,8 +820,17 @@ static int32_t count_grid_warps(const obb_ctx* ctx) { return 32 * ctx->num_sms; 
 
 static bool few_boxes(const obb_ctx* ctx, int64_t K_cap, int64_t lattice_bytes)
 {
-    return ctx->prof == 0 && K_cap <= kFewMaxBoxes && lattice_bytes <= kFewMaxLatticeBytes &&
+    return ctx->prof != 1 && K_cap <= kFewMaxBoxes && lattice_bytes <= kFewMaxLatticeBytes &&
            K_cap * lattice_bytes <= kFewMaxWork;
+}
+
+// The events around a counting launch (with profiling on): one before, one after.
+static obb_status prof_event(obb_ctx* ctx, cudaEvent_t* e)
+{
+    if (!ctx->prof) return OBB_OK;
+    OBB_CK(ctx, cudaEventCreate(e));
+    OBB_CK(ctx, cudaEventRecord(*e, ctx->stream));
+    return OBB_OK;
 }
 
 static obb_status launch_few(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats, const int32_t* d_lat_of_box,
@@ -839,11 +849,15 @@ static obb_status launch_few(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    OBB_TRY(prof_event(ctx, &e0));
     OBB_CK(ctx, cudaLaunchKernelEx(&cfg, k_count_few, d_boxes, d_fboxes, d_frame, d_K, (int32_t)K_cap, d_lats, n_lats,
                                    d_lat_of_box, CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank},
                                    reinterpret_cast<unsigned long long*>(d_counts),
                                    reinterpret_cast<unsigned long long*>(d_points), dom, ctx->d_err));
     note_launch(ctx);
+    OBB_TRY(prof_event(ctx, &e1));
+    if (ctx->prof) ctx->prof_ev.emplace_back(e0, e1);
     return OBB_OK;
 }
 
@@ -951,18 +965,12 @@ obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
         note_launch(ctx, 2);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (ctx->prof) {
-        OBB_CK(ctx, cudaEventCreate(&e0));
-        OBB_CK(ctx, cudaEventCreate(&e1));
-        OBB_CK(ctx, cudaEventRecord(e0, s));
-    }
+    OBB_TRY(prof_event(ctx, &e0));
     launch_count(ctx, s, ctx->prof == 1, lattice_bytes, prep, off, d_K, (int32_t)K_cap, d_counts, d_points,
                  ctx->prof == 1 ? ctx->d_prof : nullptr, ctx->d_prof + 2, perm);
     note_launch(ctx);
-    if (ctx->prof) {
-        OBB_CK(ctx, cudaEventRecord(e1, s));
-        ctx->prof_ev.emplace_back(e0, e1);
-    }
+    OBB_TRY(prof_event(ctx, &e1));
+    if (ctx->prof) ctx->prof_ev.emplace_back(e0, e1);
     OBB_CK(ctx, cudaGetLastError());
     return OBB_OK;
 }
