@@ -819,10 +819,20 @@ __global__ void k_sum_points(const uint64_t* __restrict__ pts, const int32_t* __
 constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each (prepared by three warps, eight each)
 constexpr int kPairMoves = 64;      // most rounds of a step that take this path
 // A captured iteration takes the pairs' rounds from this many pairs on, or with clusters beyond kPairGraphSize triangles
-// on average (the launch counter of a small captured layer is read per round): the layer's rounds walk a cluster with
-// one block (four clusters of 246,000 triangles, three iterations: 14.1 ms of extents and 6.9 of member lists, 2.4 this way).
+// on average.  Captured, the layer's rounds wait for no host either, so below both lines the two are alike (1,920
+// triangles in 1 to 32 pairs at 64^3 to 256^3, four steps: 0.44 to 1.02 ms, 0.45 to 1.18 host-driven by pairs); above, the
+// layer's walk a cluster with one block (four clusters of 246,000 triangles, three iterations: 14.1 ms of extents and 6.9
+// of member lists, 2.4 this way).
 constexpr int kPairGraphMin = 64;
 constexpr int64_t kPairGraphSize = 4096;
+
+// At most eight blocks count a pair's boxes, all of the machine counts a layer's, so large boxes in few pairs belong to
+// the layer's rounds, unless those lose more on walking large clusters with one block each.  The boxes' rows grow with
+// N^2, both walks with the triangles: N^2 <= 65,536 a pair + 32 a triangle.  Pairs against layer, us a step: one pair of
+// 1,920 triangles 1,023 : 1,252 at 256^3, 1,798 : 1,339 at 512^3, 29,795 : 2,441 at 2048^3; eight pairs of 200,000
+// 2,291 : 5,810 at 1024^3, 8,632 : 7,857 at 2048^3.  Over 738 layers (320 to 250,000 triangles, 1 to 256 pairs, 64^3 to
+// 2048^3) the slower side is 24 times slower; by this line the mean loss is 2 %, the largest 2.2 times.
+constexpr int64_t kPairRows = 65536, kPairTriRows = 32;
 
 struct PairArgs {
     const int32_t *U, *F, *adj;
@@ -2376,6 +2386,7 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, bool* yes)
     LayerMem* M = mem_of(L);
     *yes = false;
     if (ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
+    if ((int64_t)L->lat->frame.N * L->lat->frame.N > kPairRows * (L->K / 2) + kPairTriRows * L->T) return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));

@@ -1,0 +1,54 @@
+"""Which layers of sibling pairs run their rounds pair by pair (few launches a
+step) and which as the layer's rounds, and that the results do not tell."""
+import numpy as np
+import pytest
+
+from synth import meshes as M
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2203_10521_gb300 as P
+    c = P.Context(0)
+    yield c
+    torch.cuda.synchronize()
+    c.close()
+
+
+def _step(ctx, layer, **kw):
+    n0 = ctx.profile_read()["launches"]
+    st = ctx.lloyd_step(layer, **kw)
+    return st, ctx.profile_read()["launches"] - n0
+
+
+# N^2 <= 65,536 pairs + 32 triangles: both sides of the line by lattice, by pairs and by triangles
+@pytest.mark.parametrize("nu,nv,N,level,by_pairs", [(60, 16, 350, 1, True), (60, 16, 360, 1, False),
+                                                    (60, 16, 568, 3, True), (60, 16, 700, 3, False),
+                                                    (200, 100, 700, 1, True)])
+def test_large_boxes_of_few_pairs_take_the_layer_rounds(ctx, nu, nv, N, level, by_pairs):
+    m = M.torus(1.0, 0.3, nu, nv, jitter=0.004, seed=9)
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, N)
+    tree = ctx.build_tree(lat, level, 0)
+    r = ctx.tree_read(tree, level)
+    parent = (np.arange(1 << level) // 2).astype(np.int32)
+    out = []
+    for mode in (0, 1):          # profiling with counters always takes the layer's
+        layer = ctx.layer_init(lat, r["assign"], parent, r["frames"])
+        ctx.profile_enable(mode)
+        st, n = _step(ctx, layer, rounds=16, refit=0)
+        ctx.profile_enable(0)
+        out.append((st, n, ctx.layer_read(layer)))
+        layer.free()
+    (sa, na, a), (sb, nb, b) = out
+    assert sa == sb
+    for k in ("assign", "qboxes", "obv"):
+        assert np.array_equal(a[k], b[k]), k
+    assert (na < nb) == by_pairs and (na == nb) != by_pairs
+    for x in (tree, lat, mesh):
+        x.free()
