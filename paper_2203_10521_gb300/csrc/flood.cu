@@ -23,6 +23,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "counting.cuh"
@@ -465,7 +466,9 @@ __global__ void k_fl_local(const int32_t* __restrict__ U, const int32_t* __restr
     lbox[i] = s;
 }
 
-constexpr int32_t kRunSteps = 4096;   // triangles a launch takes from each group (a launch stays below 0.1 s)
+// triangles a launch takes from each group: 40 ms at 1024^3, a quarter of a second at worst (24,000 triangles in one
+// group of two boxes that fill 2048^3)
+constexpr int32_t kRunSteps = 4096;
 
 // The order of a group's triangles after its seeds, a warp per group: the
 // smallest priority among the available triangles (a list in the group's
@@ -923,8 +926,14 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     OBB_TRY(set_device_int(ctx, ctr + 2, (int32_t)(T - K)));
     obb_flood_stats st{};
     int64_t evals_total = 0;
-    // with profiling counters (mode 1) the counting kernel's own launches, a wave at a time
-    const bool run = mode == 0 && ctx->prof != 1;
+    // With profiling counters (mode 1) the counting kernel's own launches, a wave at a time; and where the boxes are large
+    // for the number of triangles: a group's cluster counts them with eight blocks, a wave with all of the machine.  A
+    // run's counts grow with the boxes that grow (about the root of the triangles) and with N^3 of the points they
+    // hold, the waves with the triangles: N^3 <= 6 10^7 sqrt(T).  Run against waves, ms: 144 triangles 2.6 : 4.7 at 512^3,
+    // 10.4 : 5.4 at 1024^3; 1,920 triangles 50 : 113 at 1024^3, 122 : 116 at 1448^3, 282 : 121 at 2048^3; 24,000 at 2048^3
+    // 1,296 : 1,583.
+    const double side = (double)lat->frame.N;
+    const bool run = mode == 0 && ctx->prof != 1 && side * side * side <= 6e7 * std::sqrt((double)T);
     if (run) OBB_TRY(flood_exact(ctx, L, mem, group, gstart, gbox, key, nassign, &st.waves, &evals_total));
     while (!run) {
         OBB_CK(ctx, cudaMemcpyAsync(hi, ctr + 2, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
