@@ -834,6 +834,17 @@ constexpr int64_t kPairGraphSize = 4096;
 // 2048^3) the slower side is 24 times slower; by this line the mean loss is 2 %, the largest 2.2 times.
 constexpr int64_t kPairRows = 65536, kPairTriRows = 32;
 
+// A layer whose last step moved nothing most likely runs one round, where all pairs take part and the pairs' rounds have
+// nothing to leave out: a pair's round is one long chain of dependent work, and from a few hundred pairs on large
+// lattices the layer's kernels, which spread the same work evenly, are through it sooner.  A settled step by pairs and
+// by the layer, us, captured | host-driven: 8,192 pairs at 1024^3 387, 179 | 391, 229; 512 pairs 209, 114 | 210, 154; 128
+// pairs at 715^3 150, 106 | 153, 116; but 128 pairs at 495^3 100, 102 | 98, 113, 256 at 256^3 75, 100 | 95, 135.  The
+// first steps of a layer go the other way (11 rounds of 8,192 pairs 1,521, 2,438 | 1,454, 3,010).
+constexpr int kSettledPairs = 128;
+constexpr int64_t kSettledSide = 512;
+// A second graph costs about what one or two settled steps gain by it.
+constexpr int kSettledHost = 1, kSettledGraph = 2;
+
 struct PairArgs {
     const int32_t *U, *F, *adj;
     int32_t* assign;
@@ -2220,15 +2231,18 @@ struct LayerMem {
     obb_qbox* pq = nullptr;         // [K * 6] probe boxes
     unsigned long long* pbest = nullptr;  // [K]
     int32_t cand_cap = 0, eval_cap = 0;
-    // a whole Lloyd iteration captured as one CUDA graph (see lloyd_step_graph)
-    cudaGraphExec_t gexec = nullptr;
-    int gkey[5] = {-1, -1, -1, -1, -1};   // rounds, refit mode, descent steps, counting-tile generation, sibling pairs
+    // a whole Lloyd iteration captured as one CUDA graph (see lloyd_step_graph), with the layer's rounds and the pairs'
+    struct StepGraph {
+        cudaGraphExec_t exec = nullptr;
+        int key[4] = {-1, -1, -1, -1};              // rounds, refit mode, descent steps, counting-tile generation
+        int64_t round = 0, rebuild = 0, post = 0;   // kernel launches per round, per rebuild, after the loop
+    } graphs[2];
     int64_t* loop = nullptr;          // [0] rounds run, [1] moves before the round, [2] rebuilds, [3] total
-    CountScratch cscr{};              // the graph's own counting scratch (fixed addresses)
+    CountScratch cscr{};              // the graphs' own counting scratch (fixed addresses)
     void* cscr_mem = nullptr;
     void* slab = nullptr;             // the arrays of the layer that are allocated with it
-    int64_t g_round = 0, g_rebuild = 0, g_post = 0;   // kernel launches per round, per rebuild, after the loop
     bool members_valid = false;
+    int settled = 0;            // steps in a row that moved no triangle, as far as the host has read them
     // sibling pairs (k_pair_rounds): 1 / 0 known, -1 to be looked at (parents may have changed)
     int paired = -1;
     int4* pinfo = nullptr;      // [K / 2]
@@ -2330,7 +2344,8 @@ void layer_destroy(obb_layer* L)
     cudaStream_t s = L->ctx ? L->ctx->stream : nullptr;
     LayerMem* M = mem_of(L);
     if (M) {
-        if (M->gexec) cudaGraphExecDestroy(M->gexec);
+        for (auto& g : M->graphs)
+            if (g.exec) cudaGraphExecDestroy(g.exec);
         if (M->loop) cudaFreeAsync(M->loop, s);
         if (M->cscr_mem) cudaFreeAsync(M->cscr_mem, s);
         for (void* p : {(void*)M->slab, (void*)M->feats, (void*)M->pred, (void*)M->skey, (void*)M->slot})
@@ -2378,15 +2393,22 @@ static obb_status check_pairs(obb_ctx* ctx, obb_layer* L)
 
 static void pairs_known(obb_ctx* ctx, obb_layer* L) { mem_of(L)->paired = ctx->h_small[kPairedSlot] != 0 ? 1 : 0; }
 
-void layer_parents_changed(obb_layer* L) { mem_of(L)->paired = -1; }
+void layer_parents_changed(obb_layer* L)
+{
+    mem_of(L)->paired = -1;
+    mem_of(L)->settled = 0;
+}
 
-// Whether the layer's rounds run pair by pair (k_pair_rounds).
-static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, bool* yes)
+// Whether the layer's rounds run pair by pair (k_pair_rounds).  settled: steps without a move after which a large layer
+// takes its own rounds.
+static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled, bool* yes)
 {
     LayerMem* M = mem_of(L);
     *yes = false;
     if (ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
-    if ((int64_t)L->lat->frame.N * L->lat->frame.N > kPairRows * (L->K / 2) + kPairTriRows * L->T) return OBB_OK;
+    const int64_t N = L->lat->frame.N;
+    if (N * N > kPairRows * (L->K / 2) + kPairTriRows * L->T) return OBB_OK;
+    if (M->settled >= settled && L->K / 2 >= kSettledPairs && N > kSettledSide) return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -2628,12 +2650,14 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
     if (opts && opts->graph && !L->mlp) return lloyd_step_graph(ctx, L, rounds, refit_mode, dsteps, st);
     bool pairs = false;
     // profiling with counters (mode 1) counts in launches of the counting kernel
-    if (ctx->prof != 1) OBB_TRY(pair_path(ctx, L, rounds, &pairs));
+    if (ctx->prof != 1) OBB_TRY(pair_path(ctx, L, rounds, kSettledHost, &pairs));
     if (pairs) {
         if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
         OBB_TRY(pair_rounds(ctx, L, rounds));
         OBB_TRY(layer_box_update(ctx, L, refit_mode, dsteps));
-        return layer_finish_stats(ctx, L, -1, st);
+        OBB_TRY(layer_finish_stats(ctx, L, -1, st));
+        M->settled = st && st->moves == 0 ? M->settled + 1 : 0;
+        return OBB_OK;
     }
     OBB_CK(ctx, cudaMemsetAsync(L->d_stats, 0, sizeof(int64_t) * kStCount, s));
     int64_t* h = host_stats(ctx);
@@ -2650,6 +2674,7 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
         if (moved > 0) M->members_valid = false;
         if (moved == 0) break;
     }
+    M->settled = before == 0 ? M->settled + 1 : 0;
     OBB_TRY(layer_box_update(ctx, L, refit_mode, dsteps));
     return layer_finish_stats(ctx, L, ran, st);
 }
@@ -2658,8 +2683,8 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
 // device-side WHILE loop (a conditional node whose condition the last kernel of
 // each round sets), the member lists are rebuilt inside an IF node after a
 // round that moved triangles, and the box update follows.  The graph is
-// captured once per (rounds, refit, descent steps, counting tile) and
-// relaunched; it runs the same kernels in the same order as the host loop, so
+// captured once per (rounds, refit, descent steps, counting tile; one with the
+// pairs' rounds, one with the layer's) and relaunched; it runs the same kernels in the same order as the host loop, so
 // results are identical, without a host round trip per round.  Its counting
 // launches use scratch of their own (fixed addresses) and are not profiled one
 // by one.
@@ -2671,12 +2696,13 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
     cudaStream_t s = ctx->stream;
     if (!M->members_valid) OBB_TRY(rebuild_members(ctx, L));
     bool pairs = false;
-    if (K / 2 >= kPairGraphMin || L->T > kPairGraphSize * K) OBB_TRY(pair_path(ctx, L, rounds, &pairs));
-    if (!M->gexec || M->gkey[0] != rounds || M->gkey[1] != refit_mode || M->gkey[2] != dsteps ||
-        M->gkey[3] != ctx->tile_gen || M->gkey[4] != (int)pairs) {
-        if (M->gexec) {
-            OBB_CK(ctx, cudaGraphExecDestroy(M->gexec));
-            M->gexec = nullptr;
+    if (K / 2 >= kPairGraphMin || L->T > kPairGraphSize * K)
+        OBB_TRY(pair_path(ctx, L, rounds, kSettledGraph, &pairs));
+    LayerMem::StepGraph& G = M->graphs[pairs];
+    if (!G.exec || G.key[0] != rounds || G.key[1] != refit_mode || G.key[2] != dsteps || G.key[3] != ctx->tile_gen) {
+        if (G.exec) {
+            OBB_CK(ctx, cudaGraphExecDestroy(G.exec));
+            G.exec = nullptr;
         }
         if (!M->loop) OBB_CK(ctx, pool_alloc((void**)&M->loop, sizeof(int64_t) * 4, s));
         if (!M->cscr_mem) {
@@ -2719,11 +2745,11 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
                 if (rc != OBB_OK) return false;
                 k_total<<<1, 1024, 0, cs[0]>>>(L->d_obv, K, M->loop + 3, nullptr);
                 note_launch(ctx);
-                M->g_post = ctx->launches - l2;
+                G.post = ctx->launches - l2;
                 if (!ck(cudaGetLastError())) return false;
                 if (!ck(cudaStreamEndCapture(cs[0], &g))) return false;
                 depth = 0;
-                return ck(cudaGraphInstantiate(&M->gexec, g, 0));
+                return ck(cudaGraphInstantiate(&G.exec, g, 0));
             };
             if (pairs) {
                 // sibling pairs: every round in one launch
@@ -2732,8 +2758,8 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
                 rc = pair_rounds(ctx, L, rounds);
                 if (rc != OBB_OK) break;
                 const int64_t n = ctx->launches - l0;
-                M->g_round = M->g_rebuild = 0;
-                if (finish()) M->g_post += n;
+                G.round = G.rebuild = 0;
+                if (finish()) G.post += n;
                 break;
             }
             ck(cudaMemsetAsync(L->d_stats, 0, sizeof(int64_t) * kStCount, cs[0]));
@@ -2766,7 +2792,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
             k_round_end<<<1, 1, 0, cs[1]>>>(L->d_stats, M->loop, rounds, again, rebuild);
             note_launch(ctx);
             if (!ck(cudaGetLastError())) break;
-            M->g_round = ctx->launches - l0;
+            G.round = ctx->launches - l0;
             cudaGraph_t bg = nullptr;
             if (!ck(cudaStreamGetCaptureInfo(cs[1], &cst, nullptr, &bg, &deps, nullptr, &nd))) break;
             cudaGraphNodeParams ip = {};
@@ -2787,7 +2813,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
             const int64_t l1 = ctx->launches;
             rc = rebuild_members(ctx, L);
             if (rc != OBB_OK) break;
-            M->g_rebuild = ctx->launches - l1;
+            G.rebuild = ctx->launches - l1;
             if (!ck(cudaStreamEndCapture(cs[2], &ibody))) break;
             depth = 2;
             if (!ck(cudaStreamEndCapture(cs[1], &bg))) break;
@@ -2808,20 +2834,20 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
         for (auto& c : cs) cudaStreamDestroy(c);
         if (rc != OBB_OK) return rc;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "capture of the Lloyd iteration");
-        M->gkey[0] = rounds;
-        M->gkey[1] = refit_mode;
-        M->gkey[2] = dsteps;
-        M->gkey[3] = ctx->tile_gen;
-        M->gkey[4] = (int)pairs;
+        G.key[0] = rounds;
+        G.key[1] = refit_mode;
+        G.key[2] = dsteps;
+        G.key[3] = ctx->tile_gen;
     }
-    OBB_CK(ctx, cudaGraphLaunch(M->gexec, s));
+    OBB_CK(ctx, cudaGraphLaunch(G.exec, s));
     int64_t* h = host_stats(ctx);
     OBB_CK(ctx, cudaMemcpyAsync(h, L->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
     OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, M->loop, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost, s));
     OBB_TRY(check_device_error(ctx));
     M->members_valid = true;
+    M->settled = h[kStAccepted] == 0 ? M->settled + 1 : 0;
     const int64_t ran = pairs ? h[kStRounds] : h[kStCount], rebuilds = h[kStCount + 2];
-    note_launch(ctx, (int)(M->g_round * ran + M->g_rebuild * rebuilds + M->g_post));
+    note_launch(ctx, (int)(G.round * ran + G.rebuild * rebuilds + G.post));
     if (st) {
         st->rounds_run = (int32_t)ran;
         st->refits_accepted = (int32_t)h[kStRefits];
@@ -3387,6 +3413,7 @@ void layer_members_changed(obb_layer* L)
 {
     mem_of(L)->members_valid = false;
     mem_of(L)->incr_ok = false;   // moved by something that keeps no move records
+    mem_of(L)->settled = 0;
 }
 
 obb_status layer_set_surrogate(obb_ctx* ctx, obb_layer* L, const obb_mlp* mlp, int32_t topk)

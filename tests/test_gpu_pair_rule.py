@@ -52,3 +52,48 @@ def test_large_boxes_of_few_pairs_take_the_layer_rounds(ctx, nu, nv, N, level, b
     assert (na < nb) == by_pairs and (na == nb) != by_pairs
     for x in (tree, lat, mesh):
         x.free()
+
+
+@pytest.mark.parametrize("graph,N,level,switches", [(False, 513, 8, True), (True, 513, 8, True), (False, 512, 8, False),
+                                                    (True, 512, 8, False), (False, 560, 7, False)])
+def test_settled_large_layers_take_their_own_rounds(ctx, graph, N, level, switches):
+    """From 128 pairs on above 512^3: after one step without a move, two when captured; a move takes them back."""
+    m = M.torus(1.0, 0.3, 90, 30, jitter=0.004, seed=3)      # 5,400 triangles
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, N)
+    tree = ctx.build_tree(lat, level, 0)
+    r = ctx.tree_read(tree, level)
+    parent = (np.arange(1 << level) // 2).astype(np.int32)
+    a = ctx.layer_init(lat, r["assign"], parent, r["frames"])
+    b = ctx.layer_init(lat, r["assign"], parent, r["frames"])
+    launches, quiet = [], 0
+    for _ in range(40):
+        st, n = _step(ctx, a, rounds=16, refit=0, graph=graph)
+        ctx.profile_enable(1)
+        assert st == ctx.lloyd_step(b, rounds=16, refit=0)   # by the layer's rounds
+        ctx.profile_enable(0)
+        quiet = quiet + 1 if st["moves"] == 0 else 0
+        launches.append((quiet, n))
+        if quiet == 5:
+            break
+    assert quiet == 5 and launches[0][0] == 0
+    by_pairs = launches[0][1]
+    assert by_pairs < 6
+    for q, n in launches:
+        later = q > (2 if graph else 1)
+        assert (n > by_pairs) == (switches and later), launches
+    # the layer changes: pairs again, and the same results
+    for x in (a, b):
+        ctx.flood_partition(x, mode=0)
+    st, n = _step(ctx, a, rounds=16, refit=0, graph=graph)
+    ctx.profile_enable(1)
+    assert st == ctx.lloyd_step(b, rounds=16, refit=0) and st["moves"] > 0
+    ctx.profile_enable(0)
+    st2, n2 = _step(ctx, a, rounds=1, refit=0, graph=graph)
+    assert n2 == by_pairs
+    ctx.lloyd_step(b, rounds=1, refit=0)
+    x, y = ctx.layer_read(a), ctx.layer_read(b)
+    for k in ("assign", "qboxes", "obv"):
+        assert np.array_equal(x[k], y[k]), k
+    for z in (a, b, tree, lat, mesh):
+        z.free()
