@@ -1405,6 +1405,53 @@ __global__ void __launch_bounds__(NT) k_moments(const float* __restrict__ V, con
     }
 }
 
+// The arithmetic of a covariance frame, FP64, every rounding written out: a
+// cluster's frame must not depend on which of the two kernels below solves it,
+// nor on what a compiler chooses to fuse there.
+
+// entry of the covariance: m / A - mu_a mu_b
+__device__ __forceinline__ double cov_entry(double m, double A, double mua, double mub)
+{
+    return __fma_rn(-mua, mub, __ddiv_rn(m, A));
+}
+
+// x y - z w and x y + z w, the second product rounded first
+__device__ __forceinline__ double mul_sub(double x, double y, double z, double w)
+{
+    return __fma_rn(x, y, -__dmul_rn(z, w));
+}
+__device__ __forceinline__ double mul_add(double x, double y, double z, double w)
+{
+    return __fma_rn(x, y, __dmul_rn(z, w));
+}
+
+// twice the sum of the squared off-diagonal entries
+__device__ __forceinline__ double off_diagonal(double a01, double a02, double a12)
+{
+    return __dmul_rn(2.0, __fma_rn(a12, a12, mul_add(a01, a01, a02, a02)));
+}
+
+// cosine and sine of the rotation that zeroes a_pq != 0
+struct JacobiTurn {
+    double c, s;
+};
+__device__ __forceinline__ JacobiTurn jacobi_turn(double app, double aqq, double apq)
+{
+    const double theta = __ddiv_rn(__dsub_rn(aqq, app), __dmul_rn(2.0, apq));
+    const double t = __ddiv_rn(theta >= 0.0 ? 1.0 : -1.0,
+                               __dadd_rn(fabs(theta), __dsqrt_rn(__fma_rn(theta, theta, 1.0))));
+    const double c = __ddiv_rn(1.0, __dsqrt_rn(__fma_rn(t, t, 1.0)));
+    return JacobiTurn{c, __dmul_rn(t, c)};
+}
+
+// row 2 of a frame: row 0 x row 1
+__device__ __forceinline__ void third_row(double* R)
+{
+    R[6] = mul_sub(R[1], R[5], R[2], R[4]);
+    R[7] = mul_sub(R[2], R[3], R[0], R[5]);
+    R[8] = mul_sub(R[0], R[4], R[1], R[3]);
+}
+
 // Cyclic Jacobi on the symmetric 3x3 covariance, FP64; frame rows = eigenvectors
 // sorted by decreasing eigenvalue, rows 0 and 1 with a positive largest-magnitude
 // component, row 2 = row 0 x row 1.
@@ -1414,31 +1461,28 @@ __device__ void jacobi3(const double c6[6], double R[9])
     double Vm[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
     double fro = 0.0;
     for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) fro += A[i][j] * A[i][j];
+        for (int j = 0; j < 3; ++j) fro = __fma_rn(A[i][j], A[i][j], fro);
     for (int sweep = 0; sweep < 16; ++sweep) {
-        double off = 2.0 * (A[0][1] * A[0][1] + A[0][2] * A[0][2] + A[1][2] * A[1][2]);
-        if (off <= 1e-30 * fro) break;
+        if (off_diagonal(A[0][1], A[0][2], A[1][2]) <= __dmul_rn(1e-30, fro)) break;
         for (int r = 0; r < 3; ++r) {
             const int p = r == 2 ? 1 : 0, qq = r == 0 ? 1 : 2;
             if (A[p][qq] == 0.0) continue;
-            double theta = (A[qq][qq] - A[p][p]) / (2.0 * A[p][qq]);
-            double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            double c = 1.0 / sqrt(t * t + 1.0);
-            double s = t * c;
+            const JacobiTurn u = jacobi_turn(A[p][p], A[qq][qq], A[p][qq]);
+            const double c = u.c, s = u.s;
             for (int k = 0; k < 3; ++k) {
                 double akp = A[k][p], akq = A[k][qq];
-                A[k][p] = c * akp - s * akq;
-                A[k][qq] = s * akp + c * akq;
+                A[k][p] = mul_sub(c, akp, s, akq);
+                A[k][qq] = mul_add(s, akp, c, akq);
             }
             for (int k = 0; k < 3; ++k) {
                 double apk = A[p][k], aqk = A[qq][k];
-                A[p][k] = c * apk - s * aqk;
-                A[qq][k] = s * apk + c * aqk;
+                A[p][k] = mul_sub(c, apk, s, aqk);
+                A[qq][k] = mul_add(s, apk, c, aqk);
             }
             for (int k = 0; k < 3; ++k) {
                 double vkp = Vm[k][p], vkq = Vm[k][qq];
-                Vm[k][p] = c * vkp - s * vkq;
-                Vm[k][qq] = s * vkp + c * vkq;
+                Vm[k][p] = mul_sub(c, vkp, s, vkq);
+                Vm[k][qq] = mul_add(s, vkp, c, vkq);
             }
         }
     }
@@ -1459,9 +1503,7 @@ __device__ void jacobi3(const double c6[6], double R[9])
         double sg = row[big] < 0.0 ? -1.0 : 1.0;
         for (int b = 0; b < 3; ++b) R[3 * a + b] = sg * row[b];
     }
-    R[6] = R[1] * R[5] - R[2] * R[4];
-    R[7] = R[2] * R[3] - R[0] * R[5];
-    R[8] = R[0] * R[4] - R[1] * R[3];
+    third_row(R);
 }
 
 __device__ __forceinline__ void put_normals(const double* R, const LatticeFrame* __restrict__ f, obb_qbox* q)
@@ -1488,10 +1530,10 @@ __global__ void k_frames_from_moments(const double* __restrict__ mom, const doub
     if (!(A > 0.0)) {
         for (int i = 0; i < 9; ++i) R[i] = fallback ? fallback[9 * (int64_t)k + i] : (i % 4 == 0 ? 1.0 : 0.0);
     } else {
-        const double mu[3] = {m[1] / A, m[2] / A, m[3] / A};
+        const double mu[3] = {__ddiv_rn(m[1], A), __ddiv_rn(m[2], A), __ddiv_rn(m[3], A)};
         const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
         double c6[6];
-        for (int q = 0; q < 6; ++q) c6[q] = m[4 + q] / A - mu[ia[q]] * mu[ib[q]];
+        for (int q = 0; q < 6; ++q) c6[q] = cov_entry(m[4 + q], A, mu[ia[q]], mu[ib[q]]);
         jacobi3(c6, R);
     }
     for (int i = 0; i < 9; ++i) out[9 * (int64_t)k + i] = R[i];
@@ -1502,8 +1544,7 @@ __global__ void k_frames_from_moments(const double* __restrict__ mom, const doub
 // divisions by A run on a lane each.  An FP64 instruction costs a warp 64
 // cycles whatever its lanes, so a cluster's chain shortens with its
 // instructions as long as every scheduler has a warp or two.  Lanes 0-2 hold
-// the rows of the covariance, 3-5 those of the eigenvectors; the products and
-// sums are fused as the compiler fuses jacobi3's.
+// the rows of the covariance, 3-5 those of the eigenvectors.
 constexpr int kFrameLanes = 8;
 __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ mom,
                                                      const double* __restrict__ fallback, int32_t K,
@@ -1522,10 +1563,10 @@ __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ 
     const bool solve = A > 0.0;
     auto get = [&](double x, int from) { return __shfl_sync(kAll, x, g0 + from); };
     // lanes 0-5: an entry of the covariance (xx, yy, zz, xy, xz, yz)
-    const double mu = (solve ? m[1 + min(r, 2)] : 0.0) / (solve ? A : 1.0);
+    const double mu = __ddiv_rn(solve ? m[1 + min(r, 2)] : 0.0, solve ? A : 1.0);
     const int ia = r == 5 ? 1 : r > 2 ? 0 : r, ib = r == 3 ? 1 : r > 3 ? 2 : r;
     const double mx = get(mu, ia), my = get(mu, min(ib, 2));
-    const double c = (solve ? m[4 + min(r, 5)] : 0.0) / (solve ? A : 1.0) - mx * my;
+    const double c = cov_entry(solve ? m[4 + min(r, 5)] : 0.0, solve ? A : 1.0, mx, my);
     double M[3];
     {
         const double xx = get(c, 0), yy = get(c, 1), zz = get(c, 2), xy = get(c, 3), xz = get(c, 4), yz = get(c, 5);
@@ -1537,25 +1578,22 @@ __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ 
     for (int i = 0; i < 3; ++i)
         for (int j = 0; j < 3; ++j) {
             const double x = get(M[j], i);
-            fro += x * x;
+            fro = __fma_rn(x, x, fro);
         }
     for (int sweep = 0; sweep < 16; ++sweep) {
         const double a01 = get(M[1], 0), a02 = get(M[2], 0), a12 = get(M[2], 1);
-        const double off = 2.0 * (a01 * a01 + a02 * a02 + a12 * a12);
-        const bool go = solve && !(off <= 1e-30 * fro);
+        const bool go = solve && !(off_diagonal(a01, a02, a12) <= __dmul_rn(1e-30, fro));
         if (!__any_sync(kAll, go)) break;
 #pragma unroll
         for (int rot = 0; rot < 3; ++rot) {
             const int p = rot == 2 ? 1 : 0, qq = rot == 0 ? 1 : 2;
             const double apq = get(M[qq], p), app = get(M[p], p), aqq = get(M[qq], qq);
             const bool turn = go && apq != 0.0;
-            const double theta = (aqq - app) / (2.0 * apq);
-            const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            const double cs = 1.0 / sqrt(t * t + 1.0);
-            const double sn = t * cs;
+            const JacobiTurn turn_by = jacobi_turn(app, aqq, apq);
+            const double cs = turn_by.c, sn = turn_by.s;
             // columns p and q of the lane's row
             const double x = M[p], y = M[qq];
-            const double xn = __fma_rn(cs, x, -__dmul_rn(sn, y)), yn = __fma_rn(sn, x, __dmul_rn(cs, y));
+            const double xn = mul_sub(cs, x, sn, y), yn = mul_add(sn, x, cs, y);
             if (turn) {
                 M[p] = xn;
                 M[qq] = yn;
@@ -1564,11 +1602,10 @@ __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ 
             const int other = r == p ? qq : r == qq ? p : r;
             double o[3];
             for (int j = 0; j < 3; ++j) o[j] = get(M[j], other);
-            // row p: c row_p - s row_q; row q: s row_p + c row_q
+            // row p: c row_p - s row_q; row q: s row_p + c row_q (a product's sign does not change its rounding)
             for (int j = 0; j < 3; ++j) {
                 const double rp = r == p ? M[j] : o[j], rq = r == p ? o[j] : M[j];
-                const double u = r == p ? cs : sn, w = r == p ? -sn : cs;
-                const double v = __fma_rn(u, rp, __dmul_rn(w, rq));
+                const double v = mul_add(r == p ? cs : sn, rp, r == p ? -sn : cs, rq);
                 if (turn && (r == p || r == qq)) M[j] = v;
             }
         }
@@ -1592,9 +1629,7 @@ __global__ void __launch_bounds__(32) k_frames_lanes(const double* __restrict__ 
             if (fabs(row[b]) > fabs(big)) big = row[b];
         for (int b = 0; b < 3; ++b) R[3 * a + b] = big < 0.0 ? -row[b] : row[b];
     }
-    R[6] = R[1] * R[5] - R[2] * R[4];
-    R[7] = R[2] * R[3] - R[0] * R[5];
-    R[8] = R[0] * R[4] - R[1] * R[3];
+    third_row(R);
     if (!on) return;
     for (int i = r; i < 9; i += kFrameLanes) {
         double x = R[0];
