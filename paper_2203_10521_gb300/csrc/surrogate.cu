@@ -385,14 +385,13 @@ __global__ void __launch_bounds__(kTcRows) k_mlp_tc(const float* __restrict__ X,
     const uint32_t aS = smem_addr(sA), bS = smem_addr(sB), cS = smem_addr(sC);
     const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);   // this warp's 32 TMEM lanes
     const __half* w2 = wtc + kChunks * kTcW1Chunk;
-    uint32_t mma = 0, ld[2] = {0, 0}, wl = 0;   // groups committed and copies issued per barrier, the same in every thread
+    uint32_t mma = 0;           // groups committed, the same in every thread
+    uint32_t loads = 1;         // thread 0: copies of W1 chunks and W3 issued, in turn on bar_ld[0] and bar_ld[1]
     bool ok = true;
     if (t == 0) {
         tc_bulk_load(sB, wtc, (uint32_t)(kTcW1Chunk * 2), &bar_ld[0]);
         tc_bulk_load(sC, w2, (uint32_t)(kH * kH * 2), &bar_w);
     }
-    ld[0] = 1;
-    wl = 1;
 
     // Layer 1, chunk q: its features into A half q & 1 (free: the MMAs of
     // chunk q - 2 were waited for), the next features on their way, W1 chunk
@@ -405,11 +404,10 @@ __global__ void __launch_bounds__(kTcRows) k_mlp_tc(const float* __restrict__ X,
         if (q + 1 < kChunks) load_x(q + 1);
         bool got = true;
         if (q > 0) got = tc_wait(&bar_mma, (mma - 1) & 1);   // the MMAs of chunk q - 1
-        if (q + 1 < kChunks) {
-            if (t == 0 && got)
-                tc_bulk_load(sB + (half ^ 1) * kHalf, wtc + (q + 1) * kTcW1Chunk, (uint32_t)(kTcW1Chunk * 2),
-                             &bar_ld[half ^ 1]);
-            ++ld[half ^ 1];
+        if (q + 1 < kChunks && t == 0 && got) {
+            tc_bulk_load(sB + (half ^ 1) * kHalf, wtc + (q + 1) * kTcW1Chunk, (uint32_t)(kTcW1Chunk * 2),
+                         &bar_ld[half ^ 1]);
+            ++loads;
         }
         got = got && tc_wait(&bar_ld[half], (q >> 1) & 1);
         tc_fence_before();
@@ -431,9 +429,9 @@ __global__ void __launch_bounds__(kTcRows) k_mlp_tc(const float* __restrict__ X,
     // becomes FP16 h in the A tile; W2 is there, W3 arrives meanwhile in the
     // place of the W1 chunks
     for (int layer = 0; layer < 2 && ok; ++layer) {
-        if (layer == 0) {
-            if (t == 0) tc_bulk_load(sB, w2 + kH * kH, (uint32_t)(kH * kH * 2), &bar_ld[0]);
-            ++ld[0];
+        if (layer == 0 && t == 0) {
+            tc_bulk_load(sB, w2 + kH * kH, (uint32_t)(kH * kH * 2), &bar_ld[kChunks & 1]);
+            ++loads;
         }
         tc_fence_after();
         for (int c = 0; c < kH / 32; ++c) {
@@ -448,7 +446,7 @@ __global__ void __launch_bounds__(kTcRows) k_mlp_tc(const float* __restrict__ X,
             }
         }
         tc_fence_smem();
-        const bool got = layer == 0 ? tc_wait(&bar_w, 0) : tc_wait(&bar_ld[0], (ld[0] - 1) & 1);
+        const bool got = layer == 0 ? tc_wait(&bar_w, 0) : tc_wait(&bar_ld[kChunks & 1], (kChunks >> 1) & 1);
         tc_fence_before();
         ok = __syncthreads_and(got);
         if (!ok) break;
@@ -478,13 +476,15 @@ __global__ void __launch_bounds__(kTcRows) k_mlp_tc(const float* __restrict__ X,
         const int m = m0 + t;
         if (m < M) y[m] = 1.f / (1.f + __expf(-acc));
     } else {
-        // a wait gave up: report it, let in-flight tensor-core work and copies
-        // finish (bounded), then free TMEM below
-        if (t == 0) atomicOr(err, kErrTimeout);
-        if (mma > 0 && !stall) tc_wait(&bar_mma, (mma - 1) & 1);
-        for (int h = 0; h < 2; ++h)
-            if (ld[h] > 0) tc_wait(&bar_ld[h], (ld[h] - 1) & 1);
-        if (wl > 0) tc_wait(&bar_w, (wl - 1) & 1);
+        // a wait gave up: thread 0, which issued everything, reports it and
+        // lets its tensor-core work and copies in flight finish (bounded);
+        // TMEM is freed below
+        if (t == 0) {
+            atomicOr(err, kErrTimeout);
+            if (mma > 0 && !stall) tc_wait(&bar_mma, (mma - 1) & 1);
+            for (uint32_t i = loads > 1 ? loads - 2 : 0; i < loads; ++i) tc_wait(&bar_ld[i & 1], (i >> 1) & 1);
+            tc_wait(&bar_w, 0);
+        }
     }
     tc_fence_before();
     __syncthreads();
