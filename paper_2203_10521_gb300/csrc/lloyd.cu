@@ -1290,8 +1290,7 @@ template <int NT, bool kComp = true, bool kDeep = false>
 __global__ void __launch_bounds__(NT) k_moments(const float* __restrict__ V, const int32_t* __restrict__ F,
                                                 const int32_t* __restrict__ members,
                                                 const int32_t* __restrict__ start,
-                                                const LatticeFrame* __restrict__ f, double* __restrict__ mom,
-                                                const uint8_t* __restrict__ dirty)
+                                                double* __restrict__ mom, const uint8_t* __restrict__ dirty)
 {
     const int32_t k = blockIdx.x;
     if (dirty && !dirty[k]) return;
@@ -1656,8 +1655,8 @@ static void launch_moments(obb_ctx* ctx, const obb_layer* L, double* mom, const 
 {
     const obb_lattice* lat = L->lat;
     const auto run = [&](auto kernel) {
-        kernel<<<L->K, kNT, 0, ctx->stream>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start,
-                                              lat->d_frame, mom, dirty);
+        kernel<<<L->K, kNT, 0, ctx->stream>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start, mom,
+                                              dirty);
     };
     // four members a thread and more on average
     if (L->T > (int64_t)4 * kNT * L->K) run(k_moments<kNT, true, true>);
@@ -3476,13 +3475,13 @@ obb_status layer_moments(obb_ctx* ctx, obb_layer* L, int32_t compensated, double
     const obb_lattice* lat = L->lat;
     double* d = nullptr;
     OBB_CK(ctx, pool_alloc((void**)&d, sizeof(double) * 10 * L->K, s));
-    if (compensated)
-        k_moments<kNT, true><<<L->K, kNT, 0, s>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start,
-                                                  lat->d_frame, d, nullptr);
-    else
-        k_moments<kNT, false><<<L->K, kNT, 0, s>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start,
-                                                   lat->d_frame, d, nullptr);
-    note_launch(ctx);
+    if (compensated) {
+        launch_moments(ctx, L, d, nullptr);
+    } else {
+        k_moments<kNT, false><<<L->K, kNT, 0, s>>>(lat->mesh->d_verts, lat->mesh->d_tris, L->d_members, L->d_start, d,
+                                                   nullptr);
+        note_launch(ctx);
+    }
     OBB_CK(ctx, cudaGetLastError());
     OBB_CK(ctx, cudaMemcpyAsync(out, d, sizeof(double) * 10 * L->K, cudaMemcpyDeviceToHost, s));
     cudaFreeAsync(d, s);
