@@ -400,8 +400,8 @@ __global__ void k_fl_centres(const LatticeFrame* __restrict__ f, const double* _
 // cluster of blocks takes its group through that order (k_fl_run), counting
 // the boxes that a triangle would grow on the way.  A wave per launch instead
 // takes eight launches and two round trips to the host for one triangle of
-// each group (10k triangles, 16 groups: 623 waves, 46.7 ms a call; this way 3.3 ms:
-// 0.38 ms for the orders, 3.8 us a triangle after that, mostly the latency of
+// each group (10k triangles, 16 groups: 623 waves, 46.7 ms a call; this way 2.7 ms:
+// 0.38 ms for the orders, 3.0 us a triangle after that, mostly the latency of
 // preparing and counting one or two grown boxes).
 //
 // A group's triangles are numbered locally (base[g] + 0, 1, ..., by its old
@@ -870,6 +870,14 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     const int64_t T = L->T;
     if (mode != 0 && mode != 1) return fail(ctx, OBB_ERR_ARG, "flood mode must be 0 (exact) or 1 (wavefront)");
     OBB_TRY(layer_members(ctx, L));
+    // With profiling counters (mode 1) the counting kernel's own launches, a wave at a time; and where the boxes are large
+    // for the number of triangles: a group's cluster counts them with eight blocks, a wave with all of the machine.  A
+    // run's counts grow with the boxes that grow (about the root of the triangles) and with N^3 of the points they
+    // hold, the waves with the triangles: N^3 <= 6 10^7 sqrt(T).  Run against waves, ms: 144 triangles 2.6 : 4.7 at 512^3,
+    // 10.4 : 5.4 at 1024^3; 1,920 triangles 50 : 113 at 1024^3, 122 : 116 at 1448^3, 282 : 121 at 2048^3; 24,000 at 2048^3
+    // 1,296 : 1,583.
+    const double side = (double)lat->frame.N;
+    const bool run = mode == 0 && ctx->prof != 1 && side * side * side <= 6e7 * std::sqrt((double)T);
     FloodMem mem;
     mem.ctx = ctx;
     // exact mode takes at most one triangle per group and wave; the wavefront
@@ -885,15 +893,24 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     int32_t* gfill = mem.get<int32_t>(K);
     int32_t* gbox = mem.get<int32_t>(K);
     int32_t* seed = mem.get<int32_t>(K);
-    unsigned long long* gbest = mem.get<unsigned long long>(K);
-    unsigned long long* gfall = mem.get<unsigned long long>(K);
     double* centre = mem.get<double>(3 * (size_t)K);
-    FloodRec* rec = mem.get<FloodRec>(rec_cap);
-    obb_qbox* evals = mem.get<obb_qbox>(eval_cap);
-    uint64_t* ecount = mem.get<uint64_t>(eval_cap);
-    uint8_t* changed = mem.get<uint8_t>(K);
-    int32_t* map = mem.get<int32_t>(K);
     int32_t* ctr = mem.get<int32_t>(4);   // records, evals, unassigned, recount size
+    // the waves' own
+    unsigned long long *gbest = nullptr, *gfall = nullptr;
+    FloodRec* rec = nullptr;
+    obb_qbox* evals = nullptr;
+    uint64_t* ecount = nullptr;
+    uint8_t* changed = nullptr;
+    int32_t* map = nullptr;
+    if (!run) {
+        gbest = mem.get<unsigned long long>(K);
+        gfall = mem.get<unsigned long long>(K);
+        rec = mem.get<FloodRec>(rec_cap);
+        evals = mem.get<obb_qbox>(eval_cap);
+        ecount = mem.get<uint64_t>(eval_cap);
+        changed = mem.get<uint8_t>(K);
+        map = mem.get<int32_t>(K);
+    }
     if (mem.e != cudaSuccess) return cuda_fail(ctx, mem.e, "flood scratch");
     const unsigned gT = (unsigned)((T + 255) / 256), gK = (unsigned)((K + 127) / 128);
     if (d_centres) OBB_CK(ctx, cudaMemcpyAsync(centre, d_centres, sizeof(double) * 3 * K, cudaMemcpyDefault, s));
@@ -904,7 +921,7 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     k_fl_group<<<gT, 256, 0, s>>>(L->d_assign, L->d_parent, T, group, nassign);
     OBB_CK(ctx, cudaMemsetAsync(gcount, 0, sizeof(int32_t) * K, s));
     OBB_CK(ctx, cudaMemsetAsync(gfill, 0, sizeof(int32_t) * K, s));
-    OBB_CK(ctx, cudaMemsetAsync(changed, 0, K, s));
+    if (!run) OBB_CK(ctx, cudaMemsetAsync(changed, 0, K, s));
     k_fl_box_count<<<gK, 128, 0, s>>>(L->d_parent, K, gcount, ctx->d_err);
     note_launch(ctx, 2);
     OBB_TRY(set_device_int(ctx, ctr + 3, K));
@@ -926,14 +943,6 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     OBB_TRY(set_device_int(ctx, ctr + 2, (int32_t)(T - K)));
     obb_flood_stats st{};
     int64_t evals_total = 0;
-    // With profiling counters (mode 1) the counting kernel's own launches, a wave at a time; and where the boxes are large
-    // for the number of triangles: a group's cluster counts them with eight blocks, a wave with all of the machine.  A
-    // run's counts grow with the boxes that grow (about the root of the triangles) and with N^3 of the points they
-    // hold, the waves with the triangles: N^3 <= 6 10^7 sqrt(T).  Run against waves, ms: 144 triangles 2.6 : 4.7 at 512^3,
-    // 10.4 : 5.4 at 1024^3; 1,920 triangles 50 : 113 at 1024^3, 122 : 116 at 1448^3, 282 : 121 at 2048^3; 24,000 at 2048^3
-    // 1,296 : 1,583.
-    const double side = (double)lat->frame.N;
-    const bool run = mode == 0 && ctx->prof != 1 && side * side * side <= 6e7 * std::sqrt((double)T);
     if (run) OBB_TRY(flood_exact(ctx, L, mem, group, gstart, gbox, key, nassign, &st.waves, &evals_total));
     while (!run) {
         OBB_CK(ctx, cudaMemcpyAsync(hi, ctr + 2, sizeof(int32_t), cudaMemcpyDeviceToHost, s));

@@ -812,10 +812,10 @@ __global__ void k_sum_points(const uint64_t* __restrict__ pts, const int32_t* __
 // order.  A pair that accepts nothing has settled: its further rounds would
 // count the same boxes again (k_pair_finish adds them to the step's counters,
 // which cover every round of every pair).  Round by round the layer takes 13
-// launches and a round trip to the host each, all pairs in every round: three
-// iterations of 200k triangles in 1,024 clusters 3.3 ms a call, this way 1.3;
-// six with rotation descent of 2M in 16,384 clusters 13.9 and 11.1 ms (1.1 and
-// 8.2 since the boxes' preparation, the counts and the box update got cheaper).
+// launches each, and a round trip to the host unless it is captured, all pairs
+// in every round: three host-driven steps of 200k triangles in 1,024 clusters
+// 2.49 ms, this way 0.87; six captured ones with rotation descent of 2M in
+// 16,384 clusters 12.0 and 7.9 ms.
 constexpr int kPairEvals = 24;      // 12 sides, a shrunk and a grown box each (prepared by three warps, eight each)
 constexpr int kPairMoves = 64;      // most rounds of a step that take this path
 // A captured iteration takes the pairs' rounds from this many pairs on, or with clusters beyond kPairGraphSize triangles
@@ -854,7 +854,7 @@ struct PairArgs {
     uint8_t* dirty;
     int64_t* stats;
     obb_qbox* evals;        // the last round's boxes and counts of every pair
-    uint64_t *ecount, *epoints;
+    uint64_t* ecount;
     int4* info;             // per pair: rounds run, boxes of its last round, their points (two words)
     const LatRef* lats;
     CountOpts o;
@@ -2478,7 +2478,6 @@ static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
     a.stats = L->d_stats;
     a.evals = M->evals;
     a.ecount = M->ecount;
-    a.epoints = M->epoints;
     a.info = M->pinfo;
     a.lats = lat->d_ref;
     a.o = CountOpts{ctx->tile_k, ctx->count_axis, ctx->count_rank};
