@@ -835,12 +835,13 @@ constexpr int64_t kPairGraphSize = 4096;
 constexpr int64_t kPairRows = 65536, kPairTriRows = 32;
 
 // A layer whose last step moved nothing most likely runs one round, where all pairs take part and the pairs' rounds have
-// nothing to leave out: a pair's round is one long chain of dependent work, and from a few hundred pairs on large
-// lattices the layer's kernels, which spread the same work evenly, are through it sooner.  A settled step by pairs and
-// by the layer, us, captured | host-driven: 8,192 pairs at 1024^3 387, 179 | 391, 229; 512 pairs 209, 114 | 210, 154; 128
-// pairs at 715^3 150, 106 | 153, 116; but 128 pairs at 495^3 100, 102 | 98, 113, 256 at 256^3 75, 100 | 95, 135.  The
-// first steps of a layer go the other way (11 rounds of 8,192 pairs 1,521, 2,438 | 1,454, 3,010).
-constexpr int kSettledPairs = 128;
+// nothing to leave out: a pair's round is one long chain of dependent work, and on large lattices the layer's kernels,
+// which spread the same work evenly, are through it sooner unless they walk large clusters with one block each
+// (kPairGraphSize again).  A settled step by pairs and by the layer, us, captured | host-driven: 8,192 pairs at 1024^3
+// 387, 179 | 391, 229; 512 pairs 209, 114 | 210, 154; 128 pairs at 715^3 150, 106 | 153, 116; but 128 pairs at 495^3 100,
+// 102 | 98, 113, 256 at 256^3 75, 100 | 95, 135.  The first steps of a layer go the other way (11 rounds of 8,192 pairs
+// 1,521, 2,438 | 1,454, 3,010).  Over 1,148 settled layers (1 to 4,096 pairs, even and uneven, 64^3 to 1600^3) the
+// mean loss by this line is 5 % against the faster side, 17 % without it.
 constexpr int64_t kSettledSide = 512;
 // A second graph costs about what one or two settled steps gain by it.
 constexpr int kSettledHost = 1, kSettledGraph = 2;
@@ -2442,7 +2443,7 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled,
     if (ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
     const int64_t N = L->lat->frame.N;
     if (N * N > kPairRows * (L->K / 2) + kPairTriRows * L->T) return OBB_OK;
-    if (M->settled >= settled && L->K / 2 >= kSettledPairs && N > kSettledSide) return OBB_OK;
+    if (M->settled >= settled && N > kSettledSide && L->T <= kPairGraphSize * L->K) return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
