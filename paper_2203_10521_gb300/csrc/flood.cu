@@ -937,7 +937,7 @@ obb_status flood_partition(obb_ctx* ctx, obb_layer* L, const double* d_centres, 
     k_fl_seed_bounds<<<gK, 128, 0, s>>>(lat->d_fixed, mesh->d_tris, seed, K, L->d_q);
     note_launch(ctx, 2);
     OBB_TRY(check_device_error(ctx));
-    OBB_TRY(count_boxes(ctx, lat, L->d_q, layer_dev_K(L), K, L->d_obv, nullptr));
+    OBB_TRY(count_known(ctx, lat, L->d_q, K, L->d_obv, nullptr));
     int64_t* h = host_stats(ctx);
     int32_t* hi = reinterpret_cast<int32_t*>(h);
     OBB_TRY(set_device_int(ctx, ctr + 2, (int32_t)(T - K)));

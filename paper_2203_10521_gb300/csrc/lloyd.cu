@@ -2408,7 +2408,7 @@ static obb_status init_boxes(obb_ctx* ctx, obb_layer* L, const double* d_frames,
     launch_tight(ctx, L, L->d_q, 1, nullptr, s);
     note_launch(ctx);
     OBB_CK(ctx, cudaGetLastError());
-    return count_boxes(ctx, lat, L->d_q, M->dK, K, L->d_obv, nullptr);
+    return count_known(ctx, lat, L->d_q, K, L->d_obv, nullptr);
 }
 
 // Looks whether the layer's clusters are sibling pairs; the answer is on the

@@ -622,7 +622,7 @@ __device__ __forceinline__ void quantize_warp(const obb_box& B, const LatticeFra
     if (lane == 12) out->reserved = 0;
 }
 
-// A few boxes (at most kFewMaxBoxes) in one launch: a cluster of kFewCluster
+// A few boxes in one launch: a cluster of kFewCluster
 // blocks per box prepares it and counts its tiles, dealt out over the
 // cluster's warps.  Such a call is latency: of the general path's six launches
 // (box count, quantisation, preparation, two for the tile offsets, counting)
@@ -634,14 +634,17 @@ __device__ __forceinline__ void quantize_warp(const obb_box& B, const LatticeFra
 
 constexpr int kFewThreads = 256;
 
-// The one-launch path takes at most kFewMaxBoxes boxes (their cap: how many
-// there are may only be known on the device) on lattices of at most
-// kFewMaxLatticeBytes (256^3), boxes times lattice bytes at most kFewMaxWork: a
+// The one-launch path takes at most kFewMaxBoxes boxes, or kFewMaxCap where how
+// many of a cap there are is only known on the device (most calls use little of
+// their cap): eight blocks a box are a wave of blocks for every 38 boxes, and
+// from about 100 on two launches are as fast (16 boxes 10 against 16 us, 64 16
+// against 19, 96 17 and 20, 128 23 and 18, 256 40 and 20, 400 55 and 24; 64^3).
+// Lattices of at most kFewMaxLatticeBytes (256^3), boxes times lattice bytes at most kFewMaxWork: a
 // cluster per box cannot share a large box out over the whole machine as the
 // general path's tile queue does (31 boxes of a tree's top levels at 1024^3: 267
 // against 106 us; 255 boxes at 544^3: 134 against 84 us; seven at 340^3: 60
 // against 73 us).  Profiling with counters (mode 1) needs the general path's.
-constexpr int64_t kFewMaxBoxes = 512;
+constexpr int64_t kFewMaxBoxes = 96, kFewMaxCap = 256;
 constexpr int64_t kFewMaxLatticeBytes = int64_t(2) << 20;
 constexpr int64_t kFewMaxWork = int64_t(64) << 20;
 constexpr int kFewCluster = 8;   // blocks per box (4: 12.8, 8: 9.6 us for the 16 to 32 boxes of a flooding wave)
@@ -818,9 +821,9 @@ constexpr int64_t kPrepScanBoxes = 4096;
 // warps of the counting kernel's grid (four blocks of 256 threads on an SM)
 static int32_t count_grid_warps(const obb_ctx* ctx) { return 32 * ctx->num_sms; }
 
-static bool few_boxes(const obb_ctx* ctx, int64_t K_cap, int64_t lattice_bytes)
+static bool few_boxes(const obb_ctx* ctx, const int32_t* d_K, int64_t K_cap, int64_t lattice_bytes)
 {
-    return ctx->prof != 1 && K_cap <= kFewMaxBoxes && lattice_bytes <= kFewMaxLatticeBytes &&
+    return ctx->prof != 1 && K_cap <= (d_K ? kFewMaxCap : kFewMaxBoxes) && lattice_bytes <= kFewMaxLatticeBytes &&
            K_cap * lattice_bytes <= kFewMaxWork;
 }
 
@@ -864,7 +867,7 @@ static obb_status launch_few(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
 obb_status count_float_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box* d_boxes, int64_t K,
                              uint64_t* d_counts, uint64_t* d_points)
 {
-    if (few_boxes(ctx, K, (int64_t)lat->n_words * 8))
+    if (few_boxes(ctx, nullptr, K, (int64_t)lat->n_words * 8))
         return launch_few(ctx, lat->d_ref, 1, nullptr, nullptr, d_boxes, lat->d_frame, nullptr, K, d_counts, d_points,
                           ctx->d_prof + 2);
     return count_boxes_multi(ctx, lat->d_ref, 1, nullptr, nullptr, nullptr, K, d_counts, d_points,
@@ -874,7 +877,7 @@ obb_status count_float_boxes(obb_ctx* ctx, const obb_lattice* lat, const obb_box
 obb_status count_known(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* d_boxes, int64_t K, uint64_t* d_counts,
                        uint64_t* d_points)
 {
-    if (few_boxes(ctx, K, (int64_t)lat->n_words * 8))
+    if (few_boxes(ctx, nullptr, K, (int64_t)lat->n_words * 8))
         return launch_few(ctx, lat->d_ref, 1, nullptr, d_boxes, nullptr, nullptr, nullptr, K, d_counts, d_points,
                           ctx->d_prof + 2);
     return count_boxes_multi(ctx, lat->d_ref, 1, nullptr, d_boxes, nullptr, K, d_counts, d_points,
@@ -901,7 +904,7 @@ obb_status count_boxes_multi(obb_ctx* ctx, const LatRef* d_lats, int32_t n_lats,
     cudaStream_t s = ctx->stream;
     if (K_cap <= 0) return OBB_OK;
     if (K_cap > (int64_t(1) << 30)) return fail(ctx, OBB_ERR_RANGE, "too many boxes in one call");
-    if (few_boxes(ctx, K_cap, lattice_bytes))
+    if (few_boxes(ctx, d_K, K_cap, lattice_bytes))
         return launch_few(ctx, d_lats, n_lats, d_lat_of_box, d_boxes, d_fboxes, d_frame, d_K, K_cap, d_counts,
                           d_points, ctx->d_prof + 2);
     BoxPrep* prep;

@@ -500,9 +500,6 @@ obb_status obb_tune_counting(obb_ctx* ctx, const obb_lattice* lat, const obb_qbo
     const obb_qbox* db;
     OBB_TRY(to_device(ctx, qboxes, (size_t)K, on_device, hb, &db));
     OBB_CK(ctx, ctx->cscratch.reserve(sizeof(uint64_t) * K, s));
-    OBB_CK(ctx, ctx->kdev.reserve(sizeof(int32_t), s));
-    int32_t* dK = ctx->kdev.as<int32_t>();
-    OBB_TRY(set_device_int(ctx, dK, (int32_t)K));
     const int32_t cand[4] = {8, 16, 32, 64};
     float t[4] = {0, 0, 0, 0};
     cudaEvent_t e0, e1;
@@ -513,11 +510,11 @@ obb_status obb_tune_counting(obb_ctx* ctx, const obb_lattice* lat, const obb_qbo
     obb_status rc = OBB_OK;
     for (int i = 0; i < 4 && rc == OBB_OK; ++i) {
         ctx->tile_k = cand[i];
-        rc = count_boxes(ctx, lat, db, dK, K, ctx->cscratch.as<uint64_t>(), nullptr);   // warm-up
+        rc = count_known(ctx, lat, db, K, ctx->cscratch.as<uint64_t>(), nullptr);   // warm-up
         if (rc != OBB_OK) break;
         cudaEventRecord(e0, s);
         for (int r = 0; r < 3 && rc == OBB_OK; ++r)
-            rc = count_boxes(ctx, lat, db, dK, K, ctx->cscratch.as<uint64_t>(), nullptr);
+            rc = count_known(ctx, lat, db, K, ctx->cscratch.as<uint64_t>(), nullptr);
         cudaEventRecord(e1, s);
         const cudaError_t ee = cudaEventSynchronize(e1);
         if (ee != cudaSuccess) rc = cuda_fail(ctx, ee, "autotune timing");
