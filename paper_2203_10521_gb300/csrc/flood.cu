@@ -408,17 +408,35 @@ __global__ void k_fl_centres(const LatticeFrame* __restrict__ f, const double* _
 // clusters), with their neighbours, vertices and assignment side by side, so
 // that its cluster works out of L1 and L2.
 
+struct FloodTotals {
+    unsigned long long evals;
+    int32_t groups, longest;   // groups that have triangles left; the most that any has after its seeds
+};
+
 // nonempty groups, and every group's number of triangles
 __global__ void k_fl_sizes(const int32_t* __restrict__ gstart, const int32_t* __restrict__ gbox,
                            const int32_t* __restrict__ mstart, int32_t K, int32_t* __restrict__ gsize,
-                           int32_t* __restrict__ glist, int32_t* __restrict__ ngroups)
+                           int32_t* __restrict__ glist, FloodTotals* __restrict__ tot)
 {
     const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= K) return;
     int32_t n = 0;
     for (int32_t i = gstart[g]; i < gstart[g + 1]; ++i) n += mstart[gbox[i] + 1] - mstart[gbox[i]];
     gsize[g] = n;
-    if (n > 0) glist[atomicAdd(ngroups, 1)] = g;
+    if (n > 0) {
+        glist[atomicAdd(&tot->groups, 1)] = g;
+        atomicMax(&tot->longest, n - (gstart[g + 1] - gstart[g]));
+    }
+}
+
+// the groups whose order is not at its end (tot->groups zeroed before)
+__global__ void k_fl_unfinished(const int32_t* __restrict__ gstart, const int32_t* __restrict__ base,
+                                const int32_t* __restrict__ done, int32_t K, int32_t* __restrict__ glist,
+                                FloodTotals* __restrict__ tot)
+{
+    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < K && base[g + 1] - base[g] - (gstart[g + 1] - gstart[g]) > done[g])
+        glist[atomicAdd(&tot->groups, 1)] = g;
 }
 
 // local numbers: block per group
@@ -469,6 +487,11 @@ __global__ void k_fl_local(const int32_t* __restrict__ U, const int32_t* __restr
 // triangles a launch takes from each group: 40 ms at 1024^3, a quarter of a second at worst (24,000 triangles in one
 // group of two boxes that fill 2048^3)
 constexpr int32_t kRunSteps = 4096;
+// ... and the first launch of uneven groups (the longest more than twice the average) too many for eight blocks each,
+// twice as many in every one after it: the blocks of groups that end sooner go to the others (24,000 triangles at
+// 400^3, 125 groups of which the longest has 4,800: 615 -> 244 ms; groups of like size only wait for one another then,
+// 10.1 -> 10.6 ms)
+constexpr int32_t kRunFirst = 128;
 
 // The order of a group's triangles after its seeds, a warp per group: the
 // smallest priority among the available triangles (a list in the group's
@@ -580,15 +603,13 @@ struct FloodBox {
 // the whole cluster prepares and counts the grown boxes (a warp prepares a box,
 // the tiles are dealt out over the cluster's warps, the sums meet in the
 // first block's shared memory) and the walker chooses.  done[g] triangles of
-// the order are behind on entry and updated on exit; *left = the most any
-// group has still before it.
+// the order are behind on entry, at most `steps` more on exit.
 __global__ void __launch_bounds__(kRunThreads) k_fl_run(
     const int32_t* __restrict__ glist, const int32_t* __restrict__ base, const int32_t* __restrict__ gstart,
     const int32_t* __restrict__ gbox, const int32_t* __restrict__ order, const int32_t* __restrict__ ladj,
     const int32_t* __restrict__ lvert, int8_t* lbox, const LatRef* __restrict__ lats, const CountOpts o, int32_t C,
-    obb_qbox* __restrict__ q, uint64_t* __restrict__ obv, int32_t* __restrict__ done,
-    unsigned long long* __restrict__ evals, int32_t* __restrict__ left, int32_t* __restrict__ longest,
-    unsigned long long* __restrict__ dom, int32_t* err)
+    int32_t steps, obb_qbox* __restrict__ q, uint64_t* __restrict__ obv, int32_t* __restrict__ done,
+    unsigned long long* __restrict__ evals, unsigned long long* __restrict__ dom, int32_t* err)
 {
     __shared__ BoxPrep prep[kMaxFloodCand];
     __shared__ obb_qbox ev[kMaxFloodCand];          // the grown boxes (the first block's are read by all)
@@ -603,7 +624,7 @@ __global__ void __launch_bounds__(kRunThreads) k_fl_run(
     const int64_t b0 = base[g];
     const int32_t nb = gstart[g + 1] - gstart[g];   // at most kMaxFloodCand (k_fl_seed checked)
     const int32_t pops = base[g + 1] - base[g] - nb;
-    const int32_t first = done[g], end = min(pops, first + kRunSteps);
+    const int32_t first = done[g], end = min(pops, first + steps);
     order += b0;
     ladj += 3 * b0;
     lvert += 9 * b0;
@@ -741,8 +762,6 @@ __global__ void __launch_bounds__(kRunThreads) k_fl_run(
         }
         if (tid == 0) {
             done[g] = step;
-            atomicMax(left, pops - step);
-            atomicMax(longest, pops);
             if (n_evals) atomicAdd(evals, n_evals);
         }
     }
@@ -803,57 +822,66 @@ obb_status flood_exact(obb_ctx* ctx, obb_layer* L, FloodMem& mem, const int32_t*
     unsigned long long* fkey = mem.get<unsigned long long>(T);
     int8_t* lbox = mem.get<int8_t>(T);
     uint8_t* state = mem.get<uint8_t>(T);
-    struct Totals {
-        unsigned long long evals;
-        int32_t groups, left, longest;
-    };
-    Totals* tot = mem.get<Totals>(1);
+    FloodTotals* tot = mem.get<FloodTotals>(1);
     if (mem.e != cudaSuccess) return cuda_fail(ctx, mem.e, "flood scratch");
     const unsigned gT = (unsigned)((T + 255) / 256), gK = (unsigned)((K + 127) / 128);
-    OBB_CK(ctx, cudaMemsetAsync(tot, 0, sizeof(Totals), s));
+    OBB_CK(ctx, cudaMemsetAsync(tot, 0, sizeof(FloodTotals), s));
     OBB_CK(ctx, cudaMemsetAsync(done, 0, sizeof(int32_t) * K, s));
     OBB_CK(ctx, cudaMemsetAsync(prog, 0, sizeof(int2) * K, s));
-    k_fl_sizes<<<gK, 128, 0, s>>>(gstart, gbox, L->d_start, K, gsize, glist, &tot->groups);
+    k_fl_sizes<<<gK, 128, 0, s>>>(gstart, gbox, L->d_start, K, gsize, glist, tot);
     launch_scan_i32(ctx, gsize, base, layer_dev_K(L));
     k_fl_number<<<K, kFT, 0, s>>>(gstart, gbox, L->d_members, L->d_start, base, ltri, lid);
     k_fl_local<<<gT, 256, 0, s>>>(lat->d_fixed, mesh->d_tris, mesh->d_adj, T, ltri, lid, group, gstart, gbox, nassign,
                                   ladj, lvert, lbox);
     note_launch(ctx, 3);
-    Totals* h = reinterpret_cast<Totals*>(host_stats(ctx));
-    OBB_CK(ctx, cudaMemcpyAsync(h, tot, sizeof(Totals), cudaMemcpyDeviceToHost, s));
-    OBB_TRY(check_device_error(ctx));
-    const int32_t groups = h->groups;
-    if (groups <= 0) return fail(ctx, OBB_ERR_STATE, "a layer without groups");
-    // blocks per group: as many as keep every group's cluster on the chip (two blocks an SM)
-    int32_t C = 8;
-    while (C > 1 && (int64_t)C * groups > 2 * ctx->num_sms) C >>= 1;
+    FloodTotals* h = reinterpret_cast<FloodTotals*>(host_stats(ctx));
+    auto read = [&]() -> obb_status {
+        OBB_CK(ctx, cudaMemcpyAsync(h, tot, sizeof(FloodTotals), cudaMemcpyDeviceToHost, s));
+        return check_device_error(ctx);
+    };
+    OBB_TRY(read());
+    if (h->groups <= 0) return fail(ctx, OBB_ERR_STATE, "a layer without groups");
+    const int32_t longest = h->longest;
+    const bool uneven = (int64_t)longest * h->groups > 2 * (T - K);
+    for (int32_t taken = 0; taken < longest; taken += kRunSteps) {
+        k_fl_order<<<h->groups, 32, 0, s>>>(glist, base, gstart, ltri, key, ladj, lbox, state, fkey, fid, order, prog);
+        note_launch(ctx);
+    }
+    OBB_CK(ctx, cudaGetLastError());
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)groups * C);
     cfg.blockDim = dim3(kRunThreads);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
     const CountOpts o{ctx->tile_k, ctx->count_axis, ctx->count_rank};
-    for (;;) {
-        k_fl_order<<<groups, 32, 0, s>>>(glist, base, gstart, ltri, key, ladj, lbox, state, fkey, fid, order, prog);
-        note_launch(ctx);
-        OBB_CK(ctx, cudaMemsetAsync(&tot->left, 0, sizeof(int32_t), s));
+    int32_t last = 0, steps = kRunSteps;
+    for (int32_t taken = 0; taken < longest;) {
+        // blocks per group: as many as keep every group's cluster on the chip (two blocks an SM)
+        int32_t C = 8;
+        while (C > 1 && (int64_t)C * h->groups > 2 * ctx->num_sms) C >>= 1;
+        steps = C == 8 || !uneven ? kRunSteps : C != last ? kRunFirst : std::min(2 * steps, kRunSteps);
+        last = C;
+        cfg.gridDim = dim3((unsigned)h->groups * C);
+        at[0].val.clusterDim.x = C;
         OBB_CK(ctx, cudaLaunchKernelEx(&cfg, k_fl_run, (const int32_t*)glist, (const int32_t*)base, gstart, gbox,
                                        (const int32_t*)order, (const int32_t*)ladj, (const int32_t*)lvert, lbox,
-                                       (const LatRef*)lat->d_ref, o, C, L->d_q, L->d_obv, done, &tot->evals, &tot->left,
-                                       &tot->longest, ctx->d_prof + 2, ctx->d_err));
+                                       (const LatRef*)lat->d_ref, o, C, steps, L->d_q, L->d_obv, done, &tot->evals,
+                                       ctx->d_prof + 2, ctx->d_err));
         note_launch(ctx);
-        OBB_CK(ctx, cudaMemcpyAsync(h, tot, sizeof(Totals), cudaMemcpyDeviceToHost, s));
-        OBB_TRY(check_device_error(ctx));
-        if (h->left <= 0) break;
+        taken += steps;   // by every group that is not at its end
+        if (taken < longest) {
+            OBB_CK(ctx, cudaMemsetAsync(&tot->groups, 0, sizeof(int32_t), s));
+            k_fl_unfinished<<<gK, 128, 0, s>>>(gstart, base, done, K, glist, tot);
+            note_launch(ctx);
+        }
+        OBB_TRY(read());
     }
     // a wave takes one triangle of every group that has any left: as many waves as the longest order has triangles
     *evals = (int64_t)h->evals;
-    *waves = h->longest;
+    *waves = longest;
     k_fl_result<<<gT, 256, 0, s>>>(ltri, group, gstart, gbox, lbox, T, nassign);
     note_launch(ctx);
     return OBB_OK;
