@@ -92,8 +92,8 @@ __device__ __forceinline__ void feature_box(const obb_qbox& q, int32_t N, Featur
     }
 }
 
-// 32 boxes a block: its first warp sets them up, a box a lane; then every
-// warp samples four of them.  Patch point s is the centre plus the edges times
+// 32 boxes a block (kFeatFew: eight): its first warp sets them up, a box a lane;
+// then every warp samples four of them (one).  Patch point s is the centre plus the edges times
 // g_a = (2 s_a - 7) / 16, ((c_r + E_r0 g_0) + E_r1 g_1) + E_r2 g_2, rounded to
 // the nearest lattice point (floor(p + 1/2)); the bit is 0 outside the
 // lattice.  A lane keeps s_0 and half of s_1, so of a sample's three sums only
@@ -101,24 +101,27 @@ __device__ __forceinline__ void feature_box(const obb_qbox& q, int32_t N, Featur
 // neighbouring columns share a line.  A block per box, one thread setting it
 // up, took 94.3 us for 32,768 boxes at 512^3; this takes 26.5 (41.1 with a
 // branch around every load; batches of 1, 2 and 8 s_2: 26.4, 26.2, 27.4),
-// 2.6 TB/s of written features.
-constexpr int kFeatBoxes = 32;
+// 2.6 TB/s of written features.  While blocks of eight boxes all fit the
+// machine at once, a warp has one box to sample instead of four in a row (300
+// boxes 10.4 -> 6.4 us, 8.4 with a block per box; 3,000 10.5 -> 10.4).
+constexpr int kFeatBoxes = 32, kFeatFew = 8;
 constexpr int kFeatThreads = 256;
 constexpr int kFeatBatch = 4;    // s_2 whose words a lane loads together
 constexpr float kFloorMagic = 12582912.0f;         // 1.5 2^23: q + it, rounded down, ends with floor(q) for |q| < 2^22
 constexpr uint32_t kFloorBits = 0x4b400000u;       // its bits
 
+template <int kBoxes>
 __global__ void __launch_bounds__(kFeatThreads) k_features(const obb_qbox* __restrict__ boxes,
                                                            const int32_t* __restrict__ d_K, int32_t K,
                                                            const uint64_t* __restrict__ cwords, int32_t N, int32_t W,
                                                            float* __restrict__ feats)
 {
-    __shared__ FeatureBox sh[kFeatBoxes];
+    __shared__ FeatureBox sh[kBoxes];
     if (d_K) K = *d_K;
-    const int64_t k0 = blockIdx.x * (int64_t)kFeatBoxes;
+    const int64_t k0 = blockIdx.x * (int64_t)kBoxes;
     if (k0 >= K) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp == 0 && k0 + lane < K) {
+    if (warp == 0 && lane < kBoxes && k0 + lane < K) {
         const obb_qbox q = boxes[k0 + lane];
         feature_box(q, N, &sh[lane]);
     }
@@ -126,7 +129,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const obb_qbox* __res
     const float g0 = __fmul_rn((float)(2 * (lane & 7) - 7), 0.0625f);
     const float g1[2] = {__fmul_rn((float)(2 * (lane >> 3) - 7), 0.0625f),
                          __fmul_rn((float)(2 * (4 + (lane >> 3)) - 7), 0.0625f)};
-    for (int i = warp; i < kFeatBoxes && k0 + i < K; i += kFeatThreads / 32) {
+    for (int i = warp; i < kBoxes && k0 + i < K; i += kFeatThreads / 32) {
         const FeatureBox& b = sh[i];
         float* f = feats + (k0 + i) * (int64_t)kIn;
         if (lane < 12) f[lane] = b.par[lane];
@@ -169,8 +172,12 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(const obb_qbox* __res
 static void launch_features(obb_ctx* ctx, const obb_lattice* lat, const obb_qbox* boxes, const int32_t* d_K, int64_t K,
                             float* feats)
 {
-    k_features<<<(unsigned)((K + kFeatBoxes - 1) / kFeatBoxes), kFeatThreads, 0, ctx->stream>>>(
-        boxes, d_K, (int32_t)K, lat->d_cwords, lat->frame.N, lat->frame.W, feats);
+    const auto run = [&](auto kernel, int per) {
+        kernel<<<(unsigned)((K + per - 1) / per), kFeatThreads, 0, ctx->stream>>>(boxes, d_K, (int32_t)K, lat->d_cwords,
+                                                                                  lat->frame.N, lat->frame.W, feats);
+    };
+    if (K <= 4 * kFeatFew * (int64_t)ctx->num_sms) run(k_features<kFeatFew>, kFeatFew);
+    else run(k_features<kFeatBoxes>, kFeatBoxes);
     note_launch(ctx);
 }
 
