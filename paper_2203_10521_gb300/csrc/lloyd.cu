@@ -41,6 +41,7 @@ constexpr int kNT = 128;   // threads of the block-per-cluster kernels
 enum { kCtrCand = 0, kCtrEval, kCtrCount };
 
 constexpr int kPairedSlot = 126;   // word of the pinned staging that check_pairs answers in
+constexpr int kCensusSlot = 124;   // words of the pinned staging that box_census answers in
 constexpr int kMaxTopk = 16;   // candidates a surrogate may keep per source cluster
 
 struct Cand {
@@ -833,6 +834,13 @@ constexpr int64_t kPairGraphSize = 4096;
 // 2,291 : 5,810 at 1024^3, 8,632 : 7,857 at 2048^3.  Over 738 layers (320 to 250,000 triangles, 1 to 256 pairs, 64^3 to
 // 2048^3) the slower side is 24 times slower; by this line the mean loss is 2 %, the largest 2.2 times.
 constexpr int64_t kPairRows = 65536, kPairTriRows = 32;
+// Boxes far larger than the layer's others, or all of them large (a partition of scattered triangles): a lane of the
+// blocks that count the largest box's rows walks its share at about 0.2 us a row, while the layer's round costs about
+// 70 us and 0.045 us (a warp a cluster; 0.0125 a block) for every triangle of its largest cluster, 1.5 times that by
+// what it adds up to over a step.  1,617 layers by both lines (median splits, uneven, a few triangles swapped, all
+// scattered): mean loss against the faster side 2.5 %, at most 2.2 times the layer's rounds; by the line above alone
+// 15 %, at most 66 times (2,048 pairs of scattered triangles at 1600^3).
+constexpr double kRowUs = 0.2, kRoundUs = 70.0, kWalkWarpUs = 0.0675, kWalkBlockUs = 0.01875;
 
 // A layer whose last step moved nothing most likely runs one round, where all pairs take part and the pairs' rounds have
 // nothing to leave out: a pair's round is one long chain of dependent work, and on large lattices the layer's kernels,
@@ -1237,6 +1245,40 @@ __global__ void k_pair_finish(const int4* __restrict__ info, int32_t pairs, int6
     if ((threadIdx.x & 31) == 0) {
         if (e) atomicAdd((unsigned long long*)&stats[kStEvals], e);
         if (n) atomicAdd((unsigned long long*)&stats[kStPoints], n);
+    }
+}
+
+// Rows that a count of the layer's largest box visits (its shadow on the (y, z) plane, as choose_axis has it) and the
+// size of its largest cluster, into out[0] and out[1] (-1 before).
+__global__ void __launch_bounds__(128) k_box_census(const obb_qbox* __restrict__ q, const int32_t* __restrict__ size,
+                                                    int32_t K, int32_t* __restrict__ out)
+{
+    const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t rows = -1, n = -1;
+    if (k < K) {
+        int64_t m[9];
+        float E[6];   // y and z components of the box's three edges
+        for (int i = 0; i < 9; ++i) m[i] = q[k].n[i];
+        const int64_t C[9] = {m[4] * m[8] - m[5] * m[7], m[2] * m[7] - m[1] * m[8], m[1] * m[5] - m[2] * m[4],
+                              m[5] * m[6] - m[3] * m[8], m[0] * m[8] - m[2] * m[6], m[2] * m[3] - m[0] * m[5],
+                              m[3] * m[7] - m[4] * m[6], m[1] * m[6] - m[0] * m[7], m[0] * m[4] - m[1] * m[3]};
+        const __int128 det = (__int128)m[0] * C[0] + (__int128)m[1] * C[3] + (__int128)m[2] * C[6];
+        const float id = 1.0f / i128_to_float(det);
+        for (int a = 0; a < 3; ++a) {
+            const float d = i64_to_float((q[k].b[2 * a + 1] >> kS) - (q[k].b[2 * a] >> kS));
+            E[a] = i64_to_float(C[3 + a]) * id * d;
+            E[3 + a] = i64_to_float(C[6 + a]) * id * d;
+        }
+        const float area = fabsf(E[0] * E[4] - E[3] * E[1]) + fabsf(E[0] * E[5] - E[3] * E[2]) +
+                           fabsf(E[1] * E[5] - E[4] * E[2]);
+        rows = area < 1e9f ? (int32_t)area : 1000000000;
+        n = size[k];
+    }
+    rows = __reduce_max_sync(0xffffffffu, rows);
+    n = __reduce_max_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n >= 0) {
+        atomicMax(&out[0], rows);
+        atomicMax(&out[1], n);
     }
 }
 
@@ -2282,6 +2324,9 @@ struct LayerMem {
     int paired = -1;
     int4* pinfo = nullptr;      // [K / 2]
     int32_t* dpaired = nullptr;
+    // the largest box's rows and the largest cluster when last looked at (box_census), -1 unknown
+    int32_t rows = -1, largest = -1;
+    int32_t* census = nullptr;
     // incremental member lists: mv [2K] the last round's leavers and joiners
     // per cluster (-1 = none), the new list and starts built beside the old
     int32_t* mv = nullptr;
@@ -2434,6 +2479,65 @@ void layer_parents_changed(obb_layer* L)
     mem_of(L)->settled = 0;
 }
 
+// Blocks of the cluster that runs a pair's rounds, and their threads.
+struct PairShape {
+    int32_t C, threads;
+};
+
+static PairShape pair_shape(const obb_ctx* ctx, const obb_layer* L)
+{
+    const int32_t pairs = L->K / 2;
+    const int64_t N = L->lat->frame.N;
+    // Threads and blocks per pair: 128 threads, eight blocks a pair while there are few (a tree's upper levels;
+    // 256 threads lengthen the chooser's serial part: 5.1 against 4.7 ms for the tree of 7k triangles at 132^3)
+    // unless the boxes are large (from 32,768 lattice rows a pair on; four pairs at 1024^3: 2.36 against 3.22 ms
+    // for four iterations), and one from 1,024 pairs on (8,192 pairs: 11.05 against 12.07 ms for six iterations);
+    // in between 256 threads, as many blocks as are resident at once (512 pairs: 1.28 against 1.43 ms for three
+    // iterations).  Clusters of sixteen blocks: no faster.
+    const bool mid = pairs >= 128 && pairs < 1024;
+    int32_t C = 8;
+    while (C > 1 && (int64_t)C * pairs > (mid ? 2 : 8) * ctx->num_sms) C >>= 1;
+    const bool big = mid || N * N >= 32768 * (int64_t)pairs;
+    return PairShape{C, big ? 256 : 128};
+}
+
+// Whether a lattice of this size can hold a box whose rows decide against the pairs' rounds.
+static bool census_matters(const obb_ctx* ctx, const obb_layer* L)
+{
+    const PairShape s = pair_shape(ctx, L);
+    const double N = L->lat->frame.N;
+    return kRowUs * 2.0 * N * N > kRoundUs * s.C * s.threads;   // a shadow is at most 1.74 N^2
+}
+
+// Looks up the largest box and cluster of the layer; the answer is on the host
+// (census_known) after the next synchronisation.
+static obb_status box_census(obb_ctx* ctx, obb_layer* L)
+{
+    LayerMem* M = mem_of(L);
+    OBB_CK(ctx, cudaMemsetAsync(M->census, 0xff, 2 * sizeof(int32_t), ctx->stream));
+    k_box_census<<<(L->K + 127) / 128, 128, 0, ctx->stream>>>(L->d_q, L->d_size, L->K, M->census);
+    note_launch(ctx);
+    OBB_CK(ctx, cudaMemcpyAsync(ctx->h_small + kCensusSlot, M->census, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                ctx->stream));
+    return OBB_OK;
+}
+
+static void census_known(obb_ctx* ctx, obb_layer* L)
+{
+    mem_of(L)->rows = ctx->h_small[kCensusSlot];
+    mem_of(L)->largest = ctx->h_small[kCensusSlot + 1];
+}
+
+// Whether the boxes, when last looked at, are small enough for the pairs' blocks.
+static bool boxes_fit_pairs(const obb_ctx* ctx, const obb_layer* L)
+{
+    const LayerMem* M = mem_of(L);
+    if (M->rows < 0) return true;
+    const PairShape s = pair_shape(ctx, L);
+    const double walk = (L->T <= (int64_t)1024 * L->K ? kWalkWarpUs : kWalkBlockUs) * M->largest;
+    return kRowUs * M->rows <= (kRoundUs + walk) * s.C * s.threads;
+}
+
 // Whether the layer's rounds run pair by pair (k_pair_rounds).  settled: steps without a move after which a large layer
 // takes its own rounds.
 static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled, bool* yes)
@@ -2446,10 +2550,13 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled,
     if (M->settled >= settled && N > kSettledSide && L->T <= kPairGraphSize * L->K) return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
+        const bool look = census_matters(ctx, L);
+        if (look) OBB_TRY(box_census(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
         pairs_known(ctx, L);
+        if (look) census_known(ctx, L);
     }
-    *yes = M->paired == 1;
+    *yes = M->paired == 1 && boxes_fit_pairs(ctx, L);
     return OBB_OK;
 }
 
@@ -2485,15 +2592,8 @@ static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
     a.rounds = rounds;
     a.dom = ctx->d_prof + 2;
     a.err = ctx->d_err;
-    // Threads and blocks per pair: 128 threads, eight blocks a pair while there are few (a tree's upper levels;
-    // 256 threads lengthen the chooser's serial part: 5.1 against 4.7 ms for the tree of 7k triangles at 132^3)
-    // unless the boxes are large (from 32,768 lattice rows a pair on; four pairs at 1024^3: 2.36 against 3.22 ms
-    // for four iterations), and one from 1,024 pairs on (8,192 pairs: 11.05 against 12.07 ms for six iterations);
-    // in between 256 threads, as many blocks as are resident at once (512 pairs: 1.28 against 1.43 ms for three
-    // iterations).  Clusters of sixteen blocks: no faster.
-    const bool mid = pairs >= 128 && pairs < 1024;
-    int32_t C = 8;
-    while (C > 1 && (int64_t)C * pairs > (mid ? 2 : 8) * ctx->num_sms) C >>= 1;
+    const PairShape shape = pair_shape(ctx, L);
+    const int32_t C = shape.C;
     a.C = C;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)pairs * C);
@@ -2504,9 +2604,8 @@ static obb_status pair_rounds(obb_ctx* ctx, obb_layer* L, int rounds)
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    const bool big = mid || (int64_t)lat->frame.N * lat->frame.N >= 32768 * (int64_t)pairs;
-    cfg.blockDim = dim3(big ? 256 : 128);
-    OBB_CK(ctx, big ? cudaLaunchKernelEx(&cfg, k_pair_rounds<256>, a) : cudaLaunchKernelEx(&cfg, k_pair_rounds<128>, a));
+    cfg.blockDim = dim3(shape.threads);
+    OBB_CK(ctx, shape.threads == 256 ? cudaLaunchKernelEx(&cfg, k_pair_rounds<256>, a) : cudaLaunchKernelEx(&cfg, k_pair_rounds<128>, a));
     k_pair_finish<<<(pairs + 255) / 256, 256, 0, s>>>(M->pinfo, pairs, L->d_stats);
     note_launch(ctx, 2);
     OBB_CK(ctx, cudaGetLastError());
@@ -2583,6 +2682,7 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     slab.add(&M->mnew, T);
     slab.add(&M->pinfo, (size_t)(K + 1) / 2);
     slab.add(&M->dpaired, 1);
+    slab.add(&M->census, 2);
     slab.add(&M->snew, (size_t)K + 1);
     cudaError_t e = slab.alloc(&M->slab, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(M->sticket, 0, sizeof(unsigned int), s);
@@ -2609,7 +2709,10 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
         if (st == OBB_OK) pairs_known(ctx, L);
     }
     if (st == OBB_OK) st = init_boxes(ctx, L, d_frames, d_fallback);
+    const bool look = st == OBB_OK && M->paired == 1 && census_matters(ctx, L);
+    if (look) st = box_census(ctx, L);
     if (st == OBB_OK) st = check_device_error(ctx);
+    if (st == OBB_OK && look) census_known(ctx, L);
     if (st != OBB_OK) {
         layer_destroy(L);
         return st;
@@ -2710,7 +2813,11 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
     }
     M->settled = before == 0 ? M->settled + 1 : 0;
     OBB_TRY(layer_box_update(ctx, L, refit_mode, dsteps));
-    return layer_finish_stats(ctx, L, ran, st);
+    const bool look = st && M->paired == 1 && !boxes_fit_pairs(ctx, L);   // until the boxes have shrunk
+    if (look) OBB_TRY(box_census(ctx, L));
+    OBB_TRY(layer_finish_stats(ctx, L, ran, st));
+    if (look) census_known(ctx, L);
+    return OBB_OK;
 }
 
 // The Lloyd iteration as one CUDA graph: the partition rounds run in a
@@ -2874,12 +2981,15 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
         G.key[3] = ctx->tile_gen;
     }
     OBB_CK(ctx, cudaGraphLaunch(G.exec, s));
+    const bool look = M->paired == 1 && !boxes_fit_pairs(ctx, L);   // until the boxes have shrunk
+    if (look) OBB_TRY(box_census(ctx, L));
     int64_t* h = host_stats(ctx);
     OBB_CK(ctx, cudaMemcpyAsync(h, L->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
     OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, M->loop, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost, s));
     OBB_TRY(check_device_error(ctx));
     M->members_valid = true;
     M->settled = h[kStAccepted] == 0 ? M->settled + 1 : 0;
+    if (look) census_known(ctx, L);
     const int64_t ran = pairs ? h[kStRounds] : h[kStCount], rebuilds = h[kStCount + 2];
     note_launch(ctx, (int)(G.round * ran + G.rebuild * rebuilds + G.post));
     if (st) {

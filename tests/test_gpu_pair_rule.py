@@ -97,3 +97,40 @@ def test_settled_large_layers_take_their_own_rounds(ctx, graph, N, level, switch
         assert np.array_equal(x[k], y[k]), k
     for z in (a, b, tree, lat, mesh):
         z.free()
+
+
+@pytest.mark.parametrize("kind,by_pairs", [("split", True), ("scattered", False), ("swapped", False)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_a_huge_box_takes_the_layer_to_its_own_rounds(ctx, kind, by_pairs, graph):
+    """The same lattice and number of pairs: compact clusters, scattered ones, and two triangles of distant clusters
+    exchanged (two boxes across the whole model)."""
+    m = M.torus(1.0, 0.3, 200, 60, jitter=0.004, seed=3)     # 24,000 triangles
+    mesh = ctx.mesh_create(m.verts, m.tris)
+    lat = ctx.build_occupancy(mesh, 640)
+    tree = ctx.build_tree(lat, 9, 0)
+    a = ctx.tree_read(tree, 9)["assign"].copy()
+    if kind == "scattered":
+        a = np.random.default_rng(1).permutation(a)
+    elif kind == "swapped":
+        c = np.asarray(m.verts)[m.tris].mean(1)
+        i = int(c.sum(1).argmin())
+        j = int(c.sum(1).argmax())           # opposite ends of the model
+        a[i], a[j] = a[j], a[i]
+    parent = (np.arange(512) // 2).astype(np.int32)
+    out = []
+    for mode in (0, 1):
+        layer = ctx.layer_init(lat, a, parent)
+        ctx.profile_enable(mode)
+        # (a captured step in mode 1 would be the same graph)
+        steps = [_step(ctx, layer, rounds=16, refit=1, graph=graph and mode == 0) for _ in range(2)]
+        ctx.profile_enable(0)
+        out.append((steps, ctx.layer_read(layer)))
+        layer.free()
+    (sa, x), (sb, y) = out
+    assert [s for s, _ in sa] == [s for s, _ in sb]
+    for k in ("assign", "qboxes", "obv", "frames"):
+        assert np.array_equal(x[k], y[k]), k
+    rounds = sa[0][0]["rounds_run"]
+    assert (sa[0][1] < 7 + 7 * rounds) == by_pairs           # a round by the layer is at least seven launches
+    for z in (tree, lat, mesh):
+        z.free()
