@@ -444,7 +444,7 @@ def lloyd_comparison(ctx, lat, tree, depth, args, flush, stream, mlp=None):
         torch.cuda.synchronize()
         lms = e0.elapsed_time(e1)
         lloyd[mode] = {"iter_per_s": 1000.0 * args.lloyd_iters / lms, "final_total_obv": int(st["total_obv"]),
-                       "exact_box_counts": int(evals)}
+                       "box_evals": int(evals)}
         lay.free()
     if "surrogate" in lloyd:
         a, b = lloyd["plain"]["final_total_obv"], lloyd["surrogate"]["final_total_obv"]

@@ -336,8 +336,10 @@ typedef struct {
     int64_t proposals;         /* over all rounds */
     int64_t moves;             /* accepted triangle moves */
     int64_t gain;              /* sum of accepted gains, lattice points */
-    int64_t box_evals;         /* exact box counts of its rounds and box update (every cluster takes part in every
-                                  round; sibling pairs that have settled keep their last counts) */
+    int64_t box_evals;         /* boxes whose exact counts its rounds and its box update used.  Every cluster takes
+                                  part in every round, so this does not depend on how the rounds are run; the counts
+                                  performed may be fewer (settled sibling pairs and boxes that did not change keep
+                                  theirs) */
     uint64_t points_counted;   /* lattice points inside those boxes */
     uint64_t total_obv;        /* sum of the layer's outer volumes after the step */
 } obb_step_stats;
