@@ -836,16 +836,17 @@ constexpr int64_t kPairGraphSize = 4096;
 constexpr int64_t kPairRows = 65536, kPairTriRows = 32;
 // Boxes far larger than the layer's others, or all of them large (a partition of scattered triangles): a lane of the
 // blocks that count the largest box's rows walks its share at about 0.2 us a row, while the layer's round costs about
-// 70 us and 0.045 us (a warp a cluster; 0.0125 a block) for every triangle of its largest cluster, 1.5 times that by
-// what it adds up to over a step.  1,617 layers by both lines (median splits, uneven, a few triangles swapped, all
-// scattered): mean loss against the faster side 2.5 %, at most 2.2 times the layer's rounds; by the line above alone
-// 15 %, at most 66 times (2,048 pairs of scattered triangles at 1600^3).
-constexpr double kRowUs = 0.2, kRoundUs = 70.0, kWalkWarpUs = 0.0675, kWalkBlockUs = 0.01875;
+// 70 us and 0.07 us (a warp a cluster; 0.02 a block) for every triangle of its largest cluster.  Twice that (kRoundUs,
+// kWalk*), since the largest box need not be counted in every round.  1,617 layers by both lines (median splits, uneven,
+// a few triangles swapped, all scattered): mean loss against the faster side 1.5 %, 1.7 %, 2.1 % and 9 %, at most 3.8
+// times the layer's rounds; by the line above alone 1.4 %, 5 %, 8 % and 38 %, at most 66 times (2,048 pairs of scattered
+// triangles at 1600^3).
+constexpr double kRowUs = 0.2, kRoundUs = 140.0, kWalkWarpUs = 0.135, kWalkBlockUs = 0.0375;
 
 // A layer whose last step moved nothing most likely runs one round, where all pairs take part and the pairs' rounds have
 // nothing to leave out: a pair's round is one long chain of dependent work, and on large lattices the layer's kernels,
-// which spread the same work evenly, are through it sooner unless they walk large clusters with one block each
-// (kPairGraphSize again).  A settled step by pairs and by the layer, us, captured | host-driven: 8,192 pairs at 1024^3
+// which spread the same work evenly, are through it sooner unless they walk large clusters with a warp or a block each
+// (kPairGraphSize again, and the largest one where it is known).  A settled step by pairs and by the layer, us, captured | host-driven: 8,192 pairs at 1024^3
 // 387, 179 | 391, 229; 512 pairs 209, 114 | 210, 154; 128 pairs at 715^3 150, 106 | 153, 116; but 128 pairs at 495^3 100,
 // 102 | 98, 113, 256 at 256^3 75, 100 | 95, 135.  The first steps of a layer go the other way (11 rounds of 8,192 pairs
 // 1,521, 2,438 | 1,454, 3,010).  Over 1,148 settled layers (1 to 4,096 pairs, even and uneven, 64^3 to 1600^3) the
@@ -2528,14 +2529,19 @@ static void census_known(obb_ctx* ctx, obb_layer* L)
     mem_of(L)->largest = ctx->h_small[kCensusSlot + 1];
 }
 
+// What the layer's rounds spend on walking its largest cluster (0 unknown), as kRoundUs has it.
+static double walk_us(const obb_layer* L)
+{
+    return (L->T <= (int64_t)1024 * L->K ? kWalkWarpUs : kWalkBlockUs) * std::max(mem_of(L)->largest, 0);
+}
+
 // Whether the boxes, when last looked at, are small enough for the pairs' blocks.
 static bool boxes_fit_pairs(const obb_ctx* ctx, const obb_layer* L)
 {
     const LayerMem* M = mem_of(L);
     if (M->rows < 0) return true;
     const PairShape s = pair_shape(ctx, L);
-    const double walk = (L->T <= (int64_t)1024 * L->K ? kWalkWarpUs : kWalkBlockUs) * M->largest;
-    return kRowUs * M->rows <= (kRoundUs + walk) * s.C * s.threads;
+    return kRowUs * M->rows <= (kRoundUs + walk_us(L)) * s.C * s.threads;
 }
 
 // Whether the layer's rounds run pair by pair (k_pair_rounds).  settled: steps without a move after which a large layer
@@ -2547,7 +2553,8 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled,
     if (ctx->count_defer || (L->mlp && L->topk > 0) || rounds > kPairMoves) return OBB_OK;
     const int64_t N = L->lat->frame.N;
     if (N * N > kPairRows * (L->K / 2) + kPairTriRows * L->T) return OBB_OK;
-    if (M->settled >= settled && N > kSettledSide && L->T <= kPairGraphSize * L->K) return OBB_OK;
+    if (M->settled >= settled && N > kSettledSide && L->T <= kPairGraphSize * L->K && walk_us(L) <= 2.0 * kRoundUs)
+        return OBB_OK;
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         const bool look = census_matters(ctx, L);

@@ -106,7 +106,7 @@ def test_a_huge_box_takes_the_layer_to_its_own_rounds(ctx, kind, by_pairs, graph
     exchanged (two boxes across the whole model)."""
     m = M.torus(1.0, 0.3, 200, 60, jitter=0.004, seed=3)     # 24,000 triangles
     mesh = ctx.mesh_create(m.verts, m.tris)
-    lat = ctx.build_occupancy(mesh, 640)
+    lat = ctx.build_occupancy(mesh, 1000)
     tree = ctx.build_tree(lat, 9, 0)
     a = ctx.tree_read(tree, 9)["assign"].copy()
     if kind == "scattered":
