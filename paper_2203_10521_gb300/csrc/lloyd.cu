@@ -41,7 +41,7 @@ constexpr int kNT = 128;   // threads of the block-per-cluster kernels
 enum { kCtrCand = 0, kCtrEval, kCtrCount };
 
 constexpr int kPairedSlot = 126;   // word of the pinned staging that check_pairs answers in
-constexpr int kCensusSlot = 124;   // words of the pinned staging that box_census answers in
+constexpr int kCensusWord = 1;     // the box census: words 1 and 2 behind the error word, on the device and in the staging
 constexpr int kMaxTopk = 16;   // candidates a surrogate may keep per source cluster
 
 struct Cand {
@@ -1250,12 +1250,12 @@ __global__ void k_pair_finish(const int4* __restrict__ info, int32_t pairs, int6
 }
 
 // Rows that a count of the layer's largest box visits (its shadow on the (y, z) plane, as choose_axis has it) and the
-// size of its largest cluster, into out[0] and out[1] (-1 before).
+// size of its largest cluster, into out[0] and out[1] (zero before).
 __global__ void __launch_bounds__(128) k_box_census(const obb_qbox* __restrict__ q, const int32_t* __restrict__ size,
                                                     int32_t K, int32_t* __restrict__ out)
 {
     const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    int32_t rows = -1, n = -1;
+    int32_t rows = 0, n = 0;
     if (k < K) {
         int64_t m[9];
         float E[6];   // y and z components of the box's three edges
@@ -1277,16 +1277,19 @@ __global__ void __launch_bounds__(128) k_box_census(const obb_qbox* __restrict__
     }
     rows = __reduce_max_sync(0xffffffffu, rows);
     n = __reduce_max_sync(0xffffffffu, n);
-    if ((threadIdx.x & 31) == 0 && n >= 0) {
+    if ((threadIdx.x & 31) == 0) {
         atomicMax(&out[0], rows);
         atomicMax(&out[1], n);
     }
 }
 
 // *paired = 0 unless clusters 2i and 2i + 1 share a parent and no others do (parents ascending by pairs)
-__global__ void k_check_pairs(const int32_t* __restrict__ parent, int32_t K, int32_t* __restrict__ paired)
+// (census: zeroed for a box census after it)
+__global__ void k_check_pairs(const int32_t* __restrict__ parent, int32_t K, int32_t* __restrict__ paired,
+                              int32_t* __restrict__ census)
 {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < 2) census[i] = 0;
     if (2 * i + 1 >= K) return;
     if (parent[2 * i] != parent[2 * i + 1] || (i > 0 && parent[2 * i - 1] >= parent[2 * i])) *paired = 0;
 }
@@ -2327,7 +2330,6 @@ struct LayerMem {
     int32_t* dpaired = nullptr;
     // the largest box's rows and the largest cluster when last looked at (box_census), -1 unknown
     int32_t rows = -1, largest = -1;
-    int32_t* census = nullptr;
     // incremental member lists: mv [2K] the last round's leavers and joiners
     // per cluster (-1 = none), the new list and starts built beside the old
     int32_t* mv = nullptr;
@@ -2466,7 +2468,8 @@ static obb_status check_pairs(obb_ctx* ctx, obb_layer* L)
     *h = 0;
     if (L->K < 2 || (L->K & 1)) return OBB_OK;
     OBB_CK(ctx, cudaMemsetAsync(M->dpaired, 0xff, sizeof(int32_t), ctx->stream));
-    k_check_pairs<<<(L->K / 2 + 127) / 128, 128, 0, ctx->stream>>>(L->d_parent, L->K, M->dpaired);
+    k_check_pairs<<<(L->K / 2 + 127) / 128, 128, 0, ctx->stream>>>(L->d_parent, L->K, M->dpaired,
+                                                                   ctx->d_err + kCensusWord);
     note_launch(ctx);
     OBB_CK(ctx, cudaMemcpyAsync(h, M->dpaired, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     return OBB_OK;
@@ -2510,23 +2513,31 @@ static bool census_matters(const obb_ctx* ctx, const obb_layer* L)
     return kRowUs * 2.0 * N * N > kRoundUs * s.C * s.threads;   // a shadow is at most 1.74 N^2
 }
 
-// Looks up the largest box and cluster of the layer; the answer is on the host
-// (census_known) after the next synchronisation.
+// Looks up the largest box and cluster of the layer after check_pairs; the
+// answer is on the host (census_known) after the next check of the error word.
 static obb_status box_census(obb_ctx* ctx, obb_layer* L)
 {
-    LayerMem* M = mem_of(L);
-    OBB_CK(ctx, cudaMemsetAsync(M->census, 0xff, 2 * sizeof(int32_t), ctx->stream));
-    k_box_census<<<(L->K + 127) / 128, 128, 0, ctx->stream>>>(L->d_q, L->d_size, L->K, M->census);
+    k_box_census<<<(L->K + 127) / 128, 128, 0, ctx->stream>>>(L->d_q, L->d_size, L->K, ctx->d_err + kCensusWord);
     note_launch(ctx);
-    OBB_CK(ctx, cudaMemcpyAsync(ctx->h_small + kCensusSlot, M->census, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                ctx->stream));
+    OBB_CK(ctx, cudaGetLastError());
+    return OBB_OK;
+}
+
+// The same without a check of either before or after it: zeroed here, on the
+// host after the next synchronisation.
+static obb_status box_census_alone(obb_ctx* ctx, obb_layer* L)
+{
+    int32_t* d = ctx->d_err + kCensusWord;
+    OBB_CK(ctx, cudaMemsetAsync(d, 0, 2 * sizeof(int32_t), ctx->stream));
+    OBB_TRY(box_census(ctx, L));
+    OBB_CK(ctx, cudaMemcpyAsync(ctx->h_small + kCensusWord, d, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     return OBB_OK;
 }
 
 static void census_known(obb_ctx* ctx, obb_layer* L)
 {
-    mem_of(L)->rows = ctx->h_small[kCensusSlot];
-    mem_of(L)->largest = ctx->h_small[kCensusSlot + 1];
+    mem_of(L)->rows = ctx->h_small[kCensusWord];
+    mem_of(L)->largest = ctx->h_small[kCensusWord + 1];
 }
 
 // What the layer's rounds spend on walking its largest cluster (0 unknown), as kRoundUs has it.
@@ -2558,7 +2569,7 @@ static obb_status pair_path(obb_ctx* ctx, obb_layer* L, int rounds, int settled,
     if (M->paired < 0) {
         OBB_TRY(check_pairs(ctx, L));
         const bool look = census_matters(ctx, L);
-        if (look) OBB_TRY(box_census(ctx, L));
+        if (look) OBB_TRY(box_census_alone(ctx, L));
         OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
         pairs_known(ctx, L);
         if (look) census_known(ctx, L);
@@ -2689,7 +2700,6 @@ obb_status layer_create(obb_ctx* ctx, const obb_lattice* lat, const int32_t* d_a
     slab.add(&M->mnew, T);
     slab.add(&M->pinfo, (size_t)(K + 1) / 2);
     slab.add(&M->dpaired, 1);
-    slab.add(&M->census, 2);
     slab.add(&M->snew, (size_t)K + 1);
     cudaError_t e = slab.alloc(&M->slab, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(M->sticket, 0, sizeof(unsigned int), s);
@@ -2821,7 +2831,7 @@ obb_status lloyd_step(obb_ctx* ctx, obb_layer* L, const obb_step_opts* opts, obb
     M->settled = before == 0 ? M->settled + 1 : 0;
     OBB_TRY(layer_box_update(ctx, L, refit_mode, dsteps));
     const bool look = st && M->paired == 1 && !boxes_fit_pairs(ctx, L);   // until the boxes have shrunk
-    if (look) OBB_TRY(box_census(ctx, L));
+    if (look) OBB_TRY(box_census_alone(ctx, L));
     OBB_TRY(layer_finish_stats(ctx, L, ran, st));
     if (look) census_known(ctx, L);
     return OBB_OK;
@@ -2989,7 +2999,7 @@ static obb_status lloyd_step_graph(obb_ctx* ctx, obb_layer* L, int rounds, int r
     }
     OBB_CK(ctx, cudaGraphLaunch(G.exec, s));
     const bool look = M->paired == 1 && !boxes_fit_pairs(ctx, L);   // until the boxes have shrunk
-    if (look) OBB_TRY(box_census(ctx, L));
+    if (look) OBB_TRY(box_census_alone(ctx, L));
     int64_t* h = host_stats(ctx);
     OBB_CK(ctx, cudaMemcpyAsync(h, L->d_stats, sizeof(int64_t) * kStCount, cudaMemcpyDeviceToHost, s));
     OBB_CK(ctx, cudaMemcpyAsync(h + kStCount, M->loop, sizeof(int64_t) * 4, cudaMemcpyDeviceToHost, s));

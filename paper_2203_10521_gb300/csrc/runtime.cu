@@ -90,7 +90,8 @@ obb_status cuda_fail(obb_ctx* ctx, cudaError_t e, const char* what)
 
 obb_status check_device_error(obb_ctx* ctx)
 {
-    OBB_CK(ctx, cudaMemcpyAsync(ctx->h_small, ctx->d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+    // the error word and the two words behind it (a layer's box census), for whoever wants them
+    OBB_CK(ctx, cudaMemcpyAsync(ctx->h_small, ctx->d_err, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     OBB_CK(ctx, cudaStreamSynchronize(ctx->stream));
     const int32_t w = ctx->h_small[0];
     if (w == 0) return OBB_OK;
@@ -218,14 +219,14 @@ obb_status obb_create(obb_ctx** out, int32_t device, void* stream)
     c->device = device;
     c->stream = static_cast<cudaStream_t>(stream);
     cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
-    if (cudaMalloc(&c->d_err, sizeof(int32_t)) != cudaSuccess ||
+    if (cudaMalloc(&c->d_err, 3 * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_ticket, sizeof(unsigned int)) != cudaSuccess ||
         cudaMalloc((void**)&c->d_prof, 8 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc((void**)&c->d_order_hist, kOrderBuckets * sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(c->d_order_hist, 0, kOrderBuckets * sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(c->d_prof, 0, 8 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMallocHost(&c->h_small, 64 * sizeof(int64_t)) != cudaSuccess ||
-        cudaMemset(c->d_err, 0, sizeof(int32_t)) != cudaSuccess ||
+        cudaMemset(c->d_err, 0, 3 * sizeof(int32_t)) != cudaSuccess ||
         cudaMemset(c->d_ticket, 0, sizeof(unsigned int)) != cudaSuccess) {
         obb_destroy(c);
         return OBB_ERR_CUDA;
